@@ -241,6 +241,16 @@ __device__ __forceinline__ void tmem_reg_fence(uint32_t* r) {
 
 // ------------------------------------------------------------------ misc ----
 
+// A value that is the same in all lanes of a converged warp, in a form the
+// compiler can see to be so.  A warp index or a size read from memory is
+// opaque to it: shuffles, votes and other warp-wide instructions under a
+// branch or loop on such a value are compiled for lanes that might have
+// diverged, at a hundred cycles and more each.
+template <class T>
+__device__ __forceinline__ T warp_uniform(T x) {
+  return __shfl_sync(0xffffffffu, x, 0);
+}
+
 // Checked build: is the element range [i, i + len) inside a buffer of n
 // elements?  If not, ROLEKV_STATUS_BOUNDS is OR-ed into *status (may be
 // null) and the caller skips the access.  The plain build compiles every

@@ -19,8 +19,6 @@
 
 namespace rolekv {
 
-size_t select_smem_bytes(int n_max);
-
 namespace {
 
 thread_local char g_err[512] = "no error";

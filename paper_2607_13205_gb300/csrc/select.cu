@@ -1,40 +1,50 @@
 // Role-conditional allocation and per-bucket top-k (Section 4.1, Algorithm 1):
 // pool the scores (optional), count the roles, split the budget ceil(B n)
 // across role buckets, and keep the top-q_r tokens of every bucket, ties to the
-// lower index.  One CTA per (layer, sequence, KV head) holds the unit's keys
-// in shared memory; everything after the fp32 -> ordered-key mapping is
-// integer, so the kept set is bit-exact for a given score row.
+// lower index.  A cluster of C CTAs per (layer, sequence, KV head), C = 1 to 8,
+// holds the unit's keys in shared memory, each CTA a contiguous slice;
+// everything after the fp32 -> ordered-key mapping is integer, so the kept set
+// is bit-exact for a given score row and does not depend on C.
 //
 // Slots.  Shared memory holds the unit in "slots": slot s is token s - off,
 // where off = (start address of the score row / 4) mod 4, so that every group
 // of four slots is one aligned 16-byte vector both in global and in shared
 // memory.  Slots outside [off, off + n) have role 0xFF and are never kept.
+// Rank k of the cluster owns groups [k gs, (k + 1) gs).
 //
 // The threshold of each bucket is found by a radix descent over the keys'
 // bits, most significant first:
 //   pass 1  load, pool, key; per role, a histogram of the key's bits
 //           30..31-NB (the top bit is shared by every key when all scores
-//           have one sign): exponent and leading mantissa bits.  The role
-//           counts are the histograms' sums.  Under GLOBAL there is one
-//           bucket, so one histogram of every eligible token.
-//   quotas  one warp, lane r for role r (water-filling, largest remainders).
-//   first digit from the pass-1 histograms, per bucket; while the keys at
-//           the threshold digits would overflow the list, a full pass over
-//           the slots per 8 more bits.
+//           have one sign): exponent and leading mantissa bits; role counts.
+//           Under GLOBAL there is one bucket, so one histogram of every
+//           eligible token.
+//   quotas  one warp, lane r for role r (water-filling, largest remainders),
+//           from the ranks' counts, in every rank alike.
+//   first digit from the ranks' pass-1 histograms, bucket b by rank b mod C;
+//           while the keys at the threshold digits would overflow the list, a
+//           full pass over the slots per 8 more bits.
 //   pass 2  every token is decided (kept / dropped) unless its key prefix is
 //           its bucket's threshold prefix; those "candidates" (a few
-//           percent) go to a list in shared memory.
-//   list    the remaining bits in 8-bit rounds over the list; ties at the
-//           threshold are ranked in index order; the kept ones join the bits.
-// A unit with a NaN, keys of both signs, or more candidates than the list
+//           percent) go to the rank's list in shared memory.
+//   list    the remaining bits in 8-bit rounds over the lists, every rank
+//           reading the ranks' digit counts; ties at the threshold are ranked
+//           in index order; the kept ones join the bits.
+// A unit with a NaN, keys of both signs, or more candidates than a list
 // holds 4 to 5 bits above the bottom takes the general path: four 8-bit
 // rounds over all slots.
-// Rows longer than kSmemMaxN tokens (streaming mode) do not keep their keys:
+// Kept positions are then written in ascending order from a scan of the bit
+// words, each rank at the offset of the ranks before it.
+//
+// Rows longer than kSmemMaxN tokens in batches of more units than clusters
+// can be resident (streaming mode, one CTA per unit) do not keep their keys:
 // every pass recomputes a group's pooled keys from the score row (read again
 // from L2), the first-digit histograms count in 32 bits and a candidate-list
 // entry carries its key beside (bucket << 24) | slot.
-// Kept positions are then written in ascending order from a block-wide scan
-// of the bit words.
+//
+// The ranks read each other's counts and histograms through distributed
+// shared memory, one cluster barrier per exchange; a digit round's counts
+// alternate between two buffers, so that a round needs one barrier.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -50,23 +60,30 @@ constexpr int kR = ROLEKV_MAX_ROLES;
 constexpr uint32_t kCodeKeep = 0x40;   // the token's bucket keeps everything
 constexpr uint32_t kCodeDrop = 0x80;   // no bucket keeps the token
 // codes 0 .. kR-1: the token's bucket keeps only keys above a threshold
+constexpr int kMaxRanks = 8;           // CTAs per unit (the portable cluster size)
+constexpr int kRankCost = 3000;        // most compares (sum of squared runs) taken by rank
 constexpr int kTieCap = 256;           // ranked ties held in shared memory
 
-// Longest row whose keys a CTA holds in shared memory; longer rows take the
-// streaming mode.
+// Longest row whose keys one CTA holds in shared memory.
 constexpr int kSmemMaxN = 40960;
 
-// Groups (of four slots) reserved per CTA: n_max tokens plus up to three
-// leading slots, rounded to a multiple of 32 groups so that the bit words
-// (one per 8 groups) end on a 16-byte boundary.
-__host__ __device__ inline int select_groups(int n_max) { return (((n_max + 3 + 3) / 4) + 31) & ~31; }
-// Width of the first digit: 2^NB bins per role.
-__host__ __device__ inline int first_digit_bits(int n_max) { return n_max > 16384 ? 11 : 10; }
-// Bytes of the region that holds the pass-1 histograms (8 roles x 2^NB bins
-// x 16-bit counts; 32-bit in streaming mode, where a bin can pass 65535),
-// reused for the candidate list (4-byte entries; 8-byte in streaming mode).
-__host__ __device__ inline size_t region_bytes(int n_max) {
-  return static_cast<size_t>(kR) * (size_t{1} << first_digit_bits(n_max)) * (n_max > kSmemMaxN ? 4 : 2);
+// How a unit's row is held.
+enum { kOne = 0, kCluster = 1, kStream = 2 };
+
+// Launch plan of one call: ranks and threads per unit, and the layout of a
+// rank's shared memory.
+struct SelectPlan {
+  int32_t ranks;       // CTAs per unit (the cluster size)
+  int32_t nb;          // first-digit bits
+  int32_t groups;      // groups (of four slots) a rank's memory holds
+  int32_t n_hist;      // buckets with a histogram
+  int32_t list_cap;    // candidate-list entries (8 bytes each in streaming mode, else 4)
+  int32_t hist_ints;   // the two digit-count buffers (and the first-digit sums)
+  int32_t region_words;   // pass-1 histograms, then the candidate list
+};
+
+__host__ __device__ inline int plan_groups(int groups, int ranks) {
+  return ((groups + ranks - 1) / ranks + 31) & ~31;
 }
 
 // Monotone map of a float to uint32 (larger float -> larger key); -0 is folded
@@ -83,11 +100,42 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
   return d;
 }
 
-// x << s, with every shift of 64 or more giving 0 (PTX clamps the amount).
-__device__ __forceinline__ uint64_t shl64(uint64_t x, uint32_t s) {
-  uint64_t r;
-  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(s));
+// Distributed shared memory: the address of a local shared object in rank
+// `rank` of the cluster, and accesses through such an address.
+__device__ __forceinline__ uint32_t map_rank(const void* p, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
   return r;
+}
+__device__ __forceinline__ int32_t ld_rank(uint32_t addr) {
+  int32_t v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ int4 ld_rank4(uint32_t addr) {
+  int4 v;
+  asm volatile("ld.shared::cluster.v4.s32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_rank(uint32_t addr, int32_t v) {
+  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void add_rank(uint32_t addr, int32_t v) {
+  asm volatile("red.relaxed.cluster.shared::cluster.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+// Barrier over the unit's CTAs (the whole cluster), or the CTA alone.
+template <bool CL>
+__device__ __forceinline__ void unit_sync() {
+  if constexpr (CL) {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+                     : "memory");
+  } else {
+    __syncthreads();
+  }
 }
 
 __device__ __forceinline__ int warp_sum(int v) {
@@ -97,6 +145,19 @@ __device__ __forceinline__ int warp_sum(int v) {
 }
 
 struct SelShared {
+  // this rank's share, read by the other ranks after a barrier
+  int32_t l_count[kR];     // tokens per role (GLOBAL: the eligible ones, in [0])
+  int32_t l_floor[kR];     // recency-floor tokens per role
+  int32_t l_nan;           // a sum of the slice's scores was NaN
+  uint32_t l_and, l_or;    // of the slice's keys
+  int32_t l_ties[kR];      // keys equal to a partial bucket's threshold
+  int32_t l_fill_ties;     // the same for the SLACK fill
+  int32_t l_total;         // kept slots
+  // first digits found by other ranks (written by them, taken over after a barrier)
+  uint32_t f_prefix[kR];
+  int32_t f_need[kR], f_cand[kR];
+  int32_t f_fail;
+  // the unit's state, the same in every rank
   int64_t keep_off;
   int32_t count[kR];       // tokens per role
   int32_t quota[kR];       // q_b per bucket
@@ -107,15 +168,9 @@ struct SelShared {
   int32_t cand[kR];        // candidates after the first digit
   int32_t code_of_role[256];
   int32_t first_of_role[256];  // pass 2: keep iff first digit > it, candidate iff ==
-  int32_t hist[kR][256];
-  int32_t warp_tot[32];
-  int32_t kept_role[kR];
   int32_t floor_role[kR];  // recency-floor tokens per role
-  uint32_t ties[kTieCap];  // (bucket << 16) | slot of keys equal to a threshold
   uint32_t top_and, top_or;
-  int32_t list_n, tie_n;
   int32_t nan_hint;        // a sum of the unit's scores was NaN
-  int32_t nan_seen;        // a pooled window held a NaN
   int32_t any_threshold;
   int32_t general;         // take the full-pass descent
   uint32_t partial_ties;   // buckets with more threshold ties than slots left
@@ -124,6 +179,13 @@ struct SelShared {
   int32_t sfast;           // SLACK: the fill's first digit is known (below)
   uint32_t sprefix;        // SLACK: shared top bit and first digit of the fill threshold
   int32_t sneed;           // SLACK: tokens at that digit still to fill
+  // this rank's own
+  int32_t warp_tot[32];
+  int32_t kept_role[kR];   // (rank 0: the ranks add to it)
+  uint32_t ties[kTieCap];  // (bucket << 16) | slot of keys equal to a threshold
+  int32_t list_n, tie_n;
+  int32_t run0[kR], run_n[kR];   // candidate runs of the buckets
+  int32_t nan_seen;        // a pooled window held a NaN
 };
 
 // Slots 4g .. 4g+3 of a score row; slots outside [off, off + n) read -inf.
@@ -156,7 +218,8 @@ __device__ __forceinline__ uint32_t load_roles(const uint8_t* rp, int off, int n
 struct UnitView {
   const float* sp;
   const uint8_t* rp;
-  int off, n, ngroups;
+  int off, n;
+  int g0, ng;      // this rank's groups: g0 .. g0 + ng - 1
   int nf;          // tokens before the recency floor (the floor is [nf, n))
   bool rvec;
 };
@@ -172,7 +235,8 @@ __device__ __forceinline__ uint32_t floor_bits(int s0, int nf, int n) {
   return m;
 }
 
-// Pass 1 for a pool half-width HW known at compile time.
+// Pass 1 over the rank's groups for a pool half-width HW known at compile
+// time; floor tokens are counted apart.
 template <int HW, int NT, bool GL, bool STREAM>
 __device__ __forceinline__ void pass1(const UnitView& v, int n_roles, uint32_t ban, int nb,
                                       uint4* keys4, uint32_t* hist16, int32_t* floor_role,
@@ -181,7 +245,8 @@ __device__ __forceinline__ void pass1(const UnitView& v, int n_roles, uint32_t b
   const int sh0 = 31 - nb;
   const uint32_t bmask = (1u << nb) - 1u;
   const int words_per_role = 1 << (nb - 1);
-  for (int g = threadIdx.x; g < v.ngroups; g += NT) {
+  for (int lg = threadIdx.x; lg < v.ng; lg += NT) {
+    const int g = v.g0 + lg;
     // the role bytes are loaded with the scores, not after the pooling
     const uint32_t rw = load_roles(v.rp, v.off, v.n, g, v.rvec);
     float x[4 * (2 * NB + 1)];
@@ -209,7 +274,7 @@ __device__ __forceinline__ void pass1(const UnitView& v, int n_roles, uint32_t b
       }
       k[j] = ordered_key(m);
     }
-    if (!STREAM) keys4[g] = make_uint4(k[0], k[1], k[2], k[3]);
+    if (!STREAM) keys4[lg] = make_uint4(k[0], k[1], k[2], k[3]);
     const uint32_t fb = floor_bits(4 * g - v.off, v.nf, v.n);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -229,6 +294,17 @@ __device__ __forceinline__ void pass1(const UnitView& v, int n_roles, uint32_t b
       }
     }
   }
+}
+
+// Quotas of one sequence by warp 0, lane r for role r: water-filling of the
+// weights over the role counts, then the integer remainders to the largest
+// fractional parts (ties to the lower role), or under CEIL the ceiling of each
+// share; the arithmetic stated in rolekv.h.
+__device__ __forceinline__ int64_t sum8(int64_t v) {
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 4);
+  return v;
 }
 
 // Streaming mode: the four keys of group g recomputed from the score row, the
@@ -260,17 +336,6 @@ __device__ __forceinline__ uint4 stream_group_keys(const UnitView& v, int g, int
     k[j] = (nan_aware && nanw) ? 0u : ordered_key(m);
   }
   return make_uint4(k[0], k[1], k[2], k[3]);
-}
-
-// Quotas of one sequence by warp 0, lane r for role r: water-filling of the
-// weights over the role counts, then the integer remainders to the largest
-// fractional parts (ties to the lower role), or under CEIL the ceiling of each
-// share; the arithmetic stated in rolekv.h.
-__device__ __forceinline__ int64_t sum8(int64_t v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
-  return v;
 }
 
 __device__ void quotas_warp(const SelectArgs& a, int lane, int64_t K_full, SelShared& S) {
@@ -360,19 +425,44 @@ __device__ void quotas_warp(const SelectArgs& a, int lane, int64_t K_full, SelSh
 }
 
 // The bucket's key among its remaining candidates with need[b] keys at or
-// above it: warp b reads the histogram of the digit at `shift` (clearing it),
+// above it: one warp sums the ranks' counts of the digit at `shift` (hist),
 // finds the digit where the count from the top reaches need[b], appends it to
 // prefix[b] and subtracts the keys above.  At shift 0 the prefix is the
-// q_b-th largest key; thr[b] and the partial-tie flag are then set.
-__device__ void descend(SelShared& S, int b, int lane, int shift) {
+// q_b-th largest key; thr[b] and the partial-tie flag are then set.  Every
+// rank does it alike.
+template <bool CL>
+__device__ void descend(SelShared& S, const int32_t* hist, int ranks, int b, int lane, int shift) {
   int c[8];
+  const int32_t* hb = hist + b * 256 + lane * 8;
+  if constexpr (CL) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) c[i] = 0;
+    // (four ranks' loads in flight)
+    for (int k0 = 0; k0 < ranks; k0 += 4) {
+      int4 x[4], y[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (k0 + k < ranks) {
+          const uint32_t addr = map_rank(hb, k0 + k);
+          x[k] = ld_rank4(addr);
+          y[k] = ld_rank4(addr + 16);
+        } else {
+          x[k] = y[k] = make_int4(0, 0, 0, 0);
+        }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        c[0] += x[k].x; c[1] += x[k].y; c[2] += x[k].z; c[3] += x[k].w;
+        c[4] += y[k].x; c[5] += y[k].y; c[6] += y[k].z; c[7] += y[k].w;
+      }
+    }
+  } else {
+    const int4 x = *reinterpret_cast<const int4*>(hb), y = *reinterpret_cast<const int4*>(hb + 4);
+    c[0] = x.x; c[1] = x.y; c[2] = x.z; c[3] = x.w;
+    c[4] = y.x; c[5] = y.y; c[6] = y.z; c[7] = y.w;
+  }
   int mine = 0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    c[i] = S.hist[b][lane * 8 + i];
-    S.hist[b][lane * 8 + i] = 0;
-    mine += c[i];
-  }
+  for (int i = 0; i < 8; ++i) mine += c[i];
   int incl = mine;   // tokens whose digit is in this lane's range or above
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -489,14 +579,15 @@ __device__ void descend_first(const SelectArgs& a, SelShared& S, const uint32_t*
 // a role's whole bin (its bucket keeps nothing, or the bin lies below the
 // bucket's digit), none (the bucket keeps the bin), or the bin less the
 // need[b] tokens the bucket keeps at its own digit.  Every thread counts a
-// few bins into `cnt` (shared memory, 2^NB ints); then warp 0 locates the
-// bin holding the slack-th token from the top: each lane sums a contiguous
-// range, the lanes' totals from the top locate the range, and the warp
-// splits that range.  On success sprefix / sneed are set and sfast = 1;
-// otherwise the fill takes its full-pass rounds.  Every thread calls it.
-template <int NB, int NT>
+// few bins of its rank into `cnt` (shared memory, 2^NB ints); rank 0 adds the
+// ranks' counts, and its warp 0 locates the bin holding the slack-th token
+// from the top: each lane sums a contiguous range, the lanes' totals from the
+// top locate the range, and the warp splits that range.  On success sprefix /
+// sneed are set and sfast = 1 in every rank; otherwise the fill takes its
+// full-pass rounds.  cnt is left with counts in it.
+template <int NB, int NT, bool CL>
 __device__ void slack_first(const SelectArgs& a, SelShared& S, const uint32_t* hist16, int* cnt,
-                            int list_cap) {
+                            int list_cap, int slice_slots, int rank, int ranks) {
   constexpr int nbins = 1 << NB;
   constexpr int bpl = nbins / 32;        // bins per lane
   constexpr int wpr = 1 << (NB - 1);     // histogram words (two bins each) per role
@@ -514,81 +605,101 @@ __device__ void slack_first(const SelectArgs& a, SelShared& S, const uint32_t* h
         c += h;                                  // its bucket keeps nothing
       } else {
         const int D = static_cast<int>((S.prefix[code] >> sh0) & (nbins - 1));
-        c += x < D ? h : (x == D ? h - S.need[code] : 0);
+        // (the need[b] tokens are the unit's: taken off once, in rank 0)
+        c += x < D ? h : (x == D ? h - (rank == 0 ? S.need[code] : 0) : 0);
       }
     }
     cnt[x] = c;
   }
-  __syncthreads();
-  if (tid < 32) {
-    const int need = S.slack;
-    int mine = 0;
-#pragma unroll 8
-    for (int i = 0; i < bpl; ++i) mine += cnt[lane * bpl + ((i + lane) & (bpl - 1))];
-    int incl = mine;                             // tokens in this lane's bins or above
+  unit_sync<CL>();
+  if (rank == 0) {
+    if constexpr (CL) {
+      for (int x = tid; x < nbins; x += NT) {
+        int c[kMaxRanks];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_down_sync(0xffffffffu, incl, o);
-      if (lane + o < 32) incl += v;
-    }
-    const int above = incl - mine;
-    const unsigned who = __ballot_sync(0xffffffffu, above < need && above + mine >= need);
-    if (who != 0) {
-      const int F = __ffs(who) - 1;
-      const int aboveF = __shfl_sync(0xffffffffu, above, F);
-      const int needF = need - aboveF;
-      // the winning range split over the warp: bpl / 32 bins a lane
-      constexpr int per = bpl / 32 > 0 ? bpl / 32 : 1;
-      int c2[per];
-      int part = 0;
+        for (int k = 0; k < kMaxRanks; ++k) c[k] = k < ranks ? ld_rank(map_rank(cnt + x, k)) : 0;
 #pragma unroll
-      for (int i = 0; i < per; ++i) {
-        c2[i] = (lane * per + i < bpl) ? cnt[F * bpl + lane * per + i] : 0;
-        part += c2[i];
+        for (int k = 1; k < kMaxRanks; ++k) c[0] += c[k];
+        cnt[x] = c[0];
       }
-      int incl2 = part;
+      __syncthreads();
+    }
+    if (warp_uniform(tid >> 5) == 0) {
+      const int need = S.slack;
+      int mine = 0;
+#pragma unroll 8
+      for (int i = 0; i < bpl; ++i) mine += cnt[lane * bpl + ((i + lane) & (bpl - 1))];
+      int incl = mine;                             // tokens in this lane's bins or above
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_down_sync(0xffffffffu, incl2, o);
-        if (lane + o < 32) incl2 += v;
+        const int v = __shfl_down_sync(0xffffffffu, incl, o);
+        if (lane + o < 32) incl += v;
       }
-      const int above2 = incl2 - part;
-      const unsigned who2 = __ballot_sync(0xffffffffu, above2 < needF && above2 + part >= needF);
-      if (who2 != 0 && lane == __ffs(who2) - 1) {
-        int acc = above2, fd = -1, nd = 0, at = 0;
+      const int above = incl - mine;
+      const unsigned who = __ballot_sync(0xffffffffu, above < need && above + mine >= need);
+      if (who != 0) {
+        const int F = __ffs(who) - 1;
+        const int aboveF = __shfl_sync(0xffffffffu, above, F);
+        const int needF = need - aboveF;
+        // the winning range split over the warp: bpl / 32 bins a lane
+        constexpr int per = bpl / 32 > 0 ? bpl / 32 : 1;
+        int c2[per];
+        int part = 0;
 #pragma unroll
-        for (int i = per - 1; i >= 0; --i) {
-          if (fd < 0 && acc + c2[i] >= needF) {
-            fd = F * bpl + lane * per + i;
-            nd = needF - acc;
-            at = c2[i];
-          }
-          acc += c2[i];
+        for (int i = 0; i < per; ++i) {
+          c2[i] = (lane * per + i < bpl) ? cnt[F * bpl + lane * per + i] : 0;
+          part += c2[i];
         }
-        if (fd >= 0 && at <= list_cap) {
-          S.sprefix = (S.top_and & 0x80000000u) | (static_cast<uint32_t>(fd) << sh0);
-          S.sneed = nd;
-          S.sfast = 1;
+        int incl2 = part;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_down_sync(0xffffffffu, incl2, o);
+          if (lane + o < 32) incl2 += v;
+        }
+        const int above2 = incl2 - part;
+        const unsigned who2 = __ballot_sync(0xffffffffu, above2 < needF && above2 + part >= needF);
+        if (who2 != 0 && lane == __ffs(who2) - 1) {
+          int acc = above2, fd = -1, nd = 0, at = 0;
+#pragma unroll
+          for (int i = per - 1; i >= 0; --i) {
+            if (fd < 0 && acc + c2[i] >= needF) {
+              fd = F * bpl + lane * per + i;
+              nd = needF - acc;
+              at = c2[i];
+            }
+            acc += c2[i];
+          }
+          if (fd >= 0 && (at <= list_cap || slice_slots <= list_cap)) {
+            const uint32_t prefix = (S.top_and & 0x80000000u) | (static_cast<uint32_t>(fd) << sh0);
+            if constexpr (CL) {
+              for (int k = 0; k < ranks; ++k) {
+                st_rank(map_rank(&S.sprefix, k), static_cast<int32_t>(prefix));
+                st_rank(map_rank(&S.sneed, k), nd);
+                st_rank(map_rank(&S.sfast, k), 1);
+              }
+            } else {
+              S.sprefix = prefix;
+              S.sneed = nd;
+              S.sfast = 1;
+            }
+          }
         }
       }
     }
   }
-  __syncthreads();
-  for (int x = tid; x < nbins; x += NT) cnt[x] = 0;
-  __syncthreads();
+  unit_sync<CL>();
 }
 
-// descend_first for the streaming mode's 32-bit bins: lane L owns bins
-// L * 2^NB / 32 ..; the lanes' totals locate the lane holding the threshold,
-// then the warp splits that lane's bins (at most 64, two per lane).
+// descend_first over the ranks' summed counts (32-bit bins, `sums`), by one
+// warp; the result goes to every rank.  Lane L owns bins L * 2^NB / 32 ..; the
+// lanes' totals locate the lane holding the threshold, then the warp splits
+// that lane's bins (at most 64, two per lane).
 template <int NB>
-__device__ void descend_first32(const SelectArgs& a, SelShared& S, const uint32_t* hist32, int b,
-                                int lane) {
+__device__ void descend_first_sums(SelShared& S, const int32_t* sums, int b, int lane, int ranks) {
   constexpr int bpl = 1 << (NB - 5);   // bins per lane
-  const uint32_t* h0 = hist32 + (b << NB);
   int mine = 0;
 #pragma unroll 8
-  for (int i = 0; i < bpl; ++i) mine += static_cast<int>(h0[lane * bpl + ((i + lane) & (bpl - 1))]);
+  for (int i = 0; i < bpl; ++i) mine += sums[lane * bpl + ((i + lane) & (bpl - 1))];
   int incl = mine;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -598,17 +709,13 @@ __device__ void descend_first32(const SelectArgs& a, SelShared& S, const uint32_
   const int above = incl - mine;
   const int need = S.need[b];
   const unsigned who = __ballot_sync(0xffffffffu, above < need && above + mine >= need);
-  if (who == 0) {
-    if (lane == 0) S.general = 1;
-    return;
-  }
-  const int F = __ffs(who) - 1;
+  const int F = who ? __ffs(who) - 1 : 0;
   const int aboveF = __shfl_sync(0xffffffffu, above, F);
   const int needF = need - aboveF;
   // lane L takes bins F * bpl + 2L, 2L + 1 (descending order: the higher bin first)
   const int i0 = 2 * lane;
-  const int lo = i0 < bpl ? static_cast<int>(h0[F * bpl + i0]) : 0;
-  const int hi = i0 + 1 < bpl ? static_cast<int>(h0[F * bpl + i0 + 1]) : 0;
+  const int lo = i0 < bpl ? sums[F * bpl + i0] : 0;
+  const int hi = i0 + 1 < bpl ? sums[F * bpl + i0 + 1] : 0;
   const int pair = lo + hi;
   int incl2 = pair;
 #pragma unroll
@@ -618,39 +725,31 @@ __device__ void descend_first32(const SelectArgs& a, SelShared& S, const uint32_
   }
   const int above2 = incl2 - pair;
   const unsigned who2 = __ballot_sync(0xffffffffu, above2 < needF && above2 + pair >= needF);
-  if (who2 == 0) {
-    if (lane == 0) S.general = 1;
-    return;
-  }
-  if (lane == __ffs(who2) - 1) {
-    const int bin0 = F * bpl + i0;
-    int fd, gb, ad;
-    if (above2 + hi >= needF) {
-      fd = bin0 + 1;
-      gb = aboveF + above2;
-      ad = hi;
+  const int src = who2 ? __ffs(who2) - 1 : 0;
+  const bool upper = above2 + hi >= needF;
+  const int fd = __shfl_sync(0xffffffffu, F * bpl + i0 + (upper ? 1 : 0), src);
+  const int gb = __shfl_sync(0xffffffffu, aboveF + above2 + (upper ? 0 : hi), src);
+  const int ad = __shfl_sync(0xffffffffu, upper ? hi : lo, src);
+  if (lane < ranks) {
+    if (who == 0 || who2 == 0) {
+      st_rank(map_rank(&S.f_fail, lane), 1);   // counts disagree with the quota: the full path decides
     } else {
-      fd = bin0;
-      gb = aboveF + above2 + hi;
-      ad = lo;
+      const uint32_t prefix = (S.top_and & 0x80000000u) | (static_cast<uint32_t>(fd) << (31 - NB));
+      st_rank(map_rank(&S.f_prefix[b], lane), static_cast<int32_t>(prefix));
+      st_rank(map_rank(&S.f_need[b], lane), need - gb);
+      st_rank(map_rank(&S.f_cand[b], lane), ad);
     }
-    const int sh0 = 31 - NB;
-    S.prefix[b] = (S.top_and & 0x80000000u) | (static_cast<uint32_t>(fd) << sh0);
-    S.need[b] = need - gb;
-    S.cand[b] = ad;
   }
 }
 
-// Exclusive prefix, in slot order, of popc(mask_of(q)) over the bit words
-// q < nwords: warp w walks a contiguous range of words (a multiple of 32), the
-// warps' totals are combined through shared memory, and body(q, mask, rank of
-// the word's first set bit) runs once per word.  Returns the total.  Every
-// thread of the CTA must call it.
-template <int NT, class MaskF, class BodyF>
-__device__ int scan_words(int nwords, MaskF mask_of, BodyF body, int32_t* warp_tot) {
+// popc(mask_of(q)) summed over the bit words q < nwords: warp w walks a
+// contiguous range of words; the warps' totals are left in warp_tot for
+// scan_words.  Returns the total.  Every thread of the CTA calls it.
+template <int NT, class MaskF>
+__device__ int count_words(int nwords, MaskF mask_of, int32_t* warp_tot) {
   constexpr int NW = NT / 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int wseg = ((nwords + NW - 1) / NW + 31) & ~31;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int wseg = (nwords + NW - 1) / NW;
   const int q_begin = warp * wseg;
   const int q_end = min(nwords, q_begin + wseg);
   int tot = 0;
@@ -661,8 +760,19 @@ __device__ int scan_words(int nwords, MaskF mask_of, BodyF body, int32_t* warp_t
   tot = warp_sum(tot);
   if (lane == 0) warp_tot[warp] = tot;
   __syncthreads();
-  int base = warp_sum(lane < warp ? warp_tot[lane] : 0);
-  const int total = warp_sum(lane < NW ? warp_tot[lane] : 0);
+  return warp_sum(lane < NW ? warp_tot[lane] : 0);
+}
+
+// After count_words: body(q, mask, rank of the word's first set bit) once per
+// word, the ranks in slot order from `base0`.
+template <int NT, class MaskF, class BodyF>
+__device__ void scan_words(int nwords, int base0, MaskF mask_of, BodyF body, const int32_t* warp_tot) {
+  constexpr int NW = NT / 32;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int wseg = (nwords + NW - 1) / NW;
+  const int q_begin = warp * wseg;
+  const int q_end = min(nwords, q_begin + wseg);
+  int base = base0 + warp_sum(lane < warp ? warp_tot[lane] : 0);
   for (int q0 = q_begin; q0 < q_end; q0 += 32) {
     const int q = q0 + lane;
     const uint32_t m = q < q_end ? mask_of(q) : 0u;
@@ -677,7 +787,6 @@ __device__ int scan_words(int nwords, MaskF mask_of, BodyF body, int32_t* warp_t
     base += __shfl_sync(0xffffffffu, incl, 31);
   }
   __syncthreads();
-  return total;
 }
 
 // Keep bits of slots 4g .. 4g+3 (bit j = slot 4g+j) packed into one 32-bit
@@ -690,22 +799,26 @@ __device__ __forceinline__ void store_bits(uint32_t* bits, int g, int nwords, in
   if ((lane & 7) == 0 && g < 8 * nwords) bits[g >> 3] = x;
 }
 
-template <int NT, bool STREAM>
-__global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs a) {
+template <int NT, int MODE>
+__global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs a, const SelectPlan p) {
+  constexpr bool CL = MODE == kCluster, STREAM = MODE == kStream;
   constexpr int NW = NT / 32;
   extern __shared__ __align__(16) uint8_t dyn[];
   __shared__ SelShared S;
   const int tid = threadIdx.x;
-  const int warp = tid >> 5, lane = tid & 31;
-  const int u = blockIdx.x;
+  const int warp = warp_uniform(tid >> 5), lane = tid & 31;
+  const int ranks = CL ? p.ranks : 1;
+  const int u = CL ? blockIdx.x / ranks : blockIdx.x;
+  const int rank = CL ? blockIdx.x % ranks : 0;   // (clusters are consecutive blocks)
   const int h = u % a.Hkv;
   const int s = (u / a.Hkv) % a.b;
   const int l = u / (a.Hkv * a.b);
   int n;
   int64_t tok0;
   if (a.varlen) {
-    tok0 = a.cu_seqlens[s];
-    n = a.cu_seqlens[s + 1] - a.cu_seqlens[s];
+    const int t0 = warp_uniform(a.cu_seqlens[s]);
+    tok0 = t0;
+    n = warp_uniform(a.cu_seqlens[s + 1]) - t0;
   } else {
     tok0 = 0;
     n = a.n_max;
@@ -721,81 +834,87 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
   v.rp = a.roles + rbase;
   v.off = static_cast<int>((reinterpret_cast<uintptr_t>(v.sp) >> 2) & 3);
   v.n = n;
-  const int nslots = v.off + n;
-  v.ngroups = (nslots + 3) >> 2;
+  const int ngroups = (v.off + n + 3) >> 2;
+  const int gs = plan_groups(ngroups, ranks);       // groups a rank owns
+  v.g0 = rank * gs;
+  v.ng = max(0, min(ngroups - v.g0, gs));
   v.rvec = ((reinterpret_cast<uintptr_t>(v.rp) - static_cast<uintptr_t>(v.off)) & 3u) == 0;
   const int64_t n_floor = a.keep_last < n ? (a.keep_last < K_s ? a.keep_last : K_s)
                                           : (n < K_s ? n : K_s);
   v.nf = n - static_cast<int>(n_floor);
-  const int off = v.off, ngroups = v.ngroups;
-  const int nwords = (nslots + 31) >> 5;
-  const int iters = (ngroups + NT - 1) / NT;
-  const int nb = first_digit_bits(a.n_max);
-  const int groups_alloc = select_groups(a.n_max);
-  // keys (in-memory mode only), keep bits, then the histogram / list region
+  const int off = v.off, ng = v.ng, g0 = v.g0;
+  const int slot0 = 4 * g0;                         // first slot of the rank
+  const int nwords = (ng + 7) >> 3;
+  const int iters = (ng + NT - 1) / NT;
+  const int nb = p.nb;
+  // keys, keep bits, the digit counts, then the histogram / list region
   uint4* keys4 = reinterpret_cast<uint4*>(dyn);
   const uint32_t* keys = reinterpret_cast<const uint32_t*>(keys4);
-  uint32_t* bits = reinterpret_cast<uint32_t*>(dyn + (STREAM ? 0 : static_cast<size_t>(groups_alloc) * 16));
-  uint32_t* region = bits + groups_alloc / 8;   // 16-byte aligned (groups_alloc % 32 == 0)
+  uint32_t* bits = reinterpret_cast<uint32_t*>(dyn + (STREAM ? 0 : static_cast<size_t>(p.groups) * 16));
+  int32_t* hist = reinterpret_cast<int32_t*>(bits + p.groups / 8);   // 16-byte aligned (groups % 32 == 0)
+  uint32_t* region = reinterpret_cast<uint32_t*>(hist + p.hist_ints);
   uint32_t* hist16 = region;                    // pass 1 histograms
   uint32_t* list = region;                      // then the candidate list
-  const int list_cap = static_cast<int>(region_bytes(a.n_max) / (STREAM ? 8 : 4));
+  const int list_cap = p.list_cap;
+  const int hsz = p.n_hist * 256;               // one digit-count buffer
   const bool global = a.policy == ROLEKV_POLICY_GLOBAL;
   const int hw = a.pool_k / 2;
-  // a group's four keys: held (in-memory mode) or recomputed from the scores
+  // a group's four keys: held, or recomputed from the scores
   bool nan_keys = false;                        // streaming mode: NaN windows give key 0
-  auto kv_of = [&](int g) -> uint4 {
-    if constexpr (STREAM) return stream_group_keys(v, g, hw, nan_keys);
-    else return keys4[g];
+  auto kv_of = [&](int lg) -> uint4 {
+    if constexpr (STREAM) return stream_group_keys(v, lg, hw, nan_keys);
+    else return keys4[lg];
   };
+  // a list entry: (bucket, slot), in streaming mode with its key before it
+  constexpr int kCodeShift = STREAM ? 24 : 16;
+  constexpr uint32_t kSlotMask = (1u << kCodeShift) - 1u;
+  auto entry = [&](int e) { return STREAM ? list[2 * e + 1] : list[e]; };
+  auto entry_key = [&](int e) { return STREAM ? list[2 * e] : keys[list[e] & kSlotMask]; };
 
   if (tid < kR) {
-    S.count[tid] = 0;
+    S.l_count[tid] = 0;
+    S.l_floor[tid] = 0;
+    S.l_ties[tid] = 0;
     S.kept_role[tid] = 0;
-    S.floor_role[tid] = 0;
   }
   if (tid == 0) {
-    S.nan_hint = 0;
+    S.l_nan = 0;
+    S.l_and = 0xFFFFFFFFu;
+    S.l_or = 0u;
+    S.l_fill_ties = 0;
+    S.f_fail = 0;
     S.nan_seen = 0;
     S.general = 0;
-    S.top_and = 0xFFFFFFFFu;
-    S.top_or = 0u;
     S.slack = 0;
     S.elig_mask = 0u;
     S.sfast = 0;
   }
-  for (int x = tid; x < kR * 256; x += NT) (&S.hist[0][0])[x] = 0;
+  for (int x = tid; x < p.hist_ints; x += NT) hist[x] = 0;
   {
     uint4* r4 = reinterpret_cast<uint4*>(region);
-    const int n4 = static_cast<int>(region_bytes(a.n_max) / 16);
+    const int n4 = (p.n_hist << (STREAM ? nb : nb - 1)) / 4;
     for (int x = tid; x < n4; x += NT) r4[x] = make_uint4(0u, 0u, 0u, 0u);
   }
 
-  // ---- offset of this unit's kept row
-  {
-    int64_t part = 0;
+  // ---- offset of this unit's kept row (warp 0)
+  if (warp == 0) {
+    int64_t off_kept = static_cast<int64_t>(u) * a.K_dense;
     if (a.varlen) {
-      for (int x = tid; x < s; x += NT)
+      int64_t part = 0;
+      for (int x = lane; x < s; x += 32)
         part += kept_rows(a.cu_seqlens[x + 1] - a.cu_seqlens[x], a.budget_fx, a.kept_extra);
-    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    __shared__ int64_t red64[NW];
-    if (lane == 0) red64[warp] = part;
-    __syncthreads();
-    if (tid == 0) {
-      int64_t cu = 0;
-      for (int w = 0; w < NW; ++w) cu += red64[w];
-      S.keep_off = a.varlen ? (static_cast<int64_t>(l) * a.Hkv + h) * a.Ktot + cu
-                            : static_cast<int64_t>(u) * a.K_dense;
+      for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+      off_kept = (static_cast<int64_t>(l) * a.Hkv + h) * a.Ktot + part;
     }
+    if (lane == 0) S.keep_off = off_kept;
   }
+  __syncthreads();
 
   // Checked build: the unit's score row (and mask row), role row, kept row
   // and per-role counts lie inside the extents the call's shapes give, or the
-  // whole unit is skipped.
+  // whole unit is skipped (by all its ranks alike, before the first exchange).
 #ifdef ROLEKV_CHECKED
-  __syncthreads();
   if (!(in_bounds(sbase, n, a.ext_scores, nullptr) && in_bounds(rbase, n, a.ext_roles, nullptr) &&
         in_bounds(S.keep_off, width, a.ext_keep, nullptr) &&
         (a.kept_per_role == nullptr ||
@@ -806,17 +925,17 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
   }
 #endif
 
-  // ---- pass 1: load, pool, key, first-digit histograms
+  // ---- pass 1: load, pool, key, first-digit histograms, role counts
   {
     bool nan_hint = false;
     uint32_t tand = 0xFFFFFFFFu, tor = 0u;
     // GLOBAL: one histogram (row 0) of every eligible token; otherwise one
     // row per role
 #define ROLEKV_PASS1(HWV)                                                                           \
-  (global ? pass1<HWV, NT, true, STREAM>(v, a.n_roles, a.ban_mask, nb, keys4, hist16, S.floor_role, \
-                                         nan_hint, tand, tor)                                       \
-          : pass1<HWV, NT, false, STREAM>(v, a.n_roles, a.ban_mask, nb, keys4, hist16, S.floor_role, \
-                                          nan_hint, tand, tor))
+  (global ? pass1<HWV, NT, true, STREAM>(v, a.n_roles, a.ban_mask, nb, keys4, hist16, S.l_floor, nan_hint,  \
+                                 tand, tor)                                                         \
+          : pass1<HWV, NT, false, STREAM>(v, a.n_roles, a.ban_mask, nb, keys4, hist16, S.l_floor, nan_hint, \
+                                  tand, tor))
     switch (a.pool_k >> 1) {
       case 0: ROLEKV_PASS1(0); break;
       case 1: ROLEKV_PASS1(1); break;
@@ -832,40 +951,97 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
     tor = __reduce_or_sync(0xffffffffu, tor);
     const bool nh = __any_sync(0xffffffffu, nan_hint);
     if (lane == 0) {
-      atomicAnd(&S.top_and, tand);
-      atomicOr(&S.top_or, tor);
-      if (nh) S.nan_hint = 1;
+      atomicAnd(&S.l_and, tand);
+      atomicOr(&S.l_or, tor);
+      if (nh) S.l_nan = 1;
     }
   }
   __syncthreads();
-
-  // Role counts: the sums of the roles' histograms (a warp's 32 words belong
-  // to one role); GLOBAL: the eligible total, in count[0].
-  {
-    const int wpr = STREAM ? (1 << nb) : (1 << (nb - 1));   // words per role
-    const int lwpr = STREAM ? nb : nb - 1;
-    for (int x0 = warp * 32; x0 < (global ? 1 : a.n_roles) * wpr; x0 += NT) {
-      const uint32_t w = hist16[x0 + lane];
-      const int c = warp_sum(STREAM ? static_cast<int>(w) : static_cast<int>((w & 0xFFFFu) + (w >> 16)));
-      if (lane == 0 && c) atomicAdd(&S.count[x0 >> lwpr], c);
+  // Role counts: the sums of the roles' histograms, a warp per role; GLOBAL:
+  // the eligible total, in count[0].
+  for (int r = warp; r < p.n_hist; r += NW) {
+    const int w4 = STREAM ? 1 << (nb - 2) : 1 << (nb - 3);   // 16-byte words per role
+    const uint4* h4 = reinterpret_cast<const uint4*>(hist16) + r * w4;
+    uint32_t c = 0;
+#pragma unroll 4
+    for (int x = lane; x < w4; x += 32) {
+      const uint4 w = h4[x];
+      if (STREAM) {
+        c += (w.x + w.y) + (w.z + w.w);
+      } else {
+        c += (w.x & 0xFFFFu) + (w.x >> 16) + (w.y & 0xFFFFu) + (w.y >> 16);
+        c += (w.z & 0xFFFFu) + (w.z >> 16) + (w.w & 0xFFFFu) + (w.w >> 16);
+      }
     }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0) S.l_count[r] = static_cast<int32_t>(c);
   }
+  unit_sync<CL>();
+
+  // ---- the unit's counts, quotas (in every rank alike)
+  if (warp == 0) {
+    int c = 0, f = 0, nan = 0;
+    uint32_t vand = 0xFFFFFFFFu, vor = 0u;
+    const int r = lane & (kR - 1);
+    if constexpr (CL) {
+      // lanes 8 j .. 8 j + 7 read ranks j and j + 4
+      int cc[2], ff[2], na[2];
+      uint32_t va[2], vo[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int k = (lane >> 3) + 4 * i;
+        const bool in = k < ranks;
+        const int kk = in ? k : rank;
+        cc[i] = ld_rank(map_rank(&S.l_count[r], kk));
+        ff[i] = ld_rank(map_rank(&S.l_floor[r], kk));
+        na[i] = ld_rank(map_rank(&S.l_nan, kk));
+        va[i] = static_cast<uint32_t>(ld_rank(map_rank(&S.l_and, kk)));
+        vo[i] = static_cast<uint32_t>(ld_rank(map_rank(&S.l_or, kk)));
+        if (!in) {
+          cc[i] = 0;
+          ff[i] = 0;
+        }
+      }
+      c = cc[0] + cc[1];
+      f = ff[0] + ff[1];
+      c += __shfl_xor_sync(0xffffffffu, c, 8);
+      c += __shfl_xor_sync(0xffffffffu, c, 16);
+      f += __shfl_xor_sync(0xffffffffu, f, 8);
+      f += __shfl_xor_sync(0xffffffffu, f, 16);
+      nan = __any_sync(0xffffffffu, na[0] | na[1]);
+      vand = __reduce_and_sync(0xffffffffu, va[0] & va[1]);
+      vor = __reduce_or_sync(0xffffffffu, vo[0] | vo[1]);
+    } else {
+      c = S.l_count[r];
+      f = S.l_floor[r];
+      nan = S.l_nan;
+      vand = S.l_and;
+      vor = S.l_or;
+    }
+    if (lane < kR) {
+      S.count[lane] = c;
+      S.floor_role[lane] = f;
+    }
+    if (lane == 0) {
+      S.nan_hint = nan;
+      S.top_and = vand;
+      S.top_or = vor;
+      if (nan || ((vand ^ vor) & 0x80000000u)) S.general = 1;
+    }
+    __syncwarp();
+    quotas_warp(a, lane, K_s - n_floor, S);
+  }
+  __syncthreads();
 
   // A NaN score (or +inf and -inf in one group): redo the keys one token at a
   // time, a window holding a NaN giving the lowest key (streaming mode: every
   // later recomputation of the keys does so).
-  if (STREAM) nan_keys = S.nan_hint != 0;
-  if (STREAM && S.nan_hint) {
-    bool seen = false;
-    for (int t = tid; t < n; t += NT) seen |= isnan(__ldg(v.sp + t));
-    if (__any_sync(0xffffffffu, seen) && lane == 0) S.nan_seen = 1;
-  }
-  if (!STREAM && S.nan_hint) {
-    const int hw = a.pool_k / 2;
+  nan_keys = S.nan_hint != 0;
+  if (S.nan_hint) {
     uint32_t* kw = reinterpret_cast<uint32_t*>(keys4);
     bool seen = false;
-    for (int t = tid; t < n; t += NT) {
-      const int lo = max(0, t - hw), hi = min(n - 1, t + hw);
+    for (int t = max(0, slot0 - off) + tid; t < min(n, slot0 + 4 * ng - off); t += NT) {
+      const int lo = max(0, t - (STREAM ? 0 : hw)), hi = min(n - 1, t + (STREAM ? 0 : hw));
       float m = __ldg(v.sp + lo);
       bool nan_w = isnan(m);
       for (int x = lo + 1; x <= hi; ++x) {
@@ -874,15 +1050,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
         m = fmaxf(m, f);
       }
       seen |= nan_w;
-      kw[t + off] = nan_w ? 0u : ordered_key(m);
+      if (!STREAM) kw[t + off - slot0] = nan_w ? 0u : ordered_key(m);
     }
     if (__any_sync(0xffffffffu, seen) && lane == 0) S.nan_seen = 1;
   }
-  __syncthreads();
 
-  // ---- quotas and the role -> code table
-  if (warp == 0) quotas_warp(a, lane, K_s - n_floor, S);
-  __syncthreads();
+  // ---- the role -> code table
   for (int x = tid; x < 256; x += NT) {
     uint32_t code = kCodeDrop;
     if (x < a.n_roles && !((a.ban_mask >> x) & 1u)) {
@@ -891,68 +1064,247 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
     }
     S.code_of_role[x] = static_cast<int32_t>(code);
   }
-  const bool any_thr = S.any_threshold != 0;
-  if (tid == 0 && (S.nan_hint || ((S.top_and ^ S.top_or) & 0x80000000u))) S.general = 1;
+  const bool any_thr = warp_uniform(S.any_threshold) != 0;
+  const bool try_fast = warp_uniform(S.general) == 0;            // (the same in every rank)
   __syncthreads();
 
   // ---- first digit per bucket
-  if (any_thr && !S.general) {
-    if (warp < kR && S.mode[warp] == 2) {
-      if (STREAM)
-        descend_first32<11>(a, S, hist16, warp, lane);
-      else if (nb == 11)
-        descend_first<11>(a, S, hist16, warp, lane);
-      else
-        descend_first<10>(a, S, hist16, warp, lane);
+  if (any_thr && try_fast) {
+    if constexpr (CL) {
+      // bucket b by rank b mod C, over the ranks' summed histograms
+      for (int b = rank; b < p.n_hist; b += ranks) {
+        if (warp_uniform(S.mode[b]) != 2) continue;
+        const int wpr = 1 << (nb - 1);
+        for (int x = tid; x < wpr / 4; x += NT) {
+          int c[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+          int4 v4[kMaxRanks];                      // (all ranks' loads in flight)
+#pragma unroll
+          for (int k = 0; k < kMaxRanks; ++k)
+            v4[k] = k < ranks ? ld_rank4(map_rank(hist16 + b * wpr + 4 * x, k)) : make_int4(0, 0, 0, 0);
+#pragma unroll
+          for (int k = 0; k < kMaxRanks; ++k) {
+            const int4 w = v4[k];
+            c[0] += w.x & 0xFFFF; c[1] += static_cast<uint32_t>(w.x) >> 16;
+            c[2] += w.y & 0xFFFF; c[3] += static_cast<uint32_t>(w.y) >> 16;
+            c[4] += w.z & 0xFFFF; c[5] += static_cast<uint32_t>(w.z) >> 16;
+            c[6] += w.w & 0xFFFF; c[7] += static_cast<uint32_t>(w.w) >> 16;
+          }
+          reinterpret_cast<int4*>(hist)[2 * x] = make_int4(c[0], c[1], c[2], c[3]);
+          reinterpret_cast<int4*>(hist)[2 * x + 1] = make_int4(c[4], c[5], c[6], c[7]);
+        }
+        __syncthreads();
+        if (warp == 0) {
+          if (nb == 11)
+            descend_first_sums<11>(S, hist, b, lane, ranks);
+          else
+            descend_first_sums<10>(S, hist, b, lane, ranks);
+        }
+        __syncthreads();
+      }
+    } else {
+      for (int b = warp; b < p.n_hist; b += NW) {
+        if (warp_uniform(S.mode[b]) != 2) continue;
+        if (STREAM)
+          descend_first_sums<11>(S, reinterpret_cast<const int32_t*>(hist16) + (b << 11), b, lane, 1);
+        else if (nb == 11)
+          descend_first<11>(a, S, hist16, b, lane);
+        else
+          descend_first<10>(a, S, hist16, b, lane);
+      }
+    }
+    if (CL || STREAM) {                            // (found by another rank, or in the sums' form)
+      unit_sync<CL>();
+      if (tid < p.n_hist && S.mode[tid] == 2) {
+        S.prefix[tid] = S.f_prefix[tid];
+        S.need[tid] = S.f_need[tid];
+        S.cand[tid] = S.f_cand[tid];
+      }
+      if (tid == 0 && S.f_fail) S.general = 1;
     }
     __syncthreads();
   }
   // SLACK: the fill's first digit from the same histograms, before their
-  // region becomes the candidate list (in-memory rows; 16-bit bins)
-  if (!STREAM && S.slack > 0 && !S.general) {
-    // (S.hist, zero until the refinement rounds, serves as the bin counts)
-    static_assert(kR * 256 >= 2048, "bin counts for an 11-bit digit");
+  // region becomes the candidate list
+  const bool slack_fast = !STREAM && warp_uniform(S.slack) > 0 && warp_uniform(S.general) == 0;
+  if (slack_fast) {
     if (nb == 11)
-      slack_first<11, NT>(a, S, hist16, &S.hist[0][0], list_cap);
+      slack_first<11, NT, CL>(a, S, hist16, hist, list_cap, 4 * gs, rank, ranks);
     else
-      slack_first<10, NT>(a, S, hist16, &S.hist[0][0], list_cap);
+      slack_first<10, NT, CL>(a, S, hist16, hist, list_cap, 4 * gs, rank, ranks);
   }
+  if ((CL && any_thr && try_fast) || slack_fast) {
+    for (int x = tid; x < p.hist_ints; x += NT) hist[x] = 0;   // (the sums above)
+    __syncthreads();
+  }
+
+  // A digit round over counts the threads added to cur_hist(): the ranks meet,
+  // the warps of every rank find the buckets' digits, and the other buffer
+  // (read by the ranks a round ago) is cleared for the next round.
+  int round_no = 0;
+  auto cur_hist = [&]() { return hist + (round_no & 1) * hsz; };
+  auto end_round = [&](int shift, bool fill) {
+    unit_sync<CL>();
+    const int32_t* H = cur_hist();
+    for (int b = warp; b < (fill ? 1 : p.n_hist); b += NW)
+      if (fill || warp_uniform(S.mode[b]) == 2) descend<CL>(S, H, ranks, b, lane, shift);
+    ++round_no;
+    int32_t* O = cur_hist();
+    for (int x = tid; x < hsz; x += NT) O[x] = 0;
+    __syncthreads();
+  };
+
   // While the keys at the buckets' first digits overflow the list (scores in
   // a narrow range, such as page bounds), one full pass per 8 more bits.
   int shd = 31 - nb;   // key bits below the decided prefixes
-  if (any_thr && !S.general) {
-    auto cand_total = [&]() {
-      int t = 0;
-      for (int b = 0; b < kR; ++b) t += S.mode[b] == 2 ? S.cand[b] : 0;
-      return t;
+  bool general = warp_uniform(S.general) != 0;
+  if (any_thr && !general) {
+    auto overflows = [&]() {
+      const int t = __reduce_add_sync(0xffffffffu, lane < p.n_hist && S.mode[lane] == 2 ? S.cand[lane] : 0);
+      return min(t, 4 * gs) > list_cap;
     };
-    while (cand_total() > list_cap && shd > 8) {
+    while (overflows() && shd > 8) {
       const int shift = shd - 8;
+      int32_t* H = cur_hist();
       for (int i = 0; i < iters; ++i) {
-        const int g = i * NT + tid;
-        if (g >= ngroups) break;
-        const uint4 kv = kv_of(g);
+        const int lg = i * NT + tid;
+        if (lg >= ng) break;
+        const uint4 kv = kv_of(lg);
         const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
-        const uint32_t rw = load_roles(v.rp, off, n, g, v.rvec);
-        const uint32_t fb = floor_bits(4 * g - off, v.nf, n);
+        const uint32_t rw = load_roles(v.rp, off, n, g0 + lg, v.rvec);
+        const uint32_t fb = floor_bits(4 * (g0 + lg) - off, v.nf, n);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const uint32_t c = static_cast<uint32_t>(S.code_of_role[(rw >> (8 * j)) & 0xFFu]);
           if (c >= static_cast<uint32_t>(kR) || ((fb >> j) & 1u)) continue;
           if ((kk[j] >> shd) != (S.prefix[c] >> shd)) continue;
-          atomicAdd(&S.hist[c][(kk[j] >> shift) & 0xFFu], 1);
+          atomicAdd(&H[c * 256 + ((kk[j] >> shift) & 0xFFu)], 1);
         }
       }
-      __syncthreads();
-      if (warp < kR && S.mode[warp] == 2) descend(S, warp, lane, shift);
-      __syncthreads();
+      end_round(shift, false);
       shd = shift;
     }
-    if (tid == 0 && cand_total() > list_cap) S.general = 1;
-    __syncthreads();
+    general = overflows();
   }
 
-  if (!S.general) {
+  // Ties of bucket b's threshold beyond the shared list, over the rank's
+  // slots: the first `need` of the words' tie bits join the keep bits.
+  auto keep_ties = [&](int need) {
+    return [&bits, need](int q, uint32_t mk, int rank0) {
+      uint32_t keepm = 0;
+      while (mk != 0 && rank0 < need) {
+        const uint32_t low = mk & (0u - mk);
+        keepm |= low;
+        mk ^= low;
+        ++rank0;
+      }
+      if (keepm) bits[q] |= keepm;
+    };
+  };
+  // need ties of the unit less those the ranks before this one hold
+  auto need_here = [&](int need, const int32_t* l_ties) {
+    if constexpr (CL)
+      for (int k = 0; k < rank; ++k) need -= ld_rank(map_rank(l_ties, k));
+    return need;
+  };
+  // slots of word q whose key is `key` and whose bucket is b
+  auto bucket_ties = [&](int b, uint32_t key) {
+    return [&, b, key](int q) {
+      uint32_t mk = 0;
+#pragma unroll
+      for (int gg = 0; gg < 8; ++gg) {
+        const int lg = 8 * q + gg;
+        if (lg >= ng) break;
+        const uint4 kv = kv_of(lg);
+        const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
+        const uint32_t rw = load_roles(v.rp, off, n, g0 + lg, v.rvec);
+        const uint32_t fb = floor_bits(4 * (g0 + lg) - off, v.nf, n);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (S.code_of_role[(rw >> (8 * j)) & 0xFFu] == b && kk[j] == key && !((fb >> j) & 1u))
+            mk |= 1u << (4 * gg + j);
+      }
+      return mk;
+    };
+  };
+
+  // Appends the slots of c4's bits (entries ent, keys kk) to the rank's list; the lane's
+  // rank among the warp's candidates comes from four ballots.
+  auto append = [&](uint32_t c4, const uint32_t* ent, const uint32_t* kk) {
+    const int nc = __popc(c4);
+    const unsigned b1 = __ballot_sync(0xffffffffu, nc >= 1);
+    if (b1 == 0) return;
+    const unsigned b2 = __ballot_sync(0xffffffffu, nc >= 2);
+    const unsigned b3 = __ballot_sync(0xffffffffu, nc >= 3);
+    const unsigned b4 = __ballot_sync(0xffffffffu, nc >= 4);
+    const unsigned lt = (1u << lane) - 1u;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(&S.list_n, __popc(b1) + __popc(b2) + __popc(b3) + __popc(b4));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    int pos = base + __popc(b1 & lt) + __popc(b2 & lt) + __popc(b3 & lt) + __popc(b4 & lt);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if ((c4 >> j) & 1u) {
+        if (pos < list_cap) {                      // (the counts bound the list)
+          if (STREAM) {
+            list[2 * pos] = kk[j];
+            list[2 * pos + 1] = ent[j];
+          } else {
+            list[pos] = ent[j];
+          }
+        }
+        ++pos;
+      }
+  };
+
+  // Short lists (one rank): each candidate counts the candidates of its bucket
+  // that come before it (larger key, or equal key and lower slot) and is kept
+  // when fewer than need[b] do -- no digit rounds, no ties apart.  The list's
+  // m entries are first sorted into bucket runs of cand_of(b) keys, held
+  // beside the complemented slot as one 64-bit word, in the digit-count
+  // buffers.  Returns false, with nothing done, when the runs are too long: 36
+  // candidates in four runs take 2.4k cycles against 6.8k for three digit
+  // rounds and the tie step, 274 take 10k.
+  auto keep_by_rank = [&](int m, const int32_t* need, auto cand_of) {
+    const int c = lane < p.n_hist ? cand_of(lane) : 0;
+    int start = c;
+#pragma unroll
+    for (int o = 1; o < kR; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, start, o);
+      if (lane >= o) start += x;
+    }
+    start -= c;
+    const int cost = __reduce_add_sync(0xffffffffu, min(c, 1024) * min(c, 1024));
+    const int total = __reduce_add_sync(0xffffffffu, c);
+    if (cost > kRankCost || 2 * m > p.hist_ints || total != m) return false;
+    if (warp == 0 && lane < kR) {
+      S.run0[lane] = start;
+      S.run_n[lane] = 0;
+    }
+    __syncthreads();
+    uint64_t* runs = reinterpret_cast<uint64_t*>(hist);
+    for (int e = tid; e < m; e += NT) {
+      const uint32_t ent = list[e], b = ent >> 16, slot = ent & 0xFFFFu;
+      runs[S.run0[b] + atomicAdd(&S.run_n[b], 1)] =
+          (static_cast<uint64_t>(keys[slot]) << 16) | (0xFFFFu - slot);
+    }
+    __syncthreads();
+    for (int e = tid; e < m; e += NT) {
+      const uint32_t ent = list[e], b = ent >> 16, slot = ent & 0xFFFFu;
+      const uint64_t mine = (static_cast<uint64_t>(keys[slot]) << 16) | (0xFFFFu - slot);
+      const uint64_t* run = runs + S.run0[b];
+      const int nr = S.run_n[b];
+      int before = 0;
+#pragma unroll 4
+      for (int x = 0; x < nr; ++x) before += run[x] > mine;
+      if (before < need[b]) atomicOr(&bits[slot >> 5], 1u << (slot & 31u));
+    }
+    __syncthreads();
+    for (int x = tid; x < 2 * m; x += NT) hist[x] = 0;
+    __syncthreads();
+    return true;
+  };
+
+  if (!general) {
     for (int x = tid; x < 256; x += NT) {
       const uint32_t code = static_cast<uint32_t>(S.code_of_role[x]);
       S.first_of_role[x] = code == kCodeKeep                  ? -1
@@ -964,25 +1316,25 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
     // list the rest
     // roles are read two iterations ahead of their use (they come from L2)
     auto roles_of = [&](int i) {
-      const int g = i * NT + tid;
-      return (i < iters && g < ngroups) ? load_roles(v.rp, off, n, g, v.rvec) : 0xFFFFFFFFu;
+      const int lg = i * NT + tid;
+      return (i < iters && lg < ng) ? load_roles(v.rp, off, n, g0 + lg, v.rvec) : 0xFFFFFFFFu;
     };
     uint32_t r_next = roles_of(0), r_after = roles_of(1);
     for (int i = 0; i < iters; ++i) {
-      const int g = i * NT + tid;
+      const int lg = i * NT + tid;
       const uint32_t rw = r_next;
       r_next = r_after;
       r_after = roles_of(i + 2);
       uint32_t m4 = 0, c4 = 0;
       uint32_t ent[4] = {0u, 0u, 0u, 0u};
       uint32_t kk[4] = {0u, 0u, 0u, 0u};
-      if (g < ngroups) {
-        const uint4 kv = kv_of(g);
+      if (lg < ng) {
+        const uint4 kv = kv_of(lg);
         kk[0] = kv.x;
         kk[1] = kv.y;
         kk[2] = kv.z;
         kk[3] = kv.w;
-        const uint32_t fb = floor_bits(4 * g - off, v.nf, n);
+        const uint32_t fb = floor_bits(4 * (g0 + lg) - off, v.nf, n);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const uint32_t r = (rw >> (8 * j)) & 0xFFu;
@@ -991,101 +1343,76 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
           m4 |= static_cast<uint32_t>(hb > T) << j;
           if (hb == T && !((fb >> j) & 1u)) {
             c4 |= 1u << j;
-            ent[j] = (static_cast<uint32_t>(S.code_of_role[r]) << (STREAM ? 24 : 16)) |
-                     static_cast<uint32_t>(4 * g + j);
+            ent[j] = (static_cast<uint32_t>(S.code_of_role[r]) << kCodeShift) | static_cast<uint32_t>(4 * lg + j);
           }
         }
         m4 |= fb;                                  // the recency floor is kept
       }
-      store_bits(bits, g, nwords, lane, m4);
-      // list slots: lane's rank among the warp's candidates from four ballots
-      const int nc = __popc(c4);
-      const unsigned b1 = __ballot_sync(0xffffffffu, nc >= 1);
-      if (b1 != 0) {
-        const unsigned b2 = __ballot_sync(0xffffffffu, nc >= 2);
-        const unsigned b3 = __ballot_sync(0xffffffffu, nc >= 3);
-        const unsigned b4 = __ballot_sync(0xffffffffu, nc >= 4);
-        const unsigned lt = (1u << lane) - 1u;
-        int base = 0;
-        if (lane == 0) base = atomicAdd(&S.list_n, __popc(b1) + __popc(b2) + __popc(b3) + __popc(b4));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        int pos = base + __popc(b1 & lt) + __popc(b2 & lt) + __popc(b3 & lt) + __popc(b4 & lt);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if ((c4 >> j) & 1u) {
-            if (pos < list_cap) {
-              if (STREAM) {
-                list[2 * pos] = kk[j];
-                list[2 * pos + 1] = ent[j];
-              } else {
-                list[pos] = ent[j];
-              }
-            }
-            ++pos;
-          }
-      }
+      store_bits(bits, lg, nwords, lane, m4);
+      append(c4, ent, kk);
     }
     __syncthreads();
-    if (S.list_n > list_cap) {
-      if (tid == 0) S.general = 1;   // (cannot happen: the counts bound the list)
-      __syncthreads();
-    }
   }
 
-  if (!S.general) {
+  if (!general) {
     if (any_thr) {
-      // ---- remaining bits over the candidate list
-      const int m = S.list_n;
-      for (int lo = shd; lo > 0;) {
+      // ---- remaining bits over the candidate lists
+      const int m = warp_uniform(min(S.list_n, list_cap));
+      bool counted = false;
+      if constexpr (MODE == kOne) counted = keep_by_rank(m, S.need, [&](int b) { return S.mode[b] == 2 ? S.cand[b] : 0; });
+      for (int lo = counted ? 0 : shd; lo > 0;) {
         const int d = lo < 8 ? lo : 8;
         const int shift = lo - d;
+        int32_t* H = cur_hist();
         for (int e = tid; e < m; e += NT) {
-          const uint32_t ent = STREAM ? list[2 * e + 1] : list[e];
-          const uint32_t c = STREAM ? ent >> 24 : ent >> 16;
-          const uint32_t key = STREAM ? list[2 * e] : keys[ent & 0xFFFFu];
+          const uint32_t c = entry(e) >> kCodeShift;
+          const uint32_t key = entry_key(e);
           if ((key >> lo) == (S.prefix[c] >> lo))
-            atomicAdd(&S.hist[c][(key >> shift) & ((1u << d) - 1u)], 1);
+            atomicAdd(&H[c * 256 + ((key >> shift) & ((1u << d) - 1u))], 1);
         }
-        __syncthreads();
-        if (warp < kR && S.mode[warp] == 2) descend(S, warp, lane, shift);
-        __syncthreads();
+        end_round(shift, false);
         lo = shift;
       }
       // kept candidates join the bits; ties of partial buckets are gathered
-      const uint32_t partial = S.partial_ties;
-      for (int e = tid; e < m; e += NT) {
-        const uint32_t ent = STREAM ? list[2 * e + 1] : list[e];
-        const uint32_t c = STREAM ? ent >> 24 : ent >> 16;
-        const uint32_t slot = STREAM ? ent & 0xFFFFFFu : ent & 0xFFFFu;
-        const uint32_t key = STREAM ? list[2 * e] : keys[slot];
+      const uint32_t partial = warp_uniform(S.partial_ties);
+      for (int e = tid; e < (counted ? 0 : m); e += NT) {
+        const uint32_t ent = entry(e);
+        const uint32_t c = ent >> kCodeShift;
+        const uint32_t slot = ent & kSlotMask;
+        const uint32_t key = entry_key(e);
         if (key >= S.thr[c]) {
           atomicOr(&bits[slot >> 5], 1u << (slot & 31u));
         } else if (((partial >> c) & 1u) && key == S.prefix[c]) {
+          atomicAdd(&S.l_ties[c], 1);
           const int t = atomicAdd(&S.tie_n, 1);
           if (t < kTieCap) S.ties[t] = ent;
         }
       }
-      __syncthreads();
-      const int nt = S.tie_n;
-      if (partial != 0 && nt <= kTieCap) {
-        // index-order rank among the bucket's ties
-        constexpr int kCodeShift = STREAM ? 24 : 16;
-        constexpr uint32_t kSlotMask = STREAM ? 0xFFFFFFu : 0xFFFFu;
-        for (int t = tid; t < nt; t += NT) {
-          const uint32_t ent = S.ties[t];
-          const uint32_t c = ent >> kCodeShift, slot = ent & kSlotMask;
-          int rank = 0;
-          for (int x = 0; x < nt; ++x) {
-            const uint32_t o = S.ties[x];
-            rank += ((o >> kCodeShift) == c && (o & kSlotMask) < slot);
+      if (partial != 0) {                          // (the same in every rank)
+        unit_sync<CL>();
+        const int nt = warp_uniform(S.tie_n);
+        if (nt <= kTieCap) {
+          // index-order rank among the bucket's ties
+          for (int t = tid; t < nt; t += NT) {
+            const uint32_t ent = S.ties[t];
+            const uint32_t c = ent >> kCodeShift, slot = ent & kSlotMask;
+            int before = 0;
+            for (int x = 0; x < nt; ++x) {
+              const uint32_t o = S.ties[x];
+              before += ((o >> kCodeShift) == c && (o & kSlotMask) < slot);
+            }
+            if (before < need_here(S.need[c], &S.l_ties[c])) atomicOr(&bits[slot >> 5], 1u << (slot & 31u));
           }
-          if (rank < S.need[c]) atomicOr(&bits[slot >> 5], 1u << (slot & 31u));
+        } else {
+          for (uint32_t pend = partial; pend != 0; pend &= pend - 1) {
+            const int b = __ffs(pend) - 1;
+            auto mask_of = bucket_ties(b, S.prefix[b]);
+            count_words<NT>(nwords, mask_of, S.warp_tot);
+            scan_words<NT>(nwords, 0, mask_of, keep_ties(need_here(S.need[b], &S.l_ties[b])), S.warp_tot);
+          }
         }
-        __syncthreads();
-      } else if (partial != 0) {
-        if (tid == 0) S.general = 2;   // too many ties: rank them over all slots
-        __syncthreads();
       }
+      __syncthreads();
     }
   } else {
     // ---- general path: four 8-bit rounds over every slot, from the top
@@ -1094,322 +1421,294 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
       S.prefix[tid] = 0;
       S.need[tid] = S.quota[tid];
     }
+    if (tid == 0) S.partial_ties = 0;
     __syncthreads();
     for (int round = 0; round < (any_thr ? 4 : 0); ++round) {
       const int shift = 24 - 8 * round;
+      int32_t* H = cur_hist();
       for (int i = 0; i < iters; ++i) {
-        const int g = i * NT + tid;
-        if (g >= ngroups) break;
-        const uint4 kv = kv_of(g);
+        const int lg = i * NT + tid;
+        if (lg >= ng) break;
+        const uint4 kv = kv_of(lg);
         const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
-        const uint32_t rw = load_roles(v.rp, off, n, g, v.rvec);
-        const uint32_t fb = floor_bits(4 * g - off, v.nf, n);
+        const uint32_t rw = load_roles(v.rp, off, n, g0 + lg, v.rvec);
+        const uint32_t fb = floor_bits(4 * (g0 + lg) - off, v.nf, n);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const uint32_t c = static_cast<uint32_t>(S.code_of_role[(rw >> (8 * j)) & 0xFFu]);
           if (c >= static_cast<uint32_t>(kR) || ((fb >> j) & 1u)) continue;
           if (round > 0 && (kk[j] >> (shift + 8)) != (S.prefix[c] >> (shift + 8))) continue;
-          atomicAdd(&S.hist[c][(kk[j] >> shift) & 0xFFu], 1);
+          atomicAdd(&H[c * 256 + ((kk[j] >> shift) & 0xFFu)], 1);
         }
       }
-      __syncthreads();
-      if (warp < kR && S.mode[warp] == 2) descend(S, warp, lane, shift);
-      __syncthreads();
+      end_round(shift, false);
     }
     for (int i = 0; i < iters; ++i) {
-      const int g = i * NT + tid;
+      const int lg = i * NT + tid;
       uint32_t m4 = 0;
-      if (g < ngroups) {
-        const uint4 kv = kv_of(g);
+      if (lg < ng) {
+        const uint4 kv = kv_of(lg);
         const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
-        const uint32_t rw = load_roles(v.rp, off, n, g, v.rvec);
+        const uint32_t rw = load_roles(v.rp, off, n, g0 + lg, v.rvec);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const uint32_t c = static_cast<uint32_t>(S.code_of_role[(rw >> (8 * j)) & 0xFFu]);
           const bool keep = (c < static_cast<uint32_t>(kR)) ? (kk[j] >= S.thr[c]) : (c == kCodeKeep);
           m4 |= static_cast<uint32_t>(keep) << j;
         }
-        m4 |= floor_bits(4 * g - off, v.nf, n);    // the recency floor is kept
+        m4 |= floor_bits(4 * (g0 + lg) - off, v.nf, n);    // the recency floor is kept
       }
-      store_bits(bits, g, nwords, lane, m4);
+      store_bits(bits, lg, nwords, lane, m4);
     }
     __syncthreads();
-  }
-
-  // Ties beyond the shared-memory list (general path, or too many ties): the
-  // first need[b] keys equal to the threshold, in index order, over all slots.
-  if (S.general) {
-    for (uint32_t pend = S.partial_ties; pend != 0; pend &= pend - 1) {
+    // the first need[b] keys equal to the threshold, in index order
+    const uint32_t partial = warp_uniform(S.partial_ties);
+    for (uint32_t pend = partial; CL && pend != 0; pend &= pend - 1) {
       const int b = __ffs(pend) - 1;
-      const uint32_t P = S.prefix[b];
-      const int need = S.need[b];
-      auto tie_mask = [&](int q) {
-        uint32_t mk = 0;
-#pragma unroll
-        for (int gg = 0; gg < 8; ++gg) {
-          const int g = 8 * q + gg;
-          if (g >= ngroups) break;
-          const uint4 kv = kv_of(g);
-          const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
-          const uint32_t rw = load_roles(v.rp, off, n, g, v.rvec);
-          const uint32_t fb = floor_bits(4 * g - off, v.nf, n);
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (S.code_of_role[(rw >> (8 * j)) & 0xFFu] == b && kk[j] == P && !((fb >> j) & 1u))
-              mk |= 1u << (4 * gg + j);
-        }
-        return mk;
-      };
-      scan_words<NT>(nwords, tie_mask, [&](int q, uint32_t mk, int rank) {
-        uint32_t keepm = 0;
-        while (mk != 0 && rank < need) {
-          const uint32_t low = mk & (0u - mk);
-          keepm |= low;
-          mk ^= low;
-          ++rank;
-        }
-        if (keepm) bits[q] |= keepm;
-      }, S.warp_tot);
+      const int c = count_words<NT>(nwords, bucket_ties(b, S.prefix[b]), S.warp_tot);
+      if (tid == 0) S.l_ties[b] = c;
+      __syncthreads();
+    }
+    if (partial != 0) unit_sync<CL>();
+    for (uint32_t pend = partial; pend != 0; pend &= pend - 1) {
+      const int b = __ffs(pend) - 1;
+      auto mask_of = bucket_ties(b, S.prefix[b]);
+      count_words<NT>(nwords, mask_of, S.warp_tot);
+      scan_words<NT>(nwords, 0, mask_of, keep_ties(need_here(S.need[b], &S.l_ties[b])), S.warp_tot);
     }
   }
 
   // ---- SLACK: the slots saturated buckets left go to the best-scoring
   // tokens of eligible roles not kept yet (ties to the lower index).  With
   // the fill's first digit known (sfast), one pass keeps such tokens above
-  // it and lists those at it; the remaining bits are resolved over the list
-  // in the state of bucket 0, whose own selection is complete.
-  if (!STREAM && S.slack > 0 && S.sfast) {
+  // it and lists those at it and the remaining bits are resolved over the
+  // lists; otherwise four 8-bit rounds over all slots.  The digits go through
+  // the state of bucket 0, whose own selection is complete.
+  if (warp_uniform(S.slack) > 0) {
+    const bool fast = warp_uniform(S.sfast) != 0;
     const uint32_t elig = S.elig_mask;
     const int sh0 = 31 - nb;
     const uint32_t bmask = (1u << nb) - 1u;
     const uint32_t DS = (S.sprefix >> sh0) & bmask;
+    // an eligible slot no bucket keeps, before the recency floor
+    auto candidate = [&](uint32_t rw, uint32_t fk, int j) {
+      const uint32_t r = (rw >> (8 * j)) & 0xFFu;
+      return r < static_cast<uint32_t>(kR) && ((elig >> r) & 1u) && !((fk >> j) & 1u);
+    };
+    __syncthreads();
     if (tid == 0) {
       S.list_n = 0;
       S.tie_n = 0;
       S.partial_ties = 0;
-      S.prefix[0] = S.sprefix;
-      S.need[0] = S.sneed;
+      S.prefix[0] = fast ? S.sprefix : 0u;
+      S.need[0] = fast ? S.sneed : S.slack;
       S.thr[0] = 0xFFFFFFFFu;
     }
-    for (int x = tid; x < 256; x += NT) S.hist[0][x] = 0;
     __syncthreads();
-    for (int i = 0; i < iters; ++i) {
-      const int g = i * NT + tid;
-      uint32_t m4 = 0, c4 = 0;
-      if (g < ngroups) {
-        const uint4 kv = keys4[g];
-        const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
-        const uint32_t rw = load_roles(v.rp, off, n, g, v.rvec);
-        const uint32_t fb = floor_bits(4 * g - off, v.nf, n);
-        const uint32_t kb = (bits[g >> 3] >> (4 * (g & 7))) & 0xFu;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t r = (rw >> (8 * j)) & 0xFFu;
-          if (r >= static_cast<uint32_t>(kR) || !((elig >> r) & 1u) || ((fb | kb) >> j) & 1u) continue;
-          const uint32_t d = (kk[j] >> sh0) & bmask;
-          m4 |= static_cast<uint32_t>(d > DS) << j;
-          c4 |= static_cast<uint32_t>(d == DS) << j;
-        }
-        if (m4) atomicOr(&bits[g >> 3], m4 << (4 * (g & 7)));
-      }
-      const int nc = __popc(c4);
-      const unsigned b1 = __ballot_sync(0xffffffffu, nc >= 1);
-      if (b1 != 0) {
-        const unsigned b2 = __ballot_sync(0xffffffffu, nc >= 2);
-        const unsigned b3 = __ballot_sync(0xffffffffu, nc >= 3);
-        const unsigned b4 = __ballot_sync(0xffffffffu, nc >= 4);
-        const unsigned lt = (1u << lane) - 1u;
-        int base = 0;
-        if (lane == 0) base = atomicAdd(&S.list_n, __popc(b1) + __popc(b2) + __popc(b3) + __popc(b4));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        int pos = base + __popc(b1 & lt) + __popc(b2 & lt) + __popc(b3 & lt) + __popc(b4 & lt);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if ((c4 >> j) & 1u) {
-            if (pos < list_cap) list[pos] = static_cast<uint32_t>(4 * g + j);
-            ++pos;
-          }
-      }
-    }
-    __syncthreads();
-    // (the histograms bound the listed count by list_cap)
-    const int m = S.list_n < list_cap ? S.list_n : list_cap;
-    for (int lo = sh0; lo > 0;) {
-      const int d = lo < 8 ? lo : 8;
-      const int shift = lo - d;
-      for (int e = tid; e < m; e += NT) {
-        const uint32_t key = keys[list[e]];
-        if ((key >> lo) == (S.prefix[0] >> lo)) atomicAdd(&S.hist[0][(key >> shift) & ((1u << d) - 1u)], 1);
-      }
-      __syncthreads();
-      if (warp == 0) descend(S, 0, lane, shift);
-      __syncthreads();
-      lo = shift;
-    }
-    const uint32_t T = S.thr[0], P = S.prefix[0];
-    const int need = S.need[0];
-    const bool partial = S.partial_ties & 1u;
-    for (int e = tid; e < m; e += NT) {
-      const uint32_t slot = list[e];
-      const uint32_t key = keys[slot];
-      if (key >= T) {
-        atomicOr(&bits[slot >> 5], 1u << (slot & 31u));
-      } else if (partial && key == P) {
-        const int t = atomicAdd(&S.tie_n, 1);
-        if (t < kTieCap) S.ties[t] = slot;
-      }
-    }
-    __syncthreads();
-    const int nt = S.tie_n;
-    if (partial && nt <= kTieCap) {
-      // index-order rank among the fill's ties
-      for (int t = tid; t < nt; t += NT) {
-        const uint32_t slot = S.ties[t];
-        int rank = 0;
-        for (int x = 0; x < nt; ++x) rank += S.ties[x] < slot;
-        if (rank < need) atomicOr(&bits[slot >> 5], 1u << (slot & 31u));
-      }
-      __syncthreads();
-    } else if (partial) {
-      // more ties than the shared list holds: rank them over all slots
-      auto tie_mask = [&](int q) {
-        uint32_t mk = 0;
-#pragma unroll
-        for (int gg = 0; gg < 8; ++gg) {
-          const int g = 8 * q + gg;
-          if (g >= ngroups) break;
-          const uint4 kv = keys4[g];
+    auto kept4 = [&](int lg) { return (bits[lg >> 3] >> (4 * (lg & 7))) & 0xFu; };
+    int m = 0;
+    if (fast) {
+      for (int i = 0; i < iters; ++i) {
+        const int lg = i * NT + tid;
+        uint32_t m4 = 0, c4 = 0;
+        uint32_t ent[4] = {0u, 0u, 0u, 0u};
+        if (lg < ng) {
+          const uint4 kv = kv_of(lg);
           const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
-          const uint32_t rw = load_roles(v.rp, off, n, g, v.rvec);
-          const uint32_t fb = floor_bits(4 * g - off, v.nf, n);
+          const uint32_t rw = load_roles(v.rp, off, n, g0 + lg, v.rvec);
+          const uint32_t fk = floor_bits(4 * (g0 + lg) - off, v.nf, n) | kept4(lg);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const uint32_t r = (rw >> (8 * j)) & 0xFFu;
-            const int slot = 4 * g + j;
-            if (kk[j] == P && r < static_cast<uint32_t>(kR) && ((elig >> r) & 1u) && !((fb >> j) & 1u) &&
-                !((bits[slot >> 5] >> (slot & 31)) & 1u))
-              mk |= 1u << (4 * gg + j);
+            if (!candidate(rw, fk, j)) continue;
+            const uint32_t d = (kk[j] >> sh0) & bmask;
+            m4 |= static_cast<uint32_t>(d > DS) << j;
+            c4 |= static_cast<uint32_t>(d == DS) << j;
+            ent[j] = static_cast<uint32_t>(4 * lg + j);
           }
+          if (m4) atomicOr(&bits[lg >> 3], m4 << (4 * (lg & 7)));
         }
-        return mk;
-      };
-      scan_words<NT>(nwords, tie_mask, [&](int q, uint32_t mk, int rank) {
-        uint32_t keepm = 0;
-        while (mk != 0 && rank < need) {
-          const uint32_t low = mk & (0u - mk);
-          keepm |= low;
-          mk ^= low;
-          ++rank;
+        append(c4, ent, ent);                      // (held keys: not stored in the list)
+      }
+      __syncthreads();
+      m = warp_uniform(min(S.list_n, list_cap));
+      if constexpr (MODE == kOne)
+        if (keep_by_rank(m, S.need, [&](int b) { return b == 0 ? m : 0; })) m = 0;
+      for (int lo = m > 0 || MODE != kOne ? sh0 : 0; lo > 0;) {
+        const int d = lo < 8 ? lo : 8;
+        const int shift = lo - d;
+        int32_t* H = cur_hist();
+        for (int e = tid; e < m; e += NT) {
+          const uint32_t key = keys[list[e]];
+          if ((key >> lo) == (S.prefix[0] >> lo)) atomicAdd(&H[(key >> shift) & ((1u << d) - 1u)], 1);
         }
-        if (keepm) bits[q] |= keepm;
-      }, S.warp_tot);
-    }
-  } else if (S.slack > 0) {
-    const uint32_t elig = S.elig_mask;
-    auto candidate = [&](uint32_t rw, uint32_t fb, int g, int j) {
-      const uint32_t r = (rw >> (8 * j)) & 0xFFu;
-      const int slot = 4 * g + j;
-      return r < static_cast<uint32_t>(kR) && ((elig >> r) & 1u) && !((fb >> j) & 1u) &&
-             !((bits[slot >> 5] >> (slot & 31)) & 1u);
-    };
-    if (tid == 0) {
-      S.prefix[0] = 0;
-      S.need[0] = S.slack;
-      S.partial_ties = 0;
-    }
-    for (int x = tid; x < 256; x += NT) S.hist[0][x] = 0;
-    __syncthreads();
-    for (int round = 0; round < 4; ++round) {
-      const int shift = 24 - 8 * round;
-      for (int i = 0; i < iters; ++i) {
-        const int g = i * NT + tid;
-        if (g >= ngroups) break;
-        const uint4 kv = kv_of(g);
-        const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
-        const uint32_t rw = load_roles(v.rp, off, n, g, v.rvec);
-        const uint32_t fb = floor_bits(4 * g - off, v.nf, n);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (!candidate(rw, fb, g, j)) continue;
-          if (round > 0 && (kk[j] >> (shift + 8)) != (S.prefix[0] >> (shift + 8))) continue;
-          atomicAdd(&S.hist[0][(kk[j] >> shift) & 0xFFu], 1);
+        end_round(shift, true);
+        lo = shift;
+      }
+      const uint32_t T = S.thr[0], P = S.prefix[0];
+      const bool partial = S.partial_ties & 1u;
+      for (int e = tid; e < m; e += NT) {
+        const uint32_t slot = list[e];
+        const uint32_t key = keys[slot];
+        if (key >= T) {
+          atomicOr(&bits[slot >> 5], 1u << (slot & 31u));
+        } else if (partial && key == P) {
+          atomicAdd(&S.l_fill_ties, 1);
+          const int t = atomicAdd(&S.tie_n, 1);
+          if (t < kTieCap) S.ties[t] = slot;
         }
       }
       __syncthreads();
-      if (warp == 0) descend(S, 0, lane, shift);
+    } else {
+      for (int round = 0; round < 4; ++round) {
+        const int shift = 24 - 8 * round;
+        int32_t* H = cur_hist();
+        for (int i = 0; i < iters; ++i) {
+          const int lg = i * NT + tid;
+          if (lg >= ng) break;
+          const uint4 kv = kv_of(lg);
+          const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
+          const uint32_t rw = load_roles(v.rp, off, n, g0 + lg, v.rvec);
+          const uint32_t fk = floor_bits(4 * (g0 + lg) - off, v.nf, n) | kept4(lg);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (!candidate(rw, fk, j)) continue;
+            if (round > 0 && (kk[j] >> (shift + 8)) != (S.prefix[0] >> (shift + 8))) continue;
+            atomicAdd(&H[(kk[j] >> shift) & 0xFFu], 1);
+          }
+        }
+        end_round(shift, true);
+      }
+      // candidates above the threshold join
+      const uint32_t T = S.thr[0];
+      for (int i = 0; i < iters; ++i) {
+        const int lg = i * NT + tid;
+        if (lg >= ng) break;
+        const uint4 kv = kv_of(lg);
+        const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
+        const uint32_t rw = load_roles(v.rp, off, n, g0 + lg, v.rvec);
+        const uint32_t fk = floor_bits(4 * (g0 + lg) - off, v.nf, n) | kept4(lg);
+        uint32_t m4 = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (kk[j] >= T && candidate(rw, fk, j)) m4 |= 1u << j;
+        if (m4) atomicOr(&bits[lg >> 3], m4 << (4 * (lg & 7)));
+      }
       __syncthreads();
     }
-    // candidates above the threshold join; the rest of the ties in index order
-    const uint32_t T = S.thr[0], P = S.prefix[0];
-    const int need = S.need[0];
-    const bool partial = S.partial_ties & 1u;
-    __syncthreads();
-    for (int i = 0; i < iters; ++i) {
-      const int g = i * NT + tid;
-      if (g >= ngroups) break;
-      const uint4 kv = kv_of(g);
-      const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
-      const uint32_t rw = load_roles(v.rp, off, n, g, v.rvec);
-      const uint32_t fb = floor_bits(4 * g - off, v.nf, n);
-      uint32_t m4 = 0;
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (kk[j] >= T && candidate(rw, fb, g, j)) m4 |= 1u << j;
-      if (m4) atomicOr(&bits[g >> 3], m4 << (4 * (g & 7)));
-    }
-    __syncthreads();
-    if (partial) {
-      auto tie_mask = [&](int q) {
+    if (warp_uniform(S.partial_ties) & 1u) {       // (the same in every rank)
+      const uint32_t P = S.prefix[0];
+      auto mask_of = [&](int q) {
         uint32_t mk = 0;
 #pragma unroll
         for (int gg = 0; gg < 8; ++gg) {
-          const int g = 8 * q + gg;
-          if (g >= ngroups) break;
-          const uint4 kv = kv_of(g);
+          const int lg = 8 * q + gg;
+          if (lg >= ng) break;
+          const uint4 kv = kv_of(lg);
           const uint32_t kk[4] = {kv.x, kv.y, kv.z, kv.w};
-          const uint32_t rw = load_roles(v.rp, off, n, g, v.rvec);
-          const uint32_t fb = floor_bits(4 * g - off, v.nf, n);
+          const uint32_t rw = load_roles(v.rp, off, n, g0 + lg, v.rvec);
+          const uint32_t fk = floor_bits(4 * (g0 + lg) - off, v.nf, n) | kept4(lg);
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            if (kk[j] == P && candidate(rw, fb, g, j)) mk |= 1u << (4 * gg + j);
+            if (kk[j] == P && candidate(rw, fk, j)) mk |= 1u << (4 * gg + j);
         }
         return mk;
       };
-      scan_words<NT>(nwords, tie_mask, [&](int q, uint32_t mk, int rank) {
-        uint32_t keepm = 0;
-        while (mk != 0 && rank < need) {
-          const uint32_t low = mk & (0u - mk);
-          keepm |= low;
-          mk ^= low;
-          ++rank;
+      if (CL && !fast) {
+        const int c = count_words<NT>(nwords, mask_of, S.warp_tot);
+        if (tid == 0) S.l_fill_ties = c;
+      }
+      unit_sync<CL>();
+      const int need = need_here(S.need[0], &S.l_fill_ties);
+      const int nt = warp_uniform(S.tie_n);
+      if (fast && nt <= kTieCap) {
+        // index-order rank among the fill's ties
+        for (int t = tid; t < nt; t += NT) {
+          const uint32_t slot = S.ties[t];
+          int before = 0;
+          for (int x = 0; x < nt; ++x) before += S.ties[x] < slot;
+          if (before < need) atomicOr(&bits[slot >> 5], 1u << (slot & 31u));
         }
-        if (keepm) bits[q] |= keepm;
-      }, S.warp_tot);
+      } else {
+        // more ties than the shared list holds: rank them over all slots
+        count_words<NT>(nwords, mask_of, S.warp_tot);
+        scan_words<NT>(nwords, 0, mask_of, keep_ties(need), S.warp_tot);
+      }
+      __syncthreads();
     }
   }
 
   // ---- kept positions in ascending order
+  auto kept_bits = [&](int q) { return bits[q]; };
+  int total = count_words<NT>(nwords, kept_bits, S.warp_tot);
+  int base0 = 0;
+  if constexpr (CL) {
+    if (tid == 0) S.l_total = total;
+    unit_sync<CL>();
+    // lane k: rank k's total
+    const int t = lane < ranks ? ld_rank(map_rank(&S.l_total, lane)) : 0;
+    base0 = warp_sum(lane < rank ? t : 0);
+    total = warp_sum(t);
+  }
   int32_t* dst = a.keep_idx + S.keep_off;
   const bool count_roles = a.kept_per_role != nullptr &&
                            (a.policy == ROLEKV_POLICY_GLOBAL || a.policy == ROLEKV_POLICY_SLACK);
-  uint64_t kr = 0;
-  const int total = scan_words<NT>(nwords, [&](int q) { return bits[q]; }, [&](int q, uint32_t m, int pos) {
-    while (m != 0) {
-      const int t = q * 32 + (__ffs(m) - 1) - off;
-      m &= m - 1;
-      if (in_bounds(pos, 1, width, a.status)) dst[pos] = t;   // (the unit's own row)
-      ++pos;
-      if (count_roles) kr += shl64(1ull, 8u * __ldg(v.rp + t));
+  // Warp w writes its words' positions, 32 words at a time, a lane per output:
+  // the lane finds its word by a search over the words' prefix counts and its
+  // bit by halves (a lane per word waits for the fullest word, 6.5k cycles at
+  // 1024 words a CTA and a tenth kept; a lane per slot idles in nine of ten).
+  uint32_t kr[kR] = {0, 0, 0, 0, 0, 0, 0, 0};
+  {
+    const int wseg = (nwords + NW - 1) / NW;
+    const int q_end = min(nwords, (warp + 1) * wseg);
+    int pos0 = base0 + warp_sum(lane < warp ? S.warp_tot[lane] : 0);
+    for (int q0 = warp * wseg; q0 < q_end; q0 += 32) {
+      const uint32_t mine = q0 + lane < q_end ? bits[q0 + lane] : 0u;
+      int incl = __popc(mine);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+      }
+      const int tot = __shfl_sync(0xffffffffu, incl, 31);
+      for (int j0 = 0; j0 < tot; j0 += 32) {
+        const int j = min(j0 + lane, tot - 1);
+        int w = 0;                                 // first word with more than j bits up to it
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+          if (__shfl_sync(0xffffffffu, incl, w + o - 1) <= j) w += o;
+        uint32_t m = __shfl_sync(0xffffffffu, mine, w);
+        int r = j - (__shfl_sync(0xffffffffu, incl, w) - __popc(m));
+        int bit = 0;                               // position of the word's r-th set bit
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const int low = __popc(m & ((1u << o) - 1u));
+          if (r >= low) {
+            r -= low;
+            m >>= o;
+            bit += o;
+          }
+        }
+        const int pos = pos0 + j, t = slot0 + (q0 + w) * 32 + bit - off;
+        if (j0 + lane < tot) {
+          if (in_bounds(pos, 1, width, a.status)) dst[pos] = t;   // (the unit's own row)
+          if (count_roles) {
+            const uint32_t role = __ldg(v.rp + t);
+#pragma unroll
+            for (int x = 0; x < kR; ++x) kr[x] += role == static_cast<uint32_t>(x);
+          }
+        }
+      }
+      pos0 += tot;
     }
-  }, S.warp_tot);
-  for (int64_t j = total + tid; j < width; j += NT) dst[j] = -1;
+  }
+  for (int64_t j = total + rank * NT + tid; j < width; j += NT * ranks) dst[j] = -1;
 
   if (a.keep_mask != nullptr) {
     uint8_t* mp = a.keep_mask + sbase;
     const bool mvec = ((reinterpret_cast<uintptr_t>(mp) - static_cast<uintptr_t>(off)) & 3u) == 0;
-    for (int g = tid; g < ngroups; g += NT) {
-      const uint32_t m4 = (bits[g >> 3] >> (4 * (g & 7))) & 15u;
-      const int s0 = 4 * g - off;
+    for (int lg = tid; lg < ng; lg += NT) {
+      const uint32_t m4 = (bits[lg >> 3] >> (4 * (lg & 7))) & 15u;
+      const int s0 = 4 * (g0 + lg) - off;
       if (mvec && s0 >= 0 && s0 + 4 <= n) {
         const uint32_t w = (m4 & 1u) | ((m4 >> 1) & 1u) << 8 | ((m4 >> 2) & 1u) << 16 | ((m4 >> 3) & 1u) << 24;
         *reinterpret_cast<uint32_t*>(mp + s0) = w;
@@ -1421,47 +1720,110 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
     }
   }
 
-  if (a.kept_per_role != nullptr) {
-    if (count_roles) {
+  if (count_roles) {
 #pragma unroll
-      for (int r = 0; r < kR; ++r) {
-        const int c = warp_sum(static_cast<int>((kr >> (8 * r)) & 0xFFu));
-        if (lane == 0 && c) atomicAdd(&S.kept_role[r], c);
+    for (int r = 0; r < kR; ++r) {
+      const int c = static_cast<int>(__reduce_add_sync(0xffffffffu, kr[r]));
+      if (lane == 0 && c) {
+        if constexpr (CL)
+          add_rank(map_rank(&S.kept_role[r], 0), c);
+        else
+          atomicAdd(&S.kept_role[r], c);
       }
-      __syncthreads();
     }
-    if (tid < a.n_roles)
-      a.kept_per_role[static_cast<int64_t>(u) * a.n_roles + tid] =
-          count_roles ? S.kept_role[tid] : S.quota[tid] + S.floor_role[tid];
   }
+  // (no rank leaves while another may still read or add to its memory)
+  unit_sync<CL>();
+  if (rank == 0 && a.kept_per_role != nullptr && tid < a.n_roles)
+    a.kept_per_role[static_cast<int64_t>(u) * a.n_roles + tid] =
+        count_roles ? S.kept_role[tid] : S.quota[tid] + S.floor_role[tid];
   if (tid == 0 && S.nan_seen && a.status != nullptr) atomicOr(a.status, ROLEKV_STATUS_NONFINITE);
 }
 
-template <int NT, bool STREAM>
-cudaError_t launch_select_nt(const SelectArgs& a, size_t smem, cudaStream_t stream) {
-  cudaError_t e = cudaFuncSetAttribute(select_kernel<NT, STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+template <int NT, int MODE>
+cudaError_t launch_select_nt(const SelectArgs& a, const SelectPlan& p, size_t smem, cudaStream_t stream) {
+  cudaError_t e = cudaFuncSetAttribute(select_kernel<NT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  select_kernel<NT, STREAM><<<a.n_units, NT, smem, stream>>>(a);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(a.n_units) * p.ranks);
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(p.ranks);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = MODE == kCluster ? 1 : 0;
+  e = cudaLaunchKernelEx(&cfg, select_kernel<NT, MODE>, a, p);
+  if (e != cudaSuccess) return e;
   return cudaGetLastError();
+}
+
+// Route, ranks and threads of a unit, by the row length and the number of
+// units.  A unit on one CTA is bound by its serial phases (set-up, quotas,
+// digit searches: 8 us for the shortest row) and by its passes over shared
+// memory (about 6 us per 8192 tokens at 1024 threads); a cluster divides the
+// passes but pays some 1 us per exchange, eight of them.  Times on a GB300,
+// role quotas, pool 7, B = 0.1:
+//   8 units x 32768   one CTA 28.7 us, cluster of 4 22.5 us
+//   8 units x 131072  streaming 102.4 us, cluster of 4 36.4 us, of 8 36.8 us
+//   64 x 131072       streaming 103.4 us, cluster of 4 70.9 us (two waves)
+//   128 x 131072      streaming 103.5 us, cluster of 4 141 us (four waves)
+//   1024 x 32768      one CTA 200 us, cluster of 4 327 us (same threads)
+// so clusters are for batches that leave SMs idle: one wave of them up to
+// kSmemMaxN tokens, two beyond.  (At 8192 tokens a cluster of 4 takes 18.4 us
+// against 15.9 us for one CTA of 512 threads.)
+void plan_select(const SelectArgs& a, SelectPlan* p, int* mode, int* nt, size_t* smem) {
+  constexpr int kSms = 152;
+  const int groups = (a.n_max + 3 + 3) / 4;        // up to three leading slots
+  int ranks = 1;
+  *mode = kOne;
+  if (a.n_max > kSmemMaxN) {
+    ranks = a.n_max > 4 * 32768 + 64 ? 8 : 4;
+    *mode = static_cast<int64_t>(a.n_units) * ranks <= 2 * kSms ? kCluster : kStream;
+  } else if (a.n_max > 16384 && a.n_units <= kSms / 4) {
+    ranks = 4;
+    *mode = kCluster;
+  }
+  if (*mode == kStream) ranks = 1;
+  p->ranks = ranks;
+  p->groups = plan_groups(groups, ranks);
+  const int slots = p->groups * 4;                 // of one rank
+  const bool stream = *mode == kStream, wide = stream || slots > 16384 + 128;
+  // Threads: enough for a short latency while the SMs hold all units, no more
+  // than leave room for several units on an SM otherwise (1024 x 8192 tokens:
+  // 60.7 us at 256 threads, 66.7 at 512; 8 x 8192: 18.9 and 15.9 us).
+  *nt = wide ? 1024 : slots > 8192 + 128 || (slots > 2048 + 128 && a.n_units <= 4 * kSms) ? 512 : 256;
+  p->nb = wide ? 11 : 10;
+  p->n_hist = a.policy == ROLEKV_POLICY_GLOBAL ? 1 : a.n_roles;
+  p->list_cap = wide ? 8192 : slots < 4096 ? slots : 4096;
+  p->hist_ints = 2 * p->n_hist * 256;
+  if ((ranks > 1 || a.policy == ROLEKV_POLICY_SLACK) && p->hist_ints < (1 << p->nb)) p->hist_ints = 1 << p->nb;
+  p->region_words = p->n_hist << (stream ? p->nb : p->nb - 1);
+  const int list_words = stream ? 2 * p->list_cap : p->list_cap;
+  if (p->region_words < list_words) p->region_words = list_words;
+  *smem = (stream ? 0 : static_cast<size_t>(p->groups) * 16) + p->groups / 8 * 4 +
+          static_cast<size_t>(p->hist_ints) * 4 + static_cast<size_t>(p->region_words) * 4;
 }
 
 }  // namespace
 
-size_t select_smem_bytes(int n_max) {
-  const size_t groups = static_cast<size_t>(select_groups(n_max));
-  return (n_max > kSmemMaxN ? 0 : groups * 16) + groups / 8 * 4 + region_bytes(n_max);
-}
-
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t stream) {
   if (a.n_units == 0) return cudaSuccess;
-  const size_t smem = select_smem_bytes(a.n_max);
-  // CTA size follows the row length so that short rows still fill the SM
-  // with several CTAs (shared memory is sized by the longest row).
-  if (a.n_max > kSmemMaxN) return launch_select_nt<1024, true>(a, smem, stream);
-  if (a.n_max > 16384) return launch_select_nt<1024, false>(a, smem, stream);
-  if (a.n_max > 8192) return launch_select_nt<512, false>(a, smem, stream);
-  return launch_select_nt<256, false>(a, smem, stream);
+  SelectPlan p;
+  int mode, nt;
+  size_t smem;
+  plan_select(a, &p, &mode, &nt, &smem);
+  if (mode == kStream) return launch_select_nt<1024, kStream>(a, p, smem, stream);
+  if (mode == kCluster)
+    return nt == 1024 ? launch_select_nt<1024, kCluster>(a, p, smem, stream)
+                      : launch_select_nt<512, kCluster>(a, p, smem, stream);
+  if (nt == 1024) return launch_select_nt<1024, kOne>(a, p, smem, stream);
+  if (nt == 512) return launch_select_nt<512, kOne>(a, p, smem, stream);
+  return launch_select_nt<256, kOne>(a, p, smem, stream);
 }
 
 }  // namespace rolekv

@@ -1,0 +1,100 @@
+"""The selector's routes (one CTA per unit, a cluster of CTAs per unit,
+streaming) give the same kept sets: a batch large enough for one route against
+its layers one at a time, which take another, and sampled units against the
+oracle."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import rolekv_oracle as O
+from paper_2607_13205_gb300 import inputs as I
+from paper_2607_13205_gb300 import rolekv as R
+from tests.gpu_helpers import lib_batch, oracle_batch
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda"
+
+
+def _scores(kind, shape, seed):
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    x = torch.randn(shape, generator=g, device=DEV)
+    if kind == "spread":
+        return torch.exp(1.5 * x)
+    if kind == "tied":                       # a few hundred values: ties at every threshold
+        return torch.exp(torch.round(8 * x) / 16)
+    if kind == "constant":                   # every key equal: ties ranked over all slots and ranks
+        return torch.full(shape, 0.37, device=DEV)
+    if kind == "signs":                      # both signs: the full-pass descent
+        return x
+    x = torch.exp(x)                         # "nan": a few of them
+    x.view(-1)[:: max(1, x.numel() // 7)] = float("nan")
+    return x
+
+
+# (n, layers, policy, pool, budget, floor, scores[, varlen lengths]): the whole
+# batch and one layer of it take different routes (4 KV heads a sequence)
+CASES = [
+    (16385, 10, R.POLICY_ROLE_QUOTA, 7, 0.1, 0, "spread"),
+    (16385, 10, R.POLICY_GLOBAL, 1, 0.3, 64, "tied"),
+    (20003, 10, R.POLICY_SLACK, 7, 0.3, 32, "spread"),
+    (20003, 10, R.POLICY_SLACK, 3, 0.5, 0, "constant"),
+    (24001, 10, R.POLICY_ROLE_QUOTA, 5, 0.2, 0, "signs"),
+    (24001, 10, R.POLICY_FAIR, 1, 0.5, 0, "constant"),
+    (40960, 10, R.POLICY_ROLE_QUOTA, 15, 0.02, 0, "nan"),
+    (40961, 20, R.POLICY_ROLE_QUOTA, 7, 0.1, 0, "tied"),
+    (40961, 20, R.POLICY_SLACK, 7, 0.3, 0, "tied"),
+    (40961, 20, R.POLICY_GLOBAL, 3, 0.1, 16, "constant"),
+    (65537, 20, R.POLICY_FAIR, 7, 0.05, 0, "nan"),
+    (131137, 10, R.POLICY_GLOBAL, 7, 0.1, 64, "spread"),
+    (262144, 10, R.POLICY_ROLE_QUOTA, 7, 0.02, 0, "tied"),
+    (50001, 7, R.POLICY_ROLE_QUOTA, 7, 0.1, 32, "tied", (50001, 3, 0, 17111, 1)),
+    (4096, 40, R.POLICY_ROLE_QUOTA, 7, 0.1, 0, "spread"),
+    (8192, 160, R.POLICY_SLACK, 7, 0.3, 0, "tied"),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=[f"{c[0]}x{c[1]}-p{c[2]}-{c[6]}" for c in CASES])
+def test_routes_agree(case):
+    n, L, policy, pool, B, floor, kind = case[:7]
+    lens = case[7] if len(case) > 7 else None
+    w = I.Workload("routes", "snapkv", L, len(lens) if lens else 1, 8, 4, 64, n, 32, pool, (B,), 4, (3, 5), (1, 3),
+                   seqlens=lens)
+    one = w.scaled(L=1)
+    roles_np = I.workload_roles(w, 3)
+    roles = torch.as_tensor(roles_np, device=DEV)
+    params = R.select_params(B, I.PAPER_ALPHA, alpha_key=0.02, key_role=I.ROLE_KEY, policy=policy, keep_last=floor)
+    whole, layer = lib_batch(w, DEV), lib_batch(one, DEV)
+    scores = _scores(kind, whole.score_shape(), 11)
+
+    def run(batch, sc):
+        idx = torch.full(batch.kept_shape(B), -7, dtype=torch.int32, device=DEV)
+        mask = torch.full(batch.score_shape(), 9, dtype=torch.uint8, device=DEV)
+        per = torch.full((batch.n_units, I.N_ROLES), -1, dtype=torch.int32, device=DEV)
+        status = torch.zeros(1, dtype=torch.int32, device=DEV)
+        R.role_alloc_select(batch, sc, roles, params, idx, pool_k=pool, keep_mask=mask, kept_per_role=per,
+                            status=status)
+        return idx, mask, per, status
+
+    a = run(whole, scores)
+    parts = [run(layer, scores[l:l + 1].contiguous()) for l in range(L)]
+    torch.cuda.synchronize()
+    for x in range(3):
+        assert torch.equal(a[x], torch.cat([p[x] for p in parts], dim=0)), ("idx", "mask", "per_role")[x]
+    assert int(a[3]) == (R.STATUS_NONFINITE if kind == "nan" else 0)
+    if kind == "nan":
+        return                               # (the oracle's NaN rule has its own test)
+    # the first layer's units against the oracle
+    ob = oracle_batch(one)
+    sc = scores[:1].cpu().numpy()
+    us = {u: ob.score_view(sc, u).astype(np.float64) for u in range(ob.n_units)}
+    us = {u: O.maxpool1d(s, pool) if s.size else s for u, s in us.items()}
+    ref = O.select_batch(ob, us, roles_np, I.N_ROLES, I.PAPER_ALPHA, I.ROLE_KEY, 0.02, B, policy, 0, keep_last=floor)
+    cu = ob.kept_offsets(B)
+    got, per = parts[0][0].cpu().numpy(), parts[0][2].cpu().numpy()
+    for u, (idx, counts) in ref.items():
+        _, s, h = ob.unit(u)
+        row = got[0, h, cu[s]:cu[s + 1]] if ob.varlen else got.reshape(ob.n_units, -1)[u]
+        assert np.array_equal(row, idx), f"unit {u}"
+        assert list(per[u]) == counts, f"unit {u} per-role counts"
