@@ -133,6 +133,8 @@ struct Unit {
   int64_t tok0;     // first token of the sequence in the packed token axis
 };
 
+// UNI: called by converged warps, whose loops then run on warp-uniform sizes.
+template <bool UNI = false>
 __device__ __forceinline__ Unit decode_unit(const ScoreArgs& a, int u) {
   Unit r;
   r.h = u % a.Hkv;
@@ -140,8 +142,13 @@ __device__ __forceinline__ Unit decode_unit(const ScoreArgs& a, int u) {
   r.s = ls % a.b;
   r.l = ls / a.b;
   if (a.varlen) {
-    r.tok0 = a.cu_seqlens[r.s];
-    r.n = a.cu_seqlens[r.s + 1] - a.cu_seqlens[r.s];
+    int t0 = a.cu_seqlens[r.s], t1 = a.cu_seqlens[r.s + 1];
+    if constexpr (UNI) {
+      t0 = warp_uniform(t0);
+      t1 = warp_uniform(t1);
+    }
+    r.tok0 = t0;
+    r.n = t1 - t0;
   } else {
     r.tok0 = 0;
     r.n = a.n_max;
@@ -350,7 +357,9 @@ __device__ __forceinline__ void rowstats_tile(const uint32_t* r, int t0, int pos
 // raw logits r, overwritten at the causal edge); (m2, l) as in
 // rowstats_tile.  Keys past the row's own position become -inf, so every
 // slice takes the same branch-free path: the reference moves to the slice's
-// maximum first (three-input max on the ALU), then one packed sum against it.
+// maximum first (three-input max on the ALU), rounded up to a whole number so
+// that moving a sum to another reference is exact, then one packed sum
+// against it.
 template <int NCOL>
 __device__ __forceinline__ void rowstats_slice(uint32_t* r, int t0, int pos, float c1,
                                                float& m2, float& l) {
@@ -361,7 +370,7 @@ __device__ __forceinline__ void rowstats_slice(uint32_t* r, int t0, int pos, flo
     for (int i = 0; i < NCOL; ++i)
       if (i > last) r[i] = 0xFF800000u;          // -inf
   }
-  const float mnew = fmaxf(m2, max_cols<NCOL>(r) * c1);
+  const float mnew = fmaxf(m2, ceilf(max_cols<NCOL>(r) * c1));
   const float s = sum_exp2_shift<NCOL>(r, c1, mnew);
   l = l * fast_exp2(m2 - mnew) + s;
   m2 = mnew;
@@ -538,7 +547,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   using C = Cfg<D, PASS>;
   extern __shared__ uint8_t smem_raw[];
   Shared sh = carve<D, PASS>(smem_raw);
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_uniform(static_cast<int>(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
 
   const Work w = decode_work(a, PASS);
@@ -771,8 +780,8 @@ struct FCfg {
   static constexpr int kOnesOff = kNlOff + kRowsMax * 32;
   static constexpr int kBarOff = kOnesOff + kTileKeys * 32;
   // k_full/k_empty[SK], q_full, q_empty, acc_full[2], acc_empty[2], merge_full,
-  // red_full[2], red_empty[2], drain, pub, lse_go, lse_ready
-  static constexpr int kNumBars = 2 * SK + 15;
+  // red_full[2], red_empty[2], drain, pub, lse_go, lse_ready, join
+  static constexpr int kNumBars = 2 * SK + 16;
   static constexpr int kMiscOff = kBarOff + kNumBars * 8;
   static constexpr int kBytes = kMiscOff + 32;
   static constexpr int kSmemAlloc = kBytes + 1024;
@@ -788,7 +797,7 @@ struct FShared {
   float2* merge;
   uint64_t *k_full, *k_empty, *q_full, *q_empty, *acc_full, *acc_empty;
   uint64_t *merge_full, *red_full, *red_empty, *drain;
-  uint64_t *pub, *lse_go, *lse_ready;
+  uint64_t *pub, *lse_go, *lse_ready, *join;
   uint32_t* tmem_base;
   volatile int* abort_flag;
 };
@@ -825,6 +834,7 @@ __device__ __forceinline__ FShared fcarve(uint8_t* raw) {
   s.pub = b++;
   s.lse_go = b++;
   s.lse_ready = b++;
+  s.join = b++;
   s.tmem_base = reinterpret_cast<uint32_t*>(base + C::kMiscOff);
   s.abort_flag = reinterpret_cast<volatile int*>(base + C::kMiscOff + 4);
   return s;
@@ -861,33 +871,68 @@ __device__ __forceinline__ void chunk_tiles(const ScoreArgs& a, int n, int c, in
   *kt1 = min(ntiles, *kt0 + ct);
 }
 
-// Item `item` of the fused launch.  SnapKV: (unit, chunk of its key tiles).
-// H2O: (unit, query block), the longest blocks first, over the key tiles up
+__device__ __forceinline__ int chunk_cells(int kt0, int kt1) {
+  return (kt1 - kt0 + kCellTiles - 1) / kCellTiles;
+}
+
+// Item `item` of the fused launch.  SnapKV: (unit, chunk of its key tiles),
+// or one of the n_parts parts of a chunk, each a run of whole cells.  H2O: (unit, query block), the longest blocks first, over the key tiles up
 // to the block's last position; its rows' normalisers are its own (no other
 // CTA contributes), so the block needs no cross-CTA exchange.
 struct FItem {
-  int u, chunk, rb, kt0, kt1;
+  int u, chunk, cell0, rb, kt0, kt1;
   Unit un;
 };
 
+template <bool PARTS, bool UNI = false>
 __device__ __forceinline__ FItem fused_item(const ScoreArgs& a, int item) {
   FItem it;
+  it.cell0 = 0;
   if (a.mode == kModeSnapKV) {
-    it.u = item / a.n_chunks;
-    it.chunk = item % a.n_chunks;
+    const int n_parts = PARTS ? a.n_parts : 1;
+    const int gang = a.n_chunks * n_parts;
+    it.u = item / gang;
+    const int x = item % gang;
+    it.chunk = x / n_parts;
     it.rb = 0;
-    it.un = decode_unit(a, it.u);
+    it.un = decode_unit<UNI>(a, it.u);
     chunk_tiles(a, it.un.n, it.chunk, &it.kt0, &it.kt1);
+    if (PARTS) {
+      const int per = (chunk_cells(it.kt0, it.kt1) + n_parts - 1) / n_parts;   // cells of a part
+      it.cell0 = (x % n_parts) * per;
+      it.kt0 = min(it.kt1, it.kt0 + it.cell0 * kCellTiles);
+      it.kt1 = min(it.kt1, it.kt0 + per * kCellTiles);
+    }
   } else {
     it.u = item % a.n_units;
     it.chunk = 0;
     it.rb = a.nrb_max - 1 - item / a.n_units;
-    it.un = decode_unit(a, it.u);
+    it.un = decode_unit<UNI>(a, it.u);
     const int n = it.un.n;
     it.kt0 = 0;
     it.kt1 = (it.rb * a.P < n) ? (min(n, (it.rb + 1) * a.P) + kTileKeys - 1) / kTileKeys : 0;
   }
   return it;
+}
+
+// (max2, sum) pairs of a row's keys: `o`'s joined to (m, l).  The roundings are
+// spelled out, so that the same pairs joined in the same order give the same
+// bits wherever that happens (in registers, or from another CTA's partials).
+__device__ __forceinline__ void join_stats(float& m, float& l, float2 o) {
+  const float mm = fmaxf(m, o.x);
+  if (mm > -INFINITY) {
+    l = __fmaf_rn(l, fast_exp2(m - mm), __fmul_rn(o.y, fast_exp2(o.x - mm)));
+    m = mm;
+  }
+}
+
+// The same over the chunks of a row.
+__device__ __forceinline__ void join_chunk(float& m, float& s, float2 v) {
+  if (v.y > 0.f) {
+    const float mn = fmaxf(m, v.x);
+    s = __fmaf_rn(s, exp2f(m - mn), __fmul_rn(v.y, exp2f(v.x - mn)));
+    m = mn;
+  }
 }
 
 // Descriptor `d` moved `bytes` further into shared memory.  The start-address
@@ -929,7 +974,9 @@ __device__ __forceinline__ void issue_mma_keys_on_lanes(uint64_t dq, uint64_t dk
   }
 }
 
-template <int D>
+// PARTS: the chunks are split over CTAs (small batches); a variant of its own,
+// so that the whole chunks' epilogue keeps its registers.
+template <int D, bool PARTS>
 __global__ void __launch_bounds__(kThreads, 1)
     snapkv_fused_kernel(const __grid_constant__ CUtensorMap k_map,
                         const __grid_constant__ CUtensorMap q_map, const FusedArgs fa) {
@@ -937,7 +984,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const ScoreArgs& a = fa.s;
   extern __shared__ uint8_t smem_raw[];
   FShared sh = fcarve<D>(smem_raw);
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_uniform(static_cast<int>(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
   const int nrt = a.nrows_pad / 128;
 
@@ -959,6 +1006,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(sh.pub, kEpiWarps * 32);
     mbar_init(sh.lse_go, 1);
     mbar_init(sh.lse_ready, kEpiWarps * 32);
+    mbar_init(sh.join, kEpiWarps * 32);
     *sh.abort_flag = 0;
     fence_mbar_init();
   }
@@ -1003,7 +1051,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // unit, so a unit's chunks run on different CTAs in the same round.
       const bool h2o = a.mode == kModeH2O;
       for (int item = blockIdx.x; item < fa.n_items; item += gridDim.x) {
-        const FItem it = fused_item(a, item);
+        const FItem it = fused_item<PARTS>(a, item);
         const Unit& un = it.un;
         const int kt0 = it.kt0, kt1 = it.kt1;
         if (kt1 == kt0) continue;
@@ -1060,7 +1108,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int p2n = a.nrows_pad == 256 ? ((a.nrows + 31) & ~31) : a.nrows_pad;
       const uint32_t idesc_nl = idesc_bf16_f32(128, p2n);
       for (int item = blockIdx.x; item < fa.n_items && ok; item += gridDim.x) {
-        const FItem it = fused_item(a, item);
+        const FItem it = fused_item<PARTS>(a, item);
         const int kt0 = it.kt0, kt1 = it.kt1;
         if (kt1 == kt0) {
           if (a.mode != kModeH2O) ++lpop;          // (the epilogue still forms them)
@@ -1139,9 +1187,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     int pair = 0, xchg = 0;
     bool ok = true;
     int ipop = 0;                                  // items done: barrier phases
+    uint32_t jphase = 0;
     const bool h2o = a.mode == kModeH2O;
     for (int item = blockIdx.x; item < fa.n_items && ok; item += gridDim.x) {
-      const FItem it = fused_item(a, item);
+      const FItem it = fused_item<PARTS, true>(a, item);
       const int u = it.u, chunk = it.chunk, rb = it.rb;
       const Unit& un = it.un;
       const int n = un.n;
@@ -1149,40 +1198,51 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (h2o && kt1 == kt0) continue;           // a block past its sequence's end
 
       if (!fa.single) {
-      // ---- pass 1: running (max2, sum) of this thread's row over its keys
+      // ---- pass 1: (max2, sum) of this thread's row over its keys, cell by
+      // cell (H2O: the block's tiles are one cell).  A chunk's cells are
+      // joined in order, here or, where the chunk is split over CTAs, from
+      // the cells' partials: the same bits either way.
       const int pos = row_position(a, n, rb, row);
+      const int step = h2o ? max(1, kt1 - kt0) : kCellTiles;
       float m2 = -INFINITY, l = 0.f;
-      for (int kt = kt0; kt < kt1; ++kt, ++pair) {
-        const int ab = pair & 1;
-        if (ab != grp) continue;                   // the other group's tile
-        ok = __all_sync(0xffffffffu, mbar_wait(&sh.acc_full[ab], (pair >> 1) & 1, sh.abort_flag, a.status));
-        if (!ok) break;
-        tc_fence_after();
-        uint32_t r[64];
-        for (int h = 0; h < p1cols / 64; ++h) {
-          tmem_load_cols<64>(tmem + lane_base + ab * 256 + col1 + h * 64, r);
-          if (h + 1 == p1cols / 64) {
-            tc_fence_before();
-            mbar_arrive(&sh.acc_empty[ab]);
+      for (int ck = kt0; ck < kt1 && ok; ck += step) {
+        float cm = -INFINITY, cl = 0.f;
+        const int ce = min(kt1, ck + step);
+        for (int kt = ck + grp; kt < ce; kt += 2) {   // (ck - kt0 and pair are even)
+          ok = __all_sync(0xffffffffu, mbar_wait(&sh.acc_full[grp], ((pair + kt - kt0) >> 1) & 1,
+                                                 sh.abort_flag, a.status));
+          if (!ok) break;
+          tc_fence_after();
+          uint32_t r[64];
+          for (int h = 0; h < p1cols / 64; ++h) {
+            tmem_load_cols<64>(tmem + lane_base + grp * 256 + col1 + h * 64, r);
+            if (h + 1 == p1cols / 64) {
+              tc_fence_before();
+              mbar_arrive(&sh.acc_empty[grp]);
+            }
+            rowstats_slice<64>(r, kt * kTileKeys + key1 + h * 64, pos, c1, cm, cl);
           }
-          rowstats_slice<64>(r, kt * kTileKeys + key1 + h * 64, pos, c1, m2, l);
+        }
+        if (!PARTS) {
+          join_stats(m2, l, make_float2(cm, cl));
+        } else {
+          const int64_t cell = (static_cast<int64_t>(u) * a.n_chunks + chunk) * a.cells_max + it.cell0 +
+                               (ck - kt0) / kCellTiles;
+          const int64_t o = cell * (kParts * 128) + sub * (nrt * 128) + row;
+          if (ok && in_bounds(o, 1, a.ext_partials, a.status)) a.partials[o] = make_float2(cm, cl);
         }
       }
+      pair += kt1 - kt0;
       if (!ok) break;
       // merge the key slices of each row, publish the chunk's partials
-      if (sub != 0) {
+      if (PARTS) {
+        __threadfence();                           // (the cells' partials above)
+      } else if (sub != 0) {
         sh.merge[sub * kRowsMax + row] = make_float2(m2, l);
         mbar_arrive(sh.merge_full);
       } else {
         ok = mbar_wait(sh.merge_full, ipop & 1, sh.abort_flag, a.status);
-        for (int x = 1; x < nsub && ok; ++x) {
-          const float2 o = sh.merge[x * kRowsMax + row];
-          const float mm = fmaxf(m2, o.x);
-          if (mm > -INFINITY) {
-            l = l * fast_exp2(m2 - mm) + o.y * fast_exp2(o.x - mm);
-            m2 = mm;
-          }
-        }
+        for (int x = 1; x < nsub && ok; ++x) join_stats(m2, l, sh.merge[x * kRowsMax + row]);
         if (h2o) {
           sh.merge[row] = make_float2(m2, l);      // (slot 0: the leader's own)
         } else {
@@ -1205,7 +1265,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           __threadfence();
           atomicAdd(fa.work + 1 + u, 1);
           const uint64_t t0 = global_timer_ns();
-          while (ld_acquire_gpu(fa.work + 1 + u) < a.n_chunks + fa.hold) {
+          while (ld_acquire_gpu(fa.work + 1 + u) < a.n_chunks * (PARTS ? a.n_parts : 1) + fa.hold) {
             if (*sh.abort_flag || global_timer_ns() - t0 > fa.wait_ns) {
               *sh.abort_flag = 1;
               if (a.status) atomicOr(a.status, ROLEKV_STATUS_TIMEOUT);
@@ -1220,6 +1280,42 @@ __global__ void __launch_bounds__(kThreads, 1)
       ok = __all_sync(0xffffffffu, mbar_wait(sh.lse_go, ipop & 1, sh.abort_flag, a.status));
       if (!ok || *sh.abort_flag) break;
       }  // pass 1
+      // A split chunk's cells joined by all epilogue threads, thread (sub, row)
+      // its slot's cells in order, then the row's slots and the chunks.
+      float jm = -INFINITY, js = 0.f;
+      if (PARTS && !fa.single) {
+        for (int c = 0; c < a.n_chunks && ok; ++c) {
+          int c0, c1t;
+          chunk_tiles(a, n, c, &c0, &c1t);
+          const int cells = chunk_cells(c0, c1t);
+          const int64_t o = (static_cast<int64_t>(u) * a.n_chunks + c) * a.cells_max * (kParts * 128) + etid;
+          float m2 = -INFINITY, l = 0.f;
+          for (int x0 = 0; x0 < cells; x0 += 8) {
+            float2 v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              v[i] = (x0 + i < cells && in_bounds(o + (x0 + i) * (kParts * 128), 1, a.ext_partials, a.status))
+                         ? __ldcg(a.partials + o + (x0 + i) * (kParts * 128))
+                         : make_float2(-INFINITY, 0.f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) join_stats(m2, l, v[i]);
+          }
+          const int jsub = etid / (nrt * 128), jrow = etid % (nrt * 128);
+          sh.merge[jsub * kRowsMax + jrow] = make_float2(m2, l);
+          mbar_arrive(sh.join);
+          ok = __all_sync(0xffffffffu, mbar_wait(sh.join, jphase, sh.abort_flag, a.status));
+          jphase ^= 1;
+          if (ok && etid < nrt * 128) {
+            float2 v = sh.merge[etid];
+            for (int x = 1; x < nsub; ++x) join_stats(v.x, v.y, sh.merge[x * kRowsMax + etid]);
+            join_chunk(jm, js, v);
+          }
+          mbar_arrive(sh.join);                    // (the slots are read)
+          ok = __all_sync(0xffffffffu, mbar_wait(sh.join, jphase, sh.abort_flag, a.status)) && ok;
+          jphase ^= 1;
+        }
+        if (!ok) break;
+      }
       // ---- normalisers of the unit's rows from all chunks' partials (or,
       // with caller-supplied window normalisers, as snapkv_lse_kernel wrote them)
       if (etid < kRowsMax) {
@@ -1242,6 +1338,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         } else if (fa.single) {
           const int64_t o = static_cast<int64_t>(u) * kRowsMax + j;
           nl = (p >= 0 && in_bounds(o, 1, a.ext_lse2, a.status)) ? a.lse2[o] : -INFINITY;
+        } else if (PARTS) {
+          if (p >= 0 && js > 0.f) nl = -(jm + log2f(js));
         } else if (p >= 0) {
           // one online merge over the chunks, eight independent loads in flight
           const float2* part_j = a.partials + static_cast<int64_t>(u) * a.n_chunks * kRowsMax + j;
@@ -1256,13 +1354,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                          ? __ldcg(&part_j[(c0 + i) * kRowsMax])
                          : make_float2(-INFINITY, 0.f);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              if (v[i].y > 0.f) {
-                const float mn = fmaxf(m, v[i].x);
-                s = s * exp2f(m - mn) + v[i].y * exp2f(v[i].x - mn);
-                m = mn;
-              }
-            }
+            for (int i = 0; i < 8; ++i) join_chunk(m, s, v[i]);
           }
           if (s > 0.f) nl = -(m + log2f(s));
         }
@@ -1451,28 +1543,28 @@ cudaError_t launch_attn_pass(int pass, int d, const CUtensorMap& kmap, const CUt
                    : launch_pass<64, kPassColsum>(kmap, qmap, a, grid, stream);
 }
 
-template <int D>
+template <int D, bool PARTS>
 static cudaError_t launch_fused(const CUtensorMap& kmap, const CUtensorMap& qmap,
                                 const FusedArgs& a, cudaStream_t stream) {
   using C = FCfg<D>;
-  cudaError_t e = cudaFuncSetAttribute(snapkv_fused_kernel<D>,
+  cudaError_t e = cudaFuncSetAttribute(snapkv_fused_kernel<D, PARTS>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemAlloc);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, snapkv_fused_kernel<D>, kThreads,
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, snapkv_fused_kernel<D, PARTS>, kThreads,
                                                          C::kSmemAlloc)) != cudaSuccess)
     return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   // One CTA per SM, all resident at once (the per-unit arrival counters are
   // waited on), which the cooperative launch guarantees.  The grid is a
-  // multiple of the chunks per unit so that items dealt round-robin put all
-  // of a unit's chunks in the same round.
-  const int nc = a.s.n_chunks;
+  // multiple of the items per unit so that items dealt round-robin put all
+  // of a unit's items in the same round.
+  const int nc = a.s.n_chunks * a.s.n_parts;
   if (nc < 1 || nc > sms) return cudaErrorInvalidConfiguration;
   // (no more CTAs than items: a small batch does not set up idle CTAs; the
-  // count stays a multiple of the chunks per unit)
+  // count stays a multiple of the items per unit)
   const int items = ((a.n_items + nc - 1) / nc) * nc;
   const int grid = std::min((sms / nc) * nc, std::max(items, nc));
   cudaLaunchConfig_t cfg = {};
@@ -1485,14 +1577,16 @@ static cudaError_t launch_fused(const CUtensorMap& kmap, const CUtensorMap& qmap
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, snapkv_fused_kernel<D>, kmap, qmap, a);
+  e = cudaLaunchKernelEx(&cfg, snapkv_fused_kernel<D, PARTS>, kmap, qmap, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
 cudaError_t launch_snapkv_fused(int d, const CUtensorMap& kmap, const CUtensorMap& qmap,
                                 const FusedArgs& a, cudaStream_t stream) {
-  return d == 128 ? launch_fused<128>(kmap, qmap, a, stream) : launch_fused<64>(kmap, qmap, a, stream);
+  if (a.s.n_parts > 1)
+    return d == 128 ? launch_fused<128, true>(kmap, qmap, a, stream) : launch_fused<64, true>(kmap, qmap, a, stream);
+  return d == 128 ? launch_fused<128, false>(kmap, qmap, a, stream) : launch_fused<64, false>(kmap, qmap, a, stream);
 }
 
 cudaError_t launch_snapkv_lse(const ScoreArgs& a, const float* lse_win, cudaStream_t stream) {

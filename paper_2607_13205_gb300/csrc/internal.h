@@ -16,6 +16,11 @@ enum { kModeSnapKV = 0, kModeH2O = 1 };
 // when it runs out the kernel records ROLEKV_STATUS_TIMEOUT and unwinds.
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
+// Key tiles of a cell, the unit in which a SnapKV chunk's row statistics are
+// joined and, in small batches, split over CTAs.  The statistics of a row are
+// joined cell by cell in both cases, so the scores do not depend on the split.
+constexpr int kCellTiles = 4;
+
 // Everything the two attention passes need, passed by value to the kernels.
 struct ScoreArgs {
   int32_t L, b, G, Hkv, d, n_max;
@@ -32,9 +37,12 @@ struct ScoreArgs {
   int64_t q_layer, q_seq, q_head, q_tok;
   float c1;                         // softmax scale * log2(e)
   int32_t chunk_tiles;              // SnapKV: 128-key tiles per CTA
-  int32_t n_chunks;                 // SnapKV: CTAs per unit
+  int32_t n_chunks;                 // SnapKV: chunks per unit
+  int32_t n_parts;                  // SnapKV, fused: CTAs a chunk is split over (1: none)
+  int32_t cells_max;                // n_parts > 1: cells of the longest chunk
   int32_t nrb_max;                  // H2O: query blocks per unit (largest sequence)
-  float2* partials;                 // SnapKV pass 1: [unit][chunk][256] (max2, sum)
+  float2* partials;                 // SnapKV pass 1: [unit][chunk][256] (max2, sum), or, n_parts
+                                    // > 1, [unit][chunk][cell][512] by epilogue slot and row
   float* lse2;                      // [unit][query block][256] log2-domain normalisers
   float* prepool;                   // score output before pooling
   int32_t* status;

@@ -230,7 +230,7 @@ int64_t score_elems(const BatchInfo& bi) {
 }
 
 int plan_score(int mode, const BatchInfo& bi, int W, bool need_partials, bool need_prepool,
-               ScorePlan* p, bool fused = false) {
+               ScorePlan* p, bool fused = false, bool split = true) {
   ScoreArgs& a = p->a;
   std::memset(&a, 0, sizeof(a));
   p->fused = fused;
@@ -255,6 +255,7 @@ int plan_score(int mode, const BatchInfo& bi, int W, bool need_partials, bool ne
     if (bi.G > 8) return fail(ROLEKV_ERR_UNSUPPORTED, "H2O takes G <= 8 query heads per KV head (G=%d)", bi.G);
     a.P = bi.G <= 4 ? 64 : 32;
   }
+  a.n_parts = 1;
   a.nrows = bi.G * a.P;
   a.nrows_pad = a.nrows <= 128 ? 128 : 256;
   const int ntiles = (bi.n_max + kTileKeys - 1) / kTileKeys;
@@ -272,8 +273,15 @@ int plan_score(int mode, const BatchInfo& bi, int W, bool need_partials, bool ne
     if (a.n_chunks < 1) a.n_chunks = 1;
     p->grid1 = a.n_units * a.n_chunks;
     p->grid2 = p->grid1;
-    p->n_items = a.n_units * a.n_chunks;
     a.nrb_max = 1;
+    // A batch of at most half as many chunks as SMs splits each chunk's cells
+    // over as many CTAs as there are SMs for.
+    a.cells_max = (a.chunk_tiles + kCellTiles - 1) / kCellTiles;
+    if (p->fused && split) {
+      const int64_t parts = num_sms() / (static_cast<int64_t>(a.n_units) * a.n_chunks);
+      a.n_parts = parts < 1 ? 1 : (parts < a.cells_max ? static_cast<int32_t>(parts) : a.cells_max);
+    }
+    p->n_items = a.n_units * a.n_chunks * a.n_parts;
   } else {
     a.nrb_max = (bi.n_max + a.P - 1) / a.P;
     p->grid1 = a.n_units * a.nrb_max;
@@ -283,7 +291,9 @@ int plan_score(int mode, const BatchInfo& bi, int W, bool need_partials, bool ne
   }
   size_t off = 256;   // first 256 bytes reserved
   p->off_partials = off;
-  if (need_partials) off += align256(static_cast<size_t>(a.n_units) * a.n_chunks * kRowsMax * 8);
+  if (need_partials)
+    off += align256(static_cast<size_t>(a.n_units) * a.n_chunks * 8 *
+                    (a.n_parts > 1 ? static_cast<size_t>(a.cells_max) * 2 * kRowsMax : kRowsMax));
   p->off_lse = off;
   if (!(p->fused && mode == kModeH2O))           // the fused H2O keeps its normalisers on chip
     off += align256(static_cast<size_t>(a.n_units) * a.nrb_max * kRowsMax * 4);
@@ -304,6 +314,16 @@ void set_strides(ScoreArgs& a, const rolekv_tensor& k, const rolekv_tensor& q) {
   a.q_seq = q.s_seq;
   a.q_head = q.s_head;
   a.q_tok = q.s_tok;
+}
+
+// The fused SnapKV plan, without the split of its chunks where the caller's
+// workspace only holds that.
+int plan_snapkv(const BatchInfo& bi, int W, bool need_partials, bool need_prepool, size_t ws_bytes,
+                ScorePlan* p) {
+  int rc = plan_score(kModeSnapKV, bi, W, need_partials, need_prepool, p, true);
+  if (rc == ROLEKV_OK && p->a.n_parts > 1 && ws_bytes < p->bytes)
+    rc = plan_score(kModeSnapKV, bi, W, need_partials, need_prepool, p, true, false);
+  return rc;
 }
 
 int bind_workspace(ScorePlan& p, void* ws, size_t ws_bytes) {
@@ -582,7 +602,7 @@ int snapkv_score(const rolekv_batch* batch, rolekv_tensor q_win, rolekv_tensor k
   if (pool_k < 1 || pool_k > 15 || pool_k % 2 == 0)
     return fail(ROLEKV_ERR_UNSUPPORTED, "pool_k=%d must be odd, 1..15", pool_k);
   ScorePlan p;
-  rc = plan_score(kModeSnapKV, bi, W, lse_win == nullptr, scores_prepool == nullptr, &p, true);
+  rc = plan_snapkv(bi, W, lse_win == nullptr, scores_prepool == nullptr, workspace_bytes, &p);
   if (rc) return rc;
   if (bi.T == 0) return ROLEKV_OK;                 // no tokens: nothing to score
   if (scores == nullptr) return fail(ROLEKV_ERR_INVALID_ARG, "scores is NULL");
@@ -928,7 +948,7 @@ int rolekv_compress(const rolekv_batch* batch, rolekv_tensor q_win, rolekv_tenso
   if (pool_k < 1 || pool_k > 15 || pool_k % 2 == 0)
     return fail(ROLEKV_ERR_UNSUPPORTED, "pool_k=%d must be odd, 1..15", pool_k);
   ScorePlan p;
-  rc = plan_score(kModeSnapKV, bi, W, true, true, &p, true);
+  rc = plan_snapkv(bi, W, true, true, workspace_bytes, &p);
   if (rc) return rc;
   SelectArgs sa;
   if ((rc = fill_select(bi, batch, params, &sa))) return rc;
