@@ -1467,6 +1467,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // partials, or taken from a caller-supplied natural-log LSE.
 __global__ void snapkv_lse_kernel(const ScoreArgs a, const float* __restrict__ lse_win) {
   const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  wait_for_previous_kernels();
   if (idx >= static_cast<int64_t>(a.n_units) * kRowsMax) return;
   const int u = static_cast<int>(idx / kRowsMax);
   const int j = static_cast<int>(idx % kRowsMax);
@@ -1546,6 +1547,7 @@ __global__ void __launch_bounds__(kPoolThreads) maxpool_kernel(const ScoreArgs a
                                                                int blocks_per_unit) {
   const int u = blockIdx.x / blocks_per_unit;
   const int g = (blockIdx.x % blocks_per_unit) * kPoolThreads + threadIdx.x;
+  wait_for_previous_kernels();
   const Unit un = decode_unit(a, u);
   const int64_t base = score_base(a, un, u);
   if (!in_bounds(base, un.n, a.ext_scores, a.status)) return;
@@ -1651,8 +1653,7 @@ cudaError_t launch_snapkv_lse(const ScoreArgs& a, const float* lse_win, cudaStre
   if (total == 0) return cudaSuccess;
   const int threads = 256;
   const int blocks = static_cast<int>((total + threads - 1) / threads);
-  snapkv_lse_kernel<<<blocks, threads, 0, stream>>>(a, lse_win);
-  return cudaGetLastError();
+  return launch_early(snapkv_lse_kernel, blocks, threads, 0, stream, 1, a, lse_win);
 }
 
 cudaError_t launch_maxpool(const ScoreArgs& a, const float* in, float* out, int pool_k,
@@ -1661,8 +1662,8 @@ cudaError_t launch_maxpool(const ScoreArgs& a, const float* in, float* out, int 
   const int groups = (a.n_max + 3 + 3) / 4;        // up to three slots before the row
   const int per_unit = (groups + kPoolThreads - 1) / kPoolThreads;
   const int64_t grid = static_cast<int64_t>(per_unit) * a.n_units;
-  maxpool_kernel<<<static_cast<unsigned>(grid), kPoolThreads, 0, stream>>>(a, in, out, pool_k, per_unit);
-  return cudaGetLastError();
+  return launch_early(maxpool_kernel, static_cast<unsigned>(grid), kPoolThreads, 0, stream, 1, a, in, out, pool_k,
+                      per_unit);
 }
 
 }  // namespace rolekv

@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(kThreads) compact_kernel(const CompactArgs a, 
   const int h = u % a.Hkv;
   const int s = (u / a.Hkv) % a.b;
   const int l = u / (a.Hkv * a.b);
+  wait_for_previous_kernels();
   int n;
   int64_t tok0, kbase, K_s;
   if (a.varlen) {
@@ -93,8 +94,7 @@ cudaError_t launch_compact(const CompactArgs& a, cudaStream_t stream) {
   if (a.n_units == 0 || a.K_max == 0) return cudaSuccess;
   const int chunks = (a.K_max + kRowsPerBlock - 1) / kRowsPerBlock;
   const int64_t grid = static_cast<int64_t>(a.n_units) * chunks;
-  compact_kernel<<<static_cast<unsigned>(grid), kThreads, 0, stream>>>(a, chunks);
-  return cudaGetLastError();
+  return launch_early(compact_kernel, static_cast<unsigned>(grid), kThreads, 0, stream, 1, a, chunks);
 }
 
 }  // namespace rolekv

@@ -120,6 +120,16 @@ __global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(const Decod
   const int s = (u / a.Hkv) % a.b;
   const int l = u / (a.Hkv * a.b);
   const int G = a.G;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kStages; ++i) {
+      mbar_init(&full_bar[i], 1);
+      mbar_init(&empty_bar[i], kDecWarps);
+    }
+    abort_flag = 0;
+    fence_mbar_init();
+  }
+  __syncthreads();
+  wait_for_previous_kernels();
   int n;
   int64_t row0;                                     // first cache row of the unit (packed layouts)
   if (a.varlen) {
@@ -157,16 +167,6 @@ __global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(const Decod
     }
   }
 #endif
-
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < kStages; ++i) {
-      mbar_init(&full_bar[i], 1);
-      mbar_init(&empty_bar[i], kDecWarps);
-    }
-    abort_flag = 0;
-    fence_mbar_init();
-  }
-  __syncthreads();
 
   // fragment-layout state: heads 2t, 2t+1 of this lane's rows
   const int g = lane >> 2, t = lane & 3;
@@ -431,6 +431,7 @@ template <int DPL>
 __global__ void __launch_bounds__(256) decode_combine_kernel(const DecodeArgs a) {
   const int64_t wid = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
+  wait_for_previous_kernels();
   if (wid >= static_cast<int64_t>(a.n_units) * a.G) return;
   const int u = static_cast<int>(wid / a.G), g = static_cast<int>(wid % a.G);
   const int h = u % a.Hkv;
@@ -494,23 +495,14 @@ cudaError_t launch_decode_dk(const DecodeArgs& a, const CUtensorMap& kmap, const
   const unsigned grid2 = static_cast<unsigned>((warps2 * 32 + 255) / 256);
   const int smem = KT ? decode_smem_bytes_kt(a.d) : decode_smem_bytes(a.d);
   cudaError_t e;
-  if (grid1 == 0) {                                  // no rows anywhere: the merge writes zeros
-    decode_combine_kernel<DPL><<<grid2, 256, 0, stream>>>(a);
-    return cudaGetLastError();
-  }
-  if (a.G <= 4) {
-    e = cudaFuncSetAttribute(decode_partial_kernel<DPL, 4, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (grid1 > 0) {                                   // (no rows anywhere: the merge writes zeros)
+    auto* partial = a.G <= 4 ? decode_partial_kernel<DPL, 4, KT> : decode_partial_kernel<DPL, 8, KT>;
+    e = cudaFuncSetAttribute(partial, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    decode_partial_kernel<DPL, 4, KT><<<static_cast<unsigned>(grid1), kDecThreads, smem, stream>>>(a, kmap, vmap);
-  } else {
-    e = cudaFuncSetAttribute(decode_partial_kernel<DPL, 8, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = launch_early(partial, static_cast<unsigned>(grid1), kDecThreads, smem, stream, 1, a, kmap, vmap);
     if (e != cudaSuccess) return e;
-    decode_partial_kernel<DPL, 8, KT><<<static_cast<unsigned>(grid1), kDecThreads, smem, stream>>>(a, kmap, vmap);
   }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  decode_combine_kernel<DPL><<<grid2, 256, 0, stream>>>(a);
-  return cudaGetLastError();
+  return launch_early(decode_combine_kernel<DPL>, grid2, 256, 0, stream, 1, a);
 }
 
 cudaError_t launch_decode(const DecodeArgs& a, const CUtensorMap& kmap, const CUtensorMap& vmap,

@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(kThreads, 3) quest_kernel(const QuestArgs a, i
   const int h = u % a.Hkv;
   const int s = (u / a.Hkv) % a.b;
   const int l = u / (a.Hkv * a.b);
+  wait_for_previous_kernels();
   int n;
   int64_t tok0;
   if (a.varlen) {
@@ -192,8 +193,7 @@ cudaError_t launch_quest(const QuestArgs& a, cudaStream_t stream) {
   const int max_pages = (a.n_max + a.page - 1) / a.page;
   const int ctas_per_unit = (max_pages + kPagesPerCta - 1) / kPagesPerCta;
   const int64_t grid = static_cast<int64_t>(a.n_units) * ctas_per_unit;
-  quest_kernel<<<static_cast<unsigned>(grid), kThreads, 0, stream>>>(a, ctas_per_unit);
-  return cudaGetLastError();
+  return launch_early(quest_kernel, static_cast<unsigned>(grid), kThreads, 0, stream, 1, a, ctas_per_unit);
 }
 
 }  // namespace rolekv

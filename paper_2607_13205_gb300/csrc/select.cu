@@ -78,6 +78,7 @@ struct SelectPlan {
   int32_t groups;      // groups (of four slots) a rank's memory holds
   int32_t n_hist;      // buckets with a histogram
   int32_t list_cap;    // candidate-list entries (8 bytes each in streaming mode, else 4)
+  int32_t hist_off;    // byte offset, after keys and keep bits, of
   int32_t hist_ints;   // the two digit-count buffers (and the first-digit sums)
   int32_t region_words;   // pass-1 histograms, then the candidate list
 };
@@ -813,6 +814,14 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
   const int h = u % a.Hkv;
   const int s = (u / a.Hkv) % a.b;
   const int l = u / (a.Hkv * a.b);
+  for (int x = tid; x < p.hist_ints; x += NT)
+    reinterpret_cast<int32_t*>(dyn + p.hist_off)[x] = 0;
+  {
+    uint4* r4 = reinterpret_cast<uint4*>(dyn + p.hist_off + static_cast<size_t>(p.hist_ints) * 4);
+    const int n4 = (p.n_hist << (STREAM ? p.nb : p.nb - 1)) / 4;
+    for (int x = tid; x < n4; x += NT) r4[x] = make_uint4(0u, 0u, 0u, 0u);
+  }
+  wait_for_previous_kernels();
   int n;
   int64_t tok0;
   if (a.varlen) {
@@ -851,7 +860,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
   uint4* keys4 = reinterpret_cast<uint4*>(dyn);
   const uint32_t* keys = reinterpret_cast<const uint32_t*>(keys4);
   uint32_t* bits = reinterpret_cast<uint32_t*>(dyn + (STREAM ? 0 : static_cast<size_t>(p.groups) * 16));
-  int32_t* hist = reinterpret_cast<int32_t*>(bits + p.groups / 8);   // 16-byte aligned (groups % 32 == 0)
+  int32_t* hist = reinterpret_cast<int32_t*>(dyn + p.hist_off);
   uint32_t* region = reinterpret_cast<uint32_t*>(hist + p.hist_ints);
   uint32_t* hist16 = region;                    // pass 1 histograms
   uint32_t* list = region;                      // then the candidate list
@@ -889,13 +898,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
     S.elig_mask = 0u;
     S.sfast = 0;
   }
-  for (int x = tid; x < p.hist_ints; x += NT) hist[x] = 0;
-  {
-    uint4* r4 = reinterpret_cast<uint4*>(region);
-    const int n4 = (p.n_hist << (STREAM ? nb : nb - 1)) / 4;
-    for (int x = tid; x < n4; x += NT) r4[x] = make_uint4(0u, 0u, 0u, 0u);
-  }
-
   // ---- offset of this unit's kept row (warp 0)
   if (warp == 0) {
     int64_t off_kept = static_cast<int64_t>(u) * a.K_dense;
@@ -1745,21 +1747,8 @@ cudaError_t launch_select_nt(const SelectArgs& a, const SelectPlan& p, size_t sm
   cudaError_t e = cudaFuncSetAttribute(select_kernel<NT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(a.n_units) * p.ranks);
-  cfg.blockDim = dim3(NT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned>(p.ranks);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = MODE == kCluster ? 1 : 0;
-  e = cudaLaunchKernelEx(&cfg, select_kernel<NT, MODE>, a, p);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return launch_early(select_kernel<NT, MODE>, static_cast<unsigned>(a.n_units) * p.ranks, NT, smem, stream,
+                      static_cast<unsigned>(p.ranks), a, p);
 }
 
 // Route, ranks and threads of a unit, by the row length and the number of
@@ -1805,8 +1794,10 @@ void plan_select(const SelectArgs& a, SelectPlan* p, int* mode, int* nt, size_t*
   p->region_words = p->n_hist << (stream ? p->nb : p->nb - 1);
   const int list_words = stream ? 2 * p->list_cap : p->list_cap;
   if (p->region_words < list_words) p->region_words = list_words;
-  *smem = (stream ? 0 : static_cast<size_t>(p->groups) * 16) + p->groups / 8 * 4 +
-          static_cast<size_t>(p->hist_ints) * 4 + static_cast<size_t>(p->region_words) * 4;
+  // (16-byte aligned: groups is a multiple of 32)
+  p->hist_off = (stream ? 0 : p->groups * 16) + p->groups / 8 * 4;
+  *smem = static_cast<size_t>(p->hist_off) + static_cast<size_t>(p->hist_ints) * 4 +
+          static_cast<size_t>(p->region_words) * 4;
 }
 
 }  // namespace
