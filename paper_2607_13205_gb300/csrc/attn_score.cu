@@ -773,12 +773,14 @@ struct FCfg {
   static constexpr int kQOff = 0;
   static constexpr int kKOff = kQOff + kQSlotBytes;
   static constexpr int kPosOff = kKOff + SK * kKTileBytes;
-  static constexpr int kRedOff = kPosOff + kRowsMax * 4;
+  // positions and (below) normalisers twice, by item parity: with supplied
+  // normalisers a thread may form the next item's while others still read
+  static constexpr int kRedOff = kPosOff + 2 * kRowsMax * 4;
   static constexpr int kMergeOff = kRedOff + (kParts - 1) * kTileKeys * 4;
   // the extra pass-2 k-step: row normalisers (256 rows) against ones (128
   // keys), 16 bf16 columns each, K-major without swizzle
   static constexpr int kNlOff = kMergeOff + kParts * kRowsMax * 8;
-  static constexpr int kOnesOff = kNlOff + kRowsMax * 32;
+  static constexpr int kOnesOff = kNlOff + 2 * kRowsMax * 32;
   static constexpr int kBarOff = kOnesOff + kTileKeys * 32;
   // k_full/k_empty[SK], q_full, q_empty, acc_full[2], acc_empty[2], merge_full,
   // red_full[2], red_empty[2], drain, pub, lse_go, lse_ready, join
@@ -791,7 +793,7 @@ struct FCfg {
 struct FShared {
   uint8_t* q;
   uint8_t* k;
-  uint8_t* nlb;      // [256 rows][16] bf16: -lse2_j / c1 in three parts, then zeros
+  uint8_t* nlb;      // [2][256 rows][16] bf16: -lse2_j / c1 in three parts, then zeros
   uint8_t* ones;     // [128 keys][16] bf16: 1, 1, 1, then zeros
   int32_t* pos;
   float* red;
@@ -1025,7 +1027,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int r = i >> 4, kk = i & 15;
     reinterpret_cast<uint16_t*>(sh.ones)[nl_elem(r, kk)] = kk < 3 ? 0x3F80u : 0u;   // bf16 1.0
   }
-  for (int i = threadIdx.x; i < kRowsMax * 8; i += kThreads) reinterpret_cast<uint32_t*>(sh.nlb)[i] = 0u;
+  for (int i = threadIdx.x; i < 2 * kRowsMax * 8; i += kThreads) reinterpret_cast<uint32_t*>(sh.nlb)[i] = 0u;
   fence_proxy_async_smem();
   if (warp == kMmaWarp) {
     tmem_alloc(sh.tmem_base, kTmemCols);
@@ -1104,7 +1106,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int lpop = 0;                                // items whose normalisers the epilogue forms
       bool ok = true;
       const uint64_t ones_desc = sdesc_kmajor_noswizzle(smem_u32(sh.ones), 128, 256);
-      const uint64_t nl_desc = sdesc_kmajor_noswizzle(smem_u32(sh.nlb), 128, 256);
+      const uint64_t nl_desc0 = sdesc_kmajor_noswizzle(smem_u32(sh.nlb), 128, 256);
       // pass 2 spans only the rows that exist, rounded up to 32 (224 of 256 at G = 7)
       const int p2n = a.nrows_pad == 256 ? ((a.nrows + 31) & ~31) : a.nrows_pad;
       const uint32_t idesc_nl = idesc_bf16_f32(128, p2n);
@@ -1142,7 +1144,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 nl_ready = true;
               }
-              mma_bf16_ss(tmem + ab * 256, ones_desc, nl_desc, idesc_nl, 1u);
+              mma_bf16_ss(tmem + ab * 256, ones_desc, desc_plus(nl_desc0, (lpop & 1) * kRowsMax * 32), idesc_nl, 1u);
             }
             mma_commit(&sh.acc_full[ab]);
             mma_commit(&sh.k_empty[kslot]);
@@ -1359,7 +1361,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           if (s > 0.f) nl = -(m + log2f(s));
         }
-        sh.pos[j] = p;
+        sh.pos[(ipop & 1) * kRowsMax + j] = p;
         // -lse2_j / c1 as the sum of three bf16 parts (exact to ~2^-24); a row
         // without keys gets -1e30, whose exponential is 0
         const float x = nl > -INFINITY ? nl / c1 : -1.0e30f;
@@ -1367,7 +1369,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float r1 = x - bf16_value(h0);
         const uint16_t h1 = bf16_bits_rn(r1);
         const uint16_t h2 = bf16_bits_rn(r1 - bf16_value(h1));
-        uint16_t* nlr = reinterpret_cast<uint16_t*>(sh.nlb);
+        uint16_t* nlr = reinterpret_cast<uint16_t*>(sh.nlb + (ipop & 1) * kRowsMax * 32);
         nlr[nl_elem(j, 0)] = h0;
         nlr[nl_elem(j, 1)] = h1;
         nlr[nl_elem(j, 2)] = h2;
@@ -1416,7 +1418,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               const float2 s2 = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
               colsum += s2.x + s2.y;
             } else {
-              const int32_t* pp = sh.pos + j0 + h * NC;
+              const int32_t* pp = sh.pos + (ipop & 1) * kRowsMax + j0 + h * NC;
               float s = 0.f;
 #pragma unroll
               for (int i = 0; i < NC; ++i) {
