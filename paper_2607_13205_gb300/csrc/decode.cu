@@ -4,7 +4,7 @@
 //   o_g = sum_j softmax_j(scale q_g . k_j) v_j
 // over the unit's cache rows (the kept slots; -1 slots of an infeasible budget
 // are skipped; with budget 1 and no index the full cache).  Memory-bound: the
-// cache rows are read once.  Split-K: CTA (unit, split) takes up to 1024 rows
+// cache rows are read once.  Split-K: CTA (unit, split) takes a run of rows
 // (a unit's splits equal in length).  A producer warp streams them into two
 // shared-memory stages of 64 K rows and 64 V rows.  K goes through a tensor
 // map, one copy per 64-column half of a stage, 128-byte swizzled so that the
@@ -62,6 +62,8 @@ constexpr int kStages = 2;         // shared-memory stages of cache rows
 constexpr int kTileRows = 16;      // rows of one MMA tile (one consumer warp)
 constexpr int kStageRows = kDecWarps * kTileRows;
 constexpr int kDecThreads = (kDecWarps + 1) * 32;   // + one producer warp
+constexpr int kMergeWarps = 4;     // warps of a merging CTA
+constexpr int kMergeSplits = 4;    // most splits one of them merges alone
 
 // K rows sit 16 bytes apart beyond their length, so that the eight rows read
 // by one fragment load fall in different banks; V rows are packed.
@@ -426,13 +428,20 @@ __global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(const Decod
   }
 }
 
-// Merge of the splits of each (unit, query head): one warp, lanes over dims.
-template <int DPL>
-__global__ void __launch_bounds__(256) decode_combine_kernel(const DecodeArgs a) {
-  const int64_t wid = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
+// Merge of the splits of each (unit, query head): a warp finds the reference
+// over all splits (a lane a split), then sums the weighted splits, the lanes
+// over the dimensions.  The loads of the splits do not depend on one another
+// (a warp that walked the splits with a test on each waited for every one: 64
+// splits took 20 us).  SHARE: the four warps of a CTA take every fourth split
+// of one head (more than kMergeSplits of them); otherwise a head each.
+template <int DPL, bool SHARE>
+__global__ void __launch_bounds__(kMergeWarps * 32) decode_combine_kernel(const DecodeArgs a) {
+  constexpr int D = DPL * 32;
+  __shared__ float part[kMergeWarps][D + 1];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   wait_for_previous_kernels();
-  if (wid >= static_cast<int64_t>(a.n_units) * a.G) return;
+  const int64_t wid = SHARE ? blockIdx.x : static_cast<int64_t>(blockIdx.x) * kMergeWarps + warp;
+  if (wid >= static_cast<int64_t>(a.n_units) * a.G) return;   // (whole warps, and only without SHARE)
   const int u = static_cast<int>(wid / a.G), g = static_cast<int>(wid % a.G);
   const int h = u % a.Hkv;
   const int s = (u / a.Hkv) % a.b;
@@ -447,24 +456,51 @@ __global__ void __launch_bounds__(256) decode_combine_kernel(const DecodeArgs a)
       !in_bounds(dst0, a.d, a.ext_out, a.status))
     return;                                          // (checked build only)
   float M = -INFINITY;
-  for (int x = 0; x < ns; ++x) M = fmaxf(M, base[x * stride + a.d]);
-  float L = 0.f, o[DPL];
+  for (int x = lane; x < ns; x += 32) M = fmaxf(M, base[x * stride + a.d]);
 #pragma unroll
-  for (int i = 0; i < DPL; ++i) o[i] = 0.f;
+  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  float L = 0.f;
+  float2 acc[DPL / 2];
+#pragma unroll
+  for (int i = 0; i < DPL / 2; ++i) acc[i] = make_float2(0.f, 0.f);
   if (M > -INFINITY) {
-    for (int x = 0; x < ns; ++x) {
+#pragma unroll 4
+    for (int x = SHARE ? warp : 0; x < ns; x += SHARE ? kMergeWarps : 1) {
       const float* p = base + x * stride;
-      const float mxs = p[a.d];
-      if (mxs == -INFINITY) continue;
-      const float w = exp2f(mxs - M);
+      const float w = exp2f(p[a.d] - M);             // (0 for a split without valid rows)
       L += w * p[a.d + 1];
 #pragma unroll
-      for (int i = 0; i < DPL; ++i) o[i] += w * p[lane * DPL + i];
+      for (int i = 0; i < DPL / 2; ++i) {
+        const float2 v = *reinterpret_cast<const float2*>(p + lane * DPL + 2 * i);
+        acc[i].x += w * v.x;
+        acc[i].y += w * v.y;
+      }
     }
   }
-  float* dst = a.out + l * a.o_layer + s * a.o_seq + static_cast<int64_t>(h * a.G + g) * a.o_head + lane * DPL;
+  if constexpr (!SHARE) {
 #pragma unroll
-  for (int i = 0; i < DPL; ++i) dst[i] = L > 0.f ? o[i] / L : 0.f;
+    for (int i = 0; i < DPL / 2; ++i) {
+      a.out[dst0 + lane * DPL + 2 * i] = L > 0.f ? acc[i].x / L : 0.f;
+      a.out[dst0 + lane * DPL + 2 * i + 1] = L > 0.f ? acc[i].y / L : 0.f;
+    }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < DPL / 2; ++i) {
+    part[warp][lane * DPL + 2 * i] = acc[i].x;
+    part[warp][lane * DPL + 2 * i + 1] = acc[i].y;
+  }
+  if (lane == 0) part[warp][D] = L;
+  __syncthreads();
+  L = 0.f;
+#pragma unroll
+  for (int w = 0; w < kMergeWarps; ++w) L += part[w][D];
+  for (int i = threadIdx.x; i < D; i += kMergeWarps * 32) {
+    float o = 0.f;
+#pragma unroll
+    for (int w = 0; w < kMergeWarps; ++w) o += part[w][i];
+    a.out[dst0 + i] = L > 0.f ? o / L : 0.f;
+  }
 }
 
 // Diagnostic: the bounded mbarrier wait of the kernels above, on a phase that
@@ -491,8 +527,7 @@ template <int DPL, bool KT>
 cudaError_t launch_decode_dk(const DecodeArgs& a, const CUtensorMap& kmap, const CUtensorMap& vmap,
                              cudaStream_t stream) {
   const int64_t grid1 = static_cast<int64_t>(a.n_units) * a.n_splits;
-  const int64_t warps2 = static_cast<int64_t>(a.n_units) * a.G;
-  const unsigned grid2 = static_cast<unsigned>((warps2 * 32 + 255) / 256);
+  const unsigned heads = static_cast<unsigned>(a.n_units) * a.G;
   const int smem = KT ? decode_smem_bytes_kt(a.d) : decode_smem_bytes(a.d);
   cudaError_t e;
   if (grid1 > 0) {                                   // (no rows anywhere: the merge writes zeros)
@@ -502,7 +537,10 @@ cudaError_t launch_decode_dk(const DecodeArgs& a, const CUtensorMap& kmap, const
     e = launch_early(partial, static_cast<unsigned>(grid1), kDecThreads, smem, stream, 1, a, kmap, vmap);
     if (e != cudaSuccess) return e;
   }
-  return launch_early(decode_combine_kernel<DPL>, grid2, 256, 0, stream, 1, a);
+  if (a.n_splits > kMergeSplits)
+    return launch_early(decode_combine_kernel<DPL, true>, heads, kMergeWarps * 32, 0, stream, 1, a);
+  return launch_early(decode_combine_kernel<DPL, false>, (heads + kMergeWarps - 1) / kMergeWarps, kMergeWarps * 32, 0,
+                      stream, 1, a);
 }
 
 cudaError_t launch_decode(const DecodeArgs& a, const CUtensorMap& kmap, const CUtensorMap& vmap,

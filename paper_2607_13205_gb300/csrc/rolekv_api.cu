@@ -762,13 +762,37 @@ int role_alloc_select(const rolekv_batch* batch, const float* scores, const uint
 
 namespace {
 constexpr int kDecodeRowsPerSplit = 1024;
+constexpr int kDecodeSplitCost = 320;       // rows a CTA could stream while one starts and ends
 
-// Splits of at most kDecodeRowsPerSplit rows, equal in length and a multiple
-// of the kernel's 64-row stage, so that a unit's splits finish together.
-void decode_split(int64_t m_max, int32_t* rows_per_split, int32_t* n_splits) {
+// Splits of a unit's rows: equal in length, a multiple of the kernel's 64-row
+// stage, so that a unit's splits finish together.  fine: as long as makes the
+// fewest rows pass one after another through an SM's CTAs (whole waves of
+// CTAs, and their starts); otherwise about kDecodeRowsPerSplit rows, which
+// they never pass (a warp's sums would get longer, their error larger).  8
+// units x 819 rows: 16.2 us in one split each, 6.7 us in seven; 32 x 3277 rows
+// 17.5 and 12.5 us; 8 x 131072 163 and 100 us.  Of start costs 40 to 320 rows
+// the last is best where the splits differ (256 x 820 rows 25.4 us, 26.4 at 80).
+void decode_split(const BatchInfo& bi, int64_t m_max, int64_t total, bool fine, int32_t* rows_per_split,
+                  int32_t* n_splits) {
   const int64_t ns = m_max > 0 ? (m_max + kDecodeRowsPerSplit - 1) / kDecodeRowsPerSplit : 1;
   int64_t r = (m_max + ns - 1) / ns;
   r = r > 0 ? (r + 63) / 64 * 64 : 64;
+  if (fine) {
+    // CTAs resident at once: limited by their two stages of shared memory
+    const int64_t slots = static_cast<int64_t>(num_sms()) * (bi.d == 128 ? 3 : 6);
+    const int64_t heads = static_cast<int64_t>(bi.L) * bi.Hkv;
+    int64_t best = INT64_MAX;
+    for (int64_t x = 128; x <= kDecodeRowsPerSplit; x += 64) {
+      // (packed batches: half a split more per sequence on average)
+      const int64_t ctas = bi.varlen ? heads * (total / x + (bi.b + 1) / 2) : heads * bi.b * ((m_max + x - 1) / x);
+      const int64_t cost = (ctas + slots - 1) / slots * (x + kDecodeSplitCost);
+      if (cost <= best) {
+        best = cost;
+        r = x;
+      }
+      if (x >= m_max) break;
+    }
+  }
   *rows_per_split = static_cast<int32_t>(r);
   *n_splits = static_cast<int32_t>((m_max + r - 1) / r);
 }
@@ -790,9 +814,9 @@ void decode_rows(const BatchInfo& bi, const rolekv_batch* bt, int64_t bfx, int64
   }
 }
 
-size_t decode_ws_bytes(const BatchInfo& bi, int64_t m_max) {
+size_t decode_ws_bytes(const BatchInfo& bi, int64_t m_max, int64_t total, bool fine) {
   int32_t rps, splits;
-  decode_split(m_max, &rps, &splits);
+  decode_split(bi, m_max, total, fine, &rps, &splits);
   return static_cast<size_t>(bi.n_units) * static_cast<size_t>(splits > 0 ? splits : 1) * bi.G *
          (bi.d + 2) * sizeof(float);
 }
@@ -807,7 +831,7 @@ int rolekv_decode_workspace_size(const rolekv_batch* batch, float budget, size_t
     return fail(ROLEKV_ERR_INVALID_ARG, "budget %g outside (0, 1]", static_cast<double>(budget));
   int64_t m_max, total;
   decode_rows(bi, batch, to_fixed(budget), &m_max, &total);
-  *bytes = decode_ws_bytes(bi, m_max);
+  *bytes = decode_ws_bytes(bi, m_max, total, true);
   return ROLEKV_OK;
 }
 
@@ -836,7 +860,9 @@ int decode_attention(const rolekv_batch* batch, rolekv_tensor q, rolekv_tensor k
     if ((rc = check_tensor("k_cache", k_cache, bi.d, bi.Hkv, bi.varlen, false))) return rc;
     if ((rc = check_tensor("v_cache", v_cache, bi.d, bi.Hkv, bi.varlen, false))) return rc;
   }
-  const size_t need = decode_ws_bytes(bi, m_max);
+  // (a workspace that only holds the coarse splits' partials is used with them)
+  const bool fine = workspace_bytes >= decode_ws_bytes(bi, m_max, total, true);
+  const size_t need = decode_ws_bytes(bi, m_max, total, fine);
   if (workspace == nullptr || workspace_bytes < need)
     return fail(ROLEKV_ERR_WORKSPACE, "workspace of %zu bytes, %zu needed", workspace_bytes, need);
   if (reinterpret_cast<uintptr_t>(workspace) & 255u)
@@ -872,7 +898,7 @@ int decode_attention(const rolekv_batch* batch, rolekv_tensor q, rolekv_tensor k
   a.v_tok = v_cache.s_tok;
   a.keep_idx = keep_idx;
   a.c1 = (scale > 0.f ? scale : 1.0f / std::sqrt(static_cast<float>(bi.d))) * 1.4426950408889634f;
-  decode_split(m_max, &a.rows_per_split, &a.n_splits);
+  decode_split(bi, m_max, total, fine, &a.rows_per_split, &a.n_splits);
   a.part = static_cast<float*>(workspace);
   a.out = out;
   a.o_seq = static_cast<int64_t>(bi.Hq) * bi.d;
