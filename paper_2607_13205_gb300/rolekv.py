@@ -55,6 +55,11 @@ class SelectParams(ctypes.Structure):
 
 _lib = None
 
+# The handle of a device's current stream.  torch.cuda.current_stream() makes a
+# Stream object around it first.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+    lambda device: torch.cuda.current_stream(device).cuda_stream)
+
 # (name, restype, argtypes) of every exported function
 _SIGNATURES = [
     ("rolekv_kept_count", ctypes.c_int64, [ctypes.c_int64, ctypes.c_float]),
@@ -128,12 +133,14 @@ def _check(rc: int):
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    # the current stream's handle without a Stream object (3.0 us of a call's 23)
+    return _raw_stream(torch.cuda.current_device())
 
 
 # ---------------------------------------------------------------- descriptors
@@ -190,16 +197,17 @@ def tensor_desc(t: torch.Tensor, packed: bool = False) -> Tensor:
     tensor, as a rolekv_tensor."""
     if t.dtype != torch.bfloat16:
         raise TypeError("rolekv tensors are bf16")
-    if t.stride(-1) != 1:
+    stride = t.stride()
+    if stride[-1] != 1:
         raise ValueError("the head-dim axis must be contiguous")
     if packed:
-        if t.dim() != 4:
+        if len(stride) != 4:
             raise ValueError("packed tensors are [L][T][H][d]")
-        sl, st, sh, _ = t.stride()
+        sl, st, sh, _ = stride
         return Tensor(t.data_ptr(), sl, 0, sh, st)
-    if t.dim() != 5:
+    if len(stride) != 5:
         raise ValueError("dense tensors are [L][b][H][n][d]")
-    sl, ss, sh, st, _ = t.stride()
+    sl, ss, sh, st, _ = stride
     return Tensor(t.data_ptr(), sl, ss, sh, st)
 
 
