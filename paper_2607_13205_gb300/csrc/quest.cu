@@ -6,8 +6,8 @@
 // runs on it unchanged.  One CTA per (layer, sequence, KV head): the mean of
 // the G x W_eff window rows goes to shared memory, then each warp takes whole
 // pages, streaming their key rows with 16-byte read-only loads (the kernel is
-// bound by reading K once from HBM).  A unit's pages are split over CTAs of
-// 256 pages, each of which forms the window mean itself (the window rows are
+// bound by reading K once from HBM).  A unit's pages are split evenly over
+// CTAs, each of which forms the window mean itself (the window rows are
 // read from L2 after the first); the page minima and maxima stay packed
 // bf16 pairs until the dot product.
 #include <cuda_runtime.h>
@@ -23,7 +23,8 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kInFlight = 8;        // key-row loads a lane issues before using them
-constexpr int kPagesPerCta = 256;   // pages of one unit handled by one CTA
+constexpr int kCtasPerSm = 3;
+constexpr int kStartTokens = 250;   // keys a CTA could stream while one forms its window mean
 
 __device__ __forceinline__ uint4 load_nc(const uint4* p) {
   uint4 v;
@@ -49,7 +50,8 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 
-__global__ void __launch_bounds__(kThreads, 3) quest_kernel(const QuestArgs a, int ctas_per_unit) {
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) quest_kernel(const QuestArgs a, int ctas_per_unit,
+                                                                     int pages_per_cta) {
   __shared__ float qpart[kThreads / 8][8 * 8 + 1];   // [row group][dims of a 16-byte chunk ...]
   __shared__ float qbar[128];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -69,9 +71,9 @@ __global__ void __launch_bounds__(kThreads, 3) quest_kernel(const QuestArgs a, i
     n = a.n_max;
   }
   const int npages = (n + a.page - 1) / a.page;
-  const int p_begin = part * kPagesPerCta;
+  const int p_begin = part * pages_per_cta;
   if (p_begin >= npages) return;                   // (uniform)
-  const int p_end = npages - p_begin < kPagesPerCta ? npages : p_begin + kPagesPerCta;
+  const int p_end = npages - p_begin < pages_per_cta ? npages : p_begin + pages_per_cta;
   const int d = a.d;
   const int CR = d / 8;                            // 16-byte chunks per row
 #ifdef ROLEKV_CHECKED
@@ -98,16 +100,24 @@ __global__ void __launch_bounds__(kThreads, 3) quest_kernel(const QuestArgs a, i
     const int RG = kThreads / CR;
     const int c = tid % CR, rg = tid / CR;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int r = rg; r < rows; r += RG) {
-      const int g = r / w_eff, i = r % w_eff;
-      const int64_t o = l * a.q_layer + s * a.q_seq + static_cast<int64_t>(h * a.G + g) * a.q_head +
-                        i * a.q_tok;
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(a.q + o) + c);
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    const uint16_t* q0 = a.q + l * a.q_layer + s * a.q_seq + static_cast<int64_t>(h) * a.G * a.q_head;
+    for (int r = rg; r < rows; r += RG * kInFlight) {
+      uint4 v[kInFlight];                          // (the rows' loads in flight, added in order)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        acc[2 * j] += bf16_lo(w[j]);
-        acc[2 * j + 1] += bf16_hi(w[j]);
+      for (int x = 0; x < kInFlight; ++x) {
+        const int rr = r + x * RG;
+        if (rr < rows)
+          v[x] = __ldg(reinterpret_cast<const uint4*>(q0 + rr / w_eff * a.q_head + rr % w_eff * a.q_tok) + c);
+      }
+#pragma unroll
+      for (int x = 0; x < kInFlight; ++x) {
+        if (r + x * RG >= rows) continue;
+        const uint32_t w[4] = {v[x].x, v[x].y, v[x].z, v[x].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          acc[2 * j] += bf16_lo(w[j]);
+          acc[2 * j + 1] += bf16_hi(w[j]);
+        }
       }
     }
     // qpart[rg][c*8 + j] holds row group rg's sum of dim c*8 + j (d <= 128:
@@ -188,12 +198,35 @@ __global__ void __launch_bounds__(kThreads, 3) quest_kernel(const QuestArgs a, i
 
 }  // namespace
 
+// CTAs per unit: the number for which the fewest keys pass one after another
+// through a CTA slot of the SMs, counting whole waves of CTAs and each one's
+// start.  64 units of 2048 pages: 8 CTAs a unit are 1.12 waves (116 us), 7
+// just under one (84 us, 81 at the copy rate); 8 units of 512 pages 35.6 us
+// with two CTAs a unit, 8.3 us with 52.  Start costs of 100 to 600 keys differ
+// by 2% where they differ (1024 units of 2048 keys: 10% more at 100).
 cudaError_t launch_quest(const QuestArgs& a, cudaStream_t stream) {
   if (a.n_units == 0 || a.n_max == 0) return cudaSuccess;
-  const int max_pages = (a.n_max + a.page - 1) / a.page;
-  const int ctas_per_unit = (max_pages + kPagesPerCta - 1) / kPagesPerCta;
-  const int64_t grid = static_cast<int64_t>(a.n_units) * ctas_per_unit;
-  return launch_early(quest_kernel, static_cast<unsigned>(grid), kThreads, 0, stream, 1, a, ctas_per_unit);
+  int dev = 0, sms = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const int64_t slots = static_cast<int64_t>(sms) * kCtasPerSm;
+  const int64_t pages = (a.n_max + a.page - 1) / a.page;
+  int64_t best = INT64_MAX, ctas = 1;
+  for (int64_t waves = (a.n_units + slots - 1) / slots, i = 0; i < 12; ++waves, ++i) {
+    int64_t c = waves * slots / a.n_units;
+    c = c < 1 ? 1 : (c < pages ? c : pages);
+    const int64_t per = (pages + c - 1) / c;
+    const int64_t cost = waves * (per * a.page + kStartTokens);
+    if (cost < best) {
+      best = cost;
+      ctas = (pages + per - 1) / per;
+    }
+    if (c == pages) break;
+  }
+  const int64_t per = (pages + ctas - 1) / ctas;
+  return launch_early(quest_kernel, static_cast<unsigned>(a.n_units * ctas), kThreads, 0, stream, 1, a,
+                      static_cast<int>(ctas), static_cast<int>(per));
 }
 
 }  // namespace rolekv
