@@ -1239,7 +1239,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) break;
       // merge the key slices of each row, publish the chunk's partials
       if (PARTS) {
-        __threadfence();                           // (the cells' partials above)
+        // (the cells' partials are out)
       } else if (sub != 0) {
         sh.merge[sub * kRowsMax + row] = make_float2(m2, l);
         mbar_arrive(sh.merge_full);
@@ -1254,17 +1254,18 @@ __global__ void __launch_bounds__(kThreads, 1)
             a.partials[slot * kRowsMax + row] = make_float2(m2, l);
           if (nrt == 1 && in_bounds(slot * kRowsMax + 128 + row, 1, a.ext_partials, a.status))
             a.partials[slot * kRowsMax + 128 + row] = make_float2(-INFINITY, 0.f);
-          __threadfence();
         }
       }
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       mbar_arrive(sh.pub);
-      if (etid == 0) {
+      if (warp == 0) {
         // every row of this chunk is visible: count it, then wait for the
-        // unit's other chunks (bounded)
-        bool got = mbar_wait(sh.pub, ipop & 1, sh.abort_flag, a.status);
-        if (got && !h2o) {
+        // unit's other chunks (bounded).  The whole warp stays together: lanes
+        // already waiting for lse_go would hold up the polling one.  One fence,
+        // after the barrier, releases all the threads' partials.
+        bool got = __all_sync(0xffffffffu, mbar_wait(sh.pub, ipop & 1, sh.abort_flag, a.status));
+        if (got && !h2o && lane == 0) {
           __threadfence();
           atomicAdd(fa.work + 1 + u, 1);
           const uint64_t t0 = global_timer_ns();
@@ -1272,13 +1273,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (*sh.abort_flag || global_timer_ns() - t0 > fa.wait_ns) {
               *sh.abort_flag = 1;
               if (a.status) atomicOr(a.status, ROLEKV_STATUS_TIMEOUT);
-              got = false;
               break;
             }
-            __nanosleep(128);
+            __nanosleep(20);
           }
         }
-        mbar_arrive(sh.lse_go);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sh.lse_go);
       }
       ok = __all_sync(0xffffffffu, mbar_wait(sh.lse_go, ipop & 1, sh.abort_flag, a.status));
       if (!ok || *sh.abort_flag) break;
@@ -1293,29 +1294,28 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int cells = chunk_cells(c0, c1t);
           const int64_t o = (static_cast<int64_t>(u) * a.n_chunks + c) * a.cells_max * (kParts * 128) + etid;
           float m2 = -INFINITY, l = 0.f;
-          for (int x0 = 0; x0 < cells; x0 += 8) {
-            float2 v[8];
+          for (int x0 = 0; x0 < cells; x0 += 16) {
+            float2 v[16];
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int i = 0; i < 16; ++i)
               v[i] = (x0 + i < cells && in_bounds(o + (x0 + i) * (kParts * 128), 1, a.ext_partials, a.status))
                          ? __ldcg(a.partials + o + (x0 + i) * (kParts * 128))
                          : make_float2(-INFINITY, 0.f);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) join_stats(m2, l, v[i]);
+            for (int i = 0; i < 16; ++i) join_stats(m2, l, v[i]);
           }
-          const int jsub = etid / (nrt * 128), jrow = etid % (nrt * 128);
-          sh.merge[jsub * kRowsMax + jrow] = make_float2(m2, l);
+          // (two sets of slots in turn: a set is written again only after the
+          // next chunk's barrier, which every reader has passed)
+          float2* slots = sh.merge + (jphase ? kParts * 128 : 0);
+          slots[etid] = make_float2(m2, l);
           mbar_arrive(sh.join);
           ok = __all_sync(0xffffffffu, mbar_wait(sh.join, jphase, sh.abort_flag, a.status));
           jphase ^= 1;
           if (ok && etid < nrt * 128) {
-            float2 v = sh.merge[etid];
-            for (int x = 1; x < nsub; ++x) join_stats(v.x, v.y, sh.merge[x * kRowsMax + etid]);
+            float2 v = slots[etid];
+            for (int x = 1; x < nsub; ++x) join_stats(v.x, v.y, slots[x * (nrt * 128) + etid]);
             join_chunk(jm, js, v);
           }
-          mbar_arrive(sh.join);                    // (the slots are read)
-          ok = __all_sync(0xffffffffu, mbar_wait(sh.join, jphase, sh.abort_flag, a.status)) && ok;
-          jphase ^= 1;
         }
         if (!ok) break;
       }
