@@ -1114,7 +1114,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         const FItem it = fused_item<PARTS>(a, item);
         const int kt0 = it.kt0, kt1 = it.kt1;
         if (kt1 == kt0) {
-          if (a.mode != kModeH2O) ++lpop;          // (the epilogue still forms them)
+          if (a.mode != kModeH2O) {
+            // the epilogue still forms them; with supplied normalisers nothing
+            // else keeps this warp from running a phase ahead of the barrier
+            if (fa.single && !mbar_wait(sh.lse_ready, lpop & 1, sh.abort_flag, a.status)) break;
+            ++lpop;
+          }
           continue;
         }
         if (!mbar_wait(sh.q_full, quse & 1, sh.abort_flag, a.status)) break;

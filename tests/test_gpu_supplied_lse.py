@@ -57,3 +57,30 @@ def test_window_lse_many_items_a_cta():
         sc = torch.empty(batch.score_shape(), device=DEV)
         R.snapkv_score(batch, qw, K, w.W, 1, sc, lse_win=lse)
         assert float(((sc - ref).abs() / ref).max()) < SCORE_RTOL
+
+
+def test_window_lse_with_empty_sequences():
+    """Empty items between full ones: the tensor core's warp must not take an
+    empty item's normaliser barrier for the next one's."""
+    lens = (700, 0, 0, 1, 0, 513, 0, 0, 0, 1100, 0, 300) * 4
+    w = I.Workload("lse", "snapkv", 6, len(lens), 8, 2, 128, max(lens), 32, 1, (0.1,), 4, (3, 5), (1, 3), seqlens=lens)
+    K, _ = I.make_kv(w, I.workload_roles(w, 3), 3, device=DEV, with_v=False)
+    qw = I.make_q_window(w, 3, device=DEV)
+    lse = torch.zeros(w.L, w.b, w.Hq, w.W, device=DEV)
+    ref = torch.zeros(w.L, w.Hkv, sum(lens), dtype=torch.float64, device=DEV)
+    t0 = 0
+    for s, n in enumerate(lens):
+        if n:
+            we = min(w.W, n)
+            q = qw[:, s].double().view(w.L, w.Hkv, w.G, w.W, w.d)[:, :, :, :we].reshape(w.L, w.Hkv, w.G * we, w.d)
+            x = torch.matmul(q, K[:, t0:t0 + n].double().permute(0, 2, 3, 1)) * w.d ** -0.5
+            pos = torch.arange(n - we, n, device=DEV).repeat(w.G)
+            x.masked_fill_(torch.arange(n, device=DEV)[None, :] > pos[:, None], float("-inf"))
+            lse[:, s, :, :we] = torch.logsumexp(x, dim=-1).view(w.L, w.Hq, we).float()
+            ref[:, :, t0:t0 + n] = torch.softmax(x, dim=-1).sum(-2)
+        t0 += n
+    batch = lib_batch(w, DEV)
+    for _ in range(8):
+        sc = torch.empty(batch.score_shape(), device=DEV)
+        R.snapkv_score(batch, qw, K, w.W, 1, sc, lse_win=lse)
+        assert float(((sc - ref).abs() / ref).max()) < SCORE_RTOL
