@@ -30,6 +30,12 @@ CASES = {
     "two_chunks": _w(10, 4, 4, 128, 8500, 32),
     "eight_chunks": _w(4, 4, 2, 64, 66000, 64),
     "varlen": _w(7, 4, 4, 128, 3000, 32, (3000, 0, 1, 700)),
+    # (several rounds of items a CTA)
+    "rounds_g1_8_rows": _w(40, 2, 1, 128, 2500, 8),
+    "rounds_d64": _w(100, 4, 4, 64, 5000, 32),
+    "rounds_32_cells": _w(12, 8, 2, 128, 16384, 64),
+    "rounds_empty_last_part": _w(80, 4, 3, 128, 2561, 40),
+    "rounds_varlen": _w(40, 2, 4, 128, 4000, 32, (4000, 1, 0, 1030, 2300)),
     "varlen_chunks_g7": _w(7, 4, 7, 128, 9000, 32, (9000, 129, 5000)),
 }
 
