@@ -1027,7 +1027,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int r = i >> 4, kk = i & 15;
     reinterpret_cast<uint16_t*>(sh.ones)[nl_elem(r, kk)] = kk < 3 ? 0x3F80u : 0u;   // bf16 1.0
   }
-  for (int i = threadIdx.x; i < 2 * kRowsMax * 8; i += kThreads) reinterpret_cast<uint32_t*>(sh.nlb)[i] = 0u;
+  for (int i = threadIdx.x; i < 2 * kRowsMax * 2; i += kThreads)
+    reinterpret_cast<uint4*>(sh.nlb)[i] = make_uint4(0u, 0u, 0u, 0u);
   fence_proxy_async_smem();
   if (warp == kMmaWarp) {
     tmem_alloc(sh.tmem_base, kTmemCols);

@@ -455,6 +455,15 @@ __global__ void __launch_bounds__(kMergeWarps * 32) decode_combine_kernel(const 
   if (!in_bounds(base - a.part, (ns > 0 ? (ns - 1) * stride : 0) + a.d + 2, a.ext_part, a.status) ||
       !in_bounds(dst0, a.d, a.ext_out, a.status))
     return;                                          // (checked build only)
+  if (!SHARE && ns == 1) {                           // (one split: no reference to wait for)
+    const float L1 = base[a.d + 1];
+#pragma unroll
+    for (int i = 0; i < DPL; ++i) {
+      const float o = base[lane * DPL + i];
+      a.out[dst0 + lane * DPL + i] = L1 > 0.f ? o / L1 : 0.f;
+    }
+    return;
+  }
   float M = -INFINITY;
   for (int x = lane; x < ns; x += 32) M = fmaxf(M, base[x * stride + a.d]);
 #pragma unroll

@@ -226,6 +226,7 @@ struct ScorePlan {
 constexpr int kFusedChunkTiles = 64;
 constexpr int kFusedMaxChunks = 8;
 constexpr int kMeetingTiles = 7;   // cost of an item's start and meeting, in key tiles
+constexpr int kJoinTiles = 3;      // and of joining a cut chunk's cells
 
 int64_t score_elems(const BatchInfo& bi) {
   return bi.varlen ? static_cast<int64_t>(bi.L) * bi.Hkv * bi.T : bi.n_units * bi.n_max;
@@ -276,28 +277,26 @@ int plan_score(int mode, const BatchInfo& bi, int W, bool need_partials, bool ne
     p->grid1 = a.n_units * a.n_chunks;
     p->grid2 = p->grid1;
     a.nrb_max = 1;
-    // A batch of at most half as many chunks as SMs splits each chunk's cells
-    // over as many CTAs as there are SMs for.
     a.cells_max = (a.chunk_tiles + kCellTiles - 1) / kCellTiles;
-    if (p->fused && split) {
-      const int64_t parts = num_sms() / (static_cast<int64_t>(a.n_units) * a.n_chunks);
-      a.n_parts = parts < 1 ? 1 : (parts < a.cells_max ? static_cast<int32_t>(parts) : a.cells_max);
-      // A few more chunks than SMs: parts where they make the rounds of items
-      // a CTA goes through (a part's tiles and its meeting, about seven tiles'
-      // worth, each) cheaper.  160 units of 64 tiles: two rounds of whole
-      // chunks 172 us, five of quarters 144 us; 256 units: two rounds, 176 us,
-      // against seven, 203 us.  (Packed batches: chunks differ in length.)
-      const int64_t chunks = static_cast<int64_t>(a.n_units) * a.n_chunks;
-      if (a.n_parts == 1 && !bi.varlen && chunks <= 4 * num_sms()) {
-        int64_t best = INT64_MAX;                  // (less 3%: of the whole chunks' cost)
-        for (int x = 1; x <= 8 && x <= a.cells_max && x * a.n_chunks <= num_sms(); ++x) {
-          const int64_t grid = num_sms() / (a.n_chunks * x) * (a.n_chunks * x);
-          const int64_t tiles = std::min((a.cells_max + x - 1) / x * kCellTiles, a.chunk_tiles);
-          const int64_t cost = (chunks * x + grid - 1) / grid * (tiles + kMeetingTiles);
-          if (cost < best) {
-            best = x == 1 ? cost - cost / 32 : cost;
-            a.n_parts = x;
-          }
+    // Chunks are cut into the number of parts whose rounds of items cost least,
+    // in key tiles: a part's own, seven for its start and meeting, three more
+    // for the join of a cut chunk's cells.  8 units of 64 tiles: one CTA each
+    // 84 us, sixteen 19 us; 160 units: two rounds of whole chunks 172 us, five
+    // of quarters 143 us; 256 units: two rounds 176 us, seven of quarters 203
+    // us; 76 units of 9 tiles: whole 29 us, halves 31 us.  (Packed batches,
+    // whose chunks differ in length, are cut only while one round holds them.)
+    const int64_t chunks = static_cast<int64_t>(a.n_units) * a.n_chunks;
+    if (p->fused && split && chunks <= 4 * num_sms()) {
+      int64_t best = INT64_MAX;
+      for (int x = 1; x <= a.cells_max && x * a.n_chunks <= num_sms(); ++x) {
+        const int64_t grid = num_sms() / (a.n_chunks * x) * (a.n_chunks * x);
+        const int64_t rounds = (chunks * x + grid - 1) / grid;
+        if (x > 1 && rounds > 1 && (bi.varlen || x > 8)) break;
+        const int64_t tiles = std::min((a.cells_max + x - 1) / x * kCellTiles, a.chunk_tiles);
+        const int64_t cost = rounds * (tiles + kMeetingTiles + (x > 1 ? kJoinTiles : 0));
+        if (cost < best) {
+          best = x == 1 ? cost - cost / 32 : cost;   // (whole chunks unless 3% dearer)
+          a.n_parts = x;
         }
       }
     }
@@ -803,9 +802,16 @@ void decode_split(const BatchInfo& bi, int64_t m_max, int64_t total, bool fine, 
     const int64_t heads = static_cast<int64_t>(bi.L) * bi.Hkv;
     int64_t best = INT64_MAX;
     for (int64_t x = 128; x <= kDecodeRowsPerSplit; x += 64) {
-      // (packed batches: half a split more per sequence on average)
-      const int64_t ctas = bi.varlen ? heads * (total / x + (bi.b + 1) / 2) : heads * bi.b * ((m_max + x - 1) / x);
-      const int64_t cost = (ctas + slots - 1) / slots * (x + kDecodeSplitCost);
+      int64_t cost;
+      if (bi.varlen) {
+        // splits of many lengths (half a split more per sequence on average):
+        // the rows and starts of a slot, and half a split until the last ends
+        const int64_t ctas = heads * (x >= m_max ? bi.b : total / x + (bi.b + 1) / 2);
+        cost = (heads * total + ctas * kDecodeSplitCost) / slots + (x + kDecodeSplitCost) / 2;
+      } else {
+        const int64_t ctas = heads * bi.b * ((m_max + x - 1) / x);
+        cost = (ctas + slots - 1) / slots * (x + kDecodeSplitCost);
+      }
       if (cost <= best) {
         best = cost;
         r = x;

@@ -1658,7 +1658,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
   // the lane finds its word by a search over the words' prefix counts and its
   // bit by halves (a lane per word waits for the fullest word, 6.5k cycles at
   // 1024 words a CTA and a tenth kept; a lane per slot idles in nine of ten).
-  uint32_t kr[kR] = {0, 0, 0, 0, 0, 0, 0, 0};
+  uint64_t kr_lo = 0, kr_hi = 0;                   // kept per role 0 .. 3, 4 .. 7, 16 bits each
   {
     const int wseg = (nwords + NW - 1) / NW;
     const int q_end = min(nwords, (warp + 1) * wseg);
@@ -1695,8 +1695,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
           if (in_bounds(pos, 1, width, a.status)) dst[pos] = t;   // (the unit's own row)
           if (count_roles) {
             const uint32_t role = __ldg(v.rp + t);
-#pragma unroll
-            for (int x = 0; x < kR; ++x) kr[x] += role == static_cast<uint32_t>(x);
+            const uint64_t one = 1ull << (16u * (role & 3u));
+            kr_lo += role < 4u ? one : 0ull;
+            kr_hi += role - 4u < 4u ? one : 0ull;
           }
         }
       }
@@ -1725,7 +1726,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
   if (count_roles) {
 #pragma unroll
     for (int r = 0; r < kR; ++r) {
-      const int c = static_cast<int>(__reduce_add_sync(0xffffffffu, kr[r]));
+      const uint32_t mine = static_cast<uint32_t>((r < 4 ? kr_lo : kr_hi) >> (16 * (r & 3))) & 0xFFFFu;
+      const int c = static_cast<int>(__reduce_add_sync(0xffffffffu, mine));
       if (lane == 0 && c) {
         if constexpr (CL)
           add_rank(map_rank(&S.kept_role[r], 0), c);
@@ -1784,8 +1786,9 @@ void plan_select(const SelectArgs& a, SelectPlan* p, int* mode, int* nt, size_t*
   const bool stream = *mode == kStream, wide = stream || slots > 16384 + 128;
   // Threads: enough for a short latency while the SMs hold all units, no more
   // than leave room for several units on an SM otherwise (1024 x 8192 tokens:
-  // 60.7 us at 256 threads, 66.7 at 512; 8 x 8192: 18.9 and 15.9 us).
-  *nt = wide ? 1024 : slots > 8192 + 128 || (slots > 2048 + 128 && a.n_units <= 4 * kSms) ? 512 : 256;
+  // 60.7 us at 256 threads, 66.7 at 512; 8 x 8192: 18.9 and 15.9; 304 CTAs of
+  // 512 threads fit: 320 x 2628 17.4 and 21.9, 560 x 6844 42 and 55).
+  *nt = wide ? 1024 : slots > 8192 + 128 || (slots > 2048 + 128 && a.n_units <= 2 * kSms) ? 512 : 256;
   p->nb = wide ? 11 : 10;
   p->n_hist = a.policy == ROLEKV_POLICY_GLOBAL ? 1 : a.n_roles;
   p->list_cap = wide ? 8192 : slots < 4096 ? slots : 4096;
