@@ -918,6 +918,44 @@ __device__ __forceinline__ FItem fused_item(const ScoreArgs& a, int item) {
   return it;
 }
 
+// Variants of the fused kernel: whole chunks (and H2O); a chunk's cells split
+// over CTAs (small batches); a dense batch with supplied normalisers, whose
+// items meet nobody, so that each CTA takes an even share of all units' key
+// tiles, an item per unit it touches.  (Each has its own registers: the
+// shares' bookkeeping spilled 60 bytes in the others, 8B 177 to 188 us.)
+enum { kWhole = 0, kSplit = 1, kShares = 2 };
+
+// A CTA's items: first_item(), then next_item() while its first argument is
+// below end_item().
+template <int V>
+__device__ __forceinline__ int first_item(const FusedArgs& fa) {
+  if (V != kShares) return blockIdx.x;
+  return static_cast<int>(static_cast<int64_t>(fa.s.n_units) * fa.unit_tiles * blockIdx.x / gridDim.x);
+}
+
+template <int V>
+__device__ __forceinline__ int end_item(const FusedArgs& fa) {
+  if (V != kShares) return fa.n_items;
+  return static_cast<int>(static_cast<int64_t>(fa.s.n_units) * fa.unit_tiles * (blockIdx.x + 1) / gridDim.x);
+}
+
+template <int V, bool UNI = false>
+__device__ __forceinline__ FItem next_item(const FusedArgs& fa, int& cur, int end) {
+  if (V != kShares) {
+    const FItem it = fused_item<V == kSplit, UNI>(fa.s, cur);
+    cur += gridDim.x;
+    return it;
+  }
+  FItem it;
+  it.u = cur / fa.unit_tiles;
+  it.chunk = it.cell0 = it.rb = 0;
+  it.kt0 = cur % fa.unit_tiles;
+  it.kt1 = min(fa.unit_tiles, it.kt0 + end - cur);
+  it.un = decode_unit<UNI>(fa.s, it.u);
+  cur += it.kt1 - it.kt0;
+  return it;
+}
+
 // (max2, sum) pairs of a row's keys: `o`'s joined to (m, l).  The roundings are
 // spelled out, so that the same pairs joined in the same order give the same
 // bits wherever that happens (in registers, or from another CTA's partials).
@@ -977,13 +1015,13 @@ __device__ __forceinline__ void issue_mma_keys_on_lanes(uint64_t dq, uint64_t dk
   }
 }
 
-// PARTS: the chunks are split over CTAs (small batches); a variant of its own,
-// so that the whole chunks' epilogue keeps its registers.
-template <int D, bool PARTS>
+template <int D, int V>
 __global__ void __launch_bounds__(kThreads, 1)
     snapkv_fused_kernel(const __grid_constant__ CUtensorMap k_map,
                         const __grid_constant__ CUtensorMap q_map, const FusedArgs fa) {
   using C = FCfg<D>;
+  constexpr bool PARTS = V == kSplit;
+  const bool single = V == kShares || fa.single;
   const ScoreArgs& a = fa.s;
   extern __shared__ uint8_t smem_raw[];
   FShared sh = fcarve<D>(smem_raw);
@@ -1054,8 +1092,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       // Items are dealt round-robin: the grid is a multiple of the chunks per
       // unit, so a unit's chunks run on different CTAs in the same round.
       const bool h2o = a.mode == kModeH2O;
-      for (int item = blockIdx.x; item < fa.n_items; item += gridDim.x) {
-        const FItem it = fused_item<PARTS>(a, item);
+      for (int cur = first_item<V>(fa), end = end_item<V>(fa); cur < end;) {
+        const FItem it = next_item<V>(fa, cur, end);
         const Unit& un = it.un;
         const int kt0 = it.kt0, kt1 = it.kt1;
         if (kt1 == kt0) continue;
@@ -1073,7 +1111,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         ++qload;
         // the chunk's key tiles, once for each pass
         bool ok = true;
-        for (int pass = fa.single; pass < 2 && ok; ++pass)
+        for (int pass = single; pass < 2 && ok; ++pass)
           for (int kt = kt0; kt < kt1; ++kt) {
             const int slot = kload % C::SK;
             if (!mbar_wait(&sh.k_empty[slot], ((kload / C::SK) & 1) ^ 1, sh.abort_flag, a.status)) {
@@ -1111,14 +1149,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       // pass 2 spans only the rows that exist, rounded up to 32 (224 of 256 at G = 7)
       const int p2n = a.nrows_pad == 256 ? ((a.nrows + 31) & ~31) : a.nrows_pad;
       const uint32_t idesc_nl = idesc_bf16_f32(128, p2n);
-      for (int item = blockIdx.x; item < fa.n_items && ok; item += gridDim.x) {
-        const FItem it = fused_item<PARTS>(a, item);
+      for (int cur = first_item<V>(fa), end = end_item<V>(fa); cur < end && ok;) {
+        const FItem it = next_item<V>(fa, cur, end);
         const int kt0 = it.kt0, kt1 = it.kt1;
         if (kt1 == kt0) {
           if (a.mode != kModeH2O) {
             // the epilogue still forms them; with supplied normalisers nothing
             // else keeps this warp from running a phase ahead of the barrier
-            if (fa.single && !mbar_wait(sh.lse_ready, lpop & 1, sh.abort_flag, a.status)) break;
+            if (single && !mbar_wait(sh.lse_ready, lpop & 1, sh.abort_flag, a.status)) break;
             ++lpop;
           }
           continue;
@@ -1127,7 +1165,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         ++quse;
         const uint64_t dq = sdesc_kmajor_sw128(smem_u32(sh.q));
         bool nl_ready = false;
-        for (int pass = fa.single; pass < 2 && ok; ++pass)
+        for (int pass = single; pass < 2 && ok; ++pass)
           for (int kt = kt0; kt < kt1; ++kt) {
             const int kslot = kuse % C::SK;
             const int ab = pair & 1;
@@ -1198,15 +1236,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     int ipop = 0;                                  // items done: barrier phases
     uint32_t jphase = 0;
     const bool h2o = a.mode == kModeH2O;
-    for (int item = blockIdx.x; item < fa.n_items && ok; item += gridDim.x) {
-      const FItem it = fused_item<PARTS, true>(a, item);
+    for (int cur = first_item<V>(fa), end = end_item<V>(fa); cur < end && ok;) {
+      const FItem it = next_item<V, true>(fa, cur, end);
       const int u = it.u, chunk = it.chunk, rb = it.rb;
       const Unit& un = it.un;
       const int n = un.n;
       const int kt0 = it.kt0, kt1 = it.kt1;
       if (h2o && kt1 == kt0) continue;           // a block past its sequence's end
 
-      if (!fa.single) {
+      if (!single) {
       // ---- pass 1: (max2, sum) of this thread's row over its keys, cell by
       // cell (H2O: the block's tiles are one cell).  A chunk's cells are
       // joined in order, here or, where the chunk is split over CTAs, from
@@ -1293,7 +1331,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // A split chunk's cells joined by all epilogue threads, thread (sub, row)
       // its slot's cells in order, then the row's slots and the chunks.
       float jm = -INFINITY, js = 0.f;
-      if (PARTS && !fa.single) {
+      if (PARTS && !single) {
         for (int c = 0; c < a.n_chunks && ok; ++c) {
           int c0, c1t;
           chunk_tiles(a, n, c, &c0, &c1t);
@@ -1331,7 +1369,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int j = etid;
         const int p = row_position(a, n, rb, j);
         float nl = -INFINITY;
-        if (h2o && fa.single) {
+        if (h2o && single) {
           // the caller's natural-log LSE of the query row (head g, position p)
           if (p >= 0) {
             const int g = j / a.P;
@@ -1344,7 +1382,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         } else if (h2o) {
           const float2 ml = sh.merge[j];
           if (p >= 0 && ml.y > 0.f) nl = -(ml.x + log2f(ml.y));
-        } else if (fa.single) {
+        } else if (single) {
           const int64_t o = static_cast<int64_t>(u) * kRowsMax + j;
           nl = (p >= 0 && in_bounds(o, 1, a.ext_lse2, a.status)) ? a.lse2[o] : -INFINITY;
         } else if (PARTS) {
@@ -1610,17 +1648,17 @@ cudaError_t launch_attn_pass(int pass, int d, const CUtensorMap& kmap, const CUt
                    : launch_pass<64, kPassColsum>(kmap, qmap, a, grid, stream);
 }
 
-template <int D, bool PARTS>
+template <int D, int V>
 static cudaError_t launch_fused(const CUtensorMap& kmap, const CUtensorMap& qmap,
                                 const FusedArgs& a, cudaStream_t stream) {
   using C = FCfg<D>;
-  cudaError_t e = cudaFuncSetAttribute(snapkv_fused_kernel<D, PARTS>,
+  cudaError_t e = cudaFuncSetAttribute(snapkv_fused_kernel<D, V>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemAlloc);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, snapkv_fused_kernel<D, PARTS>, kThreads,
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, snapkv_fused_kernel<D, V>, kThreads,
                                                          C::kSmemAlloc)) != cudaSuccess)
     return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
@@ -1633,7 +1671,8 @@ static cudaError_t launch_fused(const CUtensorMap& kmap, const CUtensorMap& qmap
   // (no more CTAs than items: a small batch does not set up idle CTAs; the
   // count stays a multiple of the items per unit)
   const int items = ((a.n_items + nc - 1) / nc) * nc;
-  const int grid = std::min((sms / nc) * nc, std::max(items, nc));
+  const int grid = V == kShares ? static_cast<int>(std::min<int64_t>(sms, static_cast<int64_t>(a.s.n_units) * a.unit_tiles))
+                                : std::min((sms / nc) * nc, std::max(items, nc));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(grid));
   cfg.blockDim = dim3(kThreads);
@@ -1644,16 +1683,18 @@ static cudaError_t launch_fused(const CUtensorMap& kmap, const CUtensorMap& qmap
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, snapkv_fused_kernel<D, PARTS>, kmap, qmap, a);
+  e = cudaLaunchKernelEx(&cfg, snapkv_fused_kernel<D, V>, kmap, qmap, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
 cudaError_t launch_snapkv_fused(int d, const CUtensorMap& kmap, const CUtensorMap& qmap,
                                 const FusedArgs& a, cudaStream_t stream) {
+  if (a.unit_tiles > 0)
+    return d == 128 ? launch_fused<128, kShares>(kmap, qmap, a, stream) : launch_fused<64, kShares>(kmap, qmap, a, stream);
   if (a.s.n_parts > 1)
-    return d == 128 ? launch_fused<128, true>(kmap, qmap, a, stream) : launch_fused<64, true>(kmap, qmap, a, stream);
-  return d == 128 ? launch_fused<128, false>(kmap, qmap, a, stream) : launch_fused<64, false>(kmap, qmap, a, stream);
+    return d == 128 ? launch_fused<128, kSplit>(kmap, qmap, a, stream) : launch_fused<64, kSplit>(kmap, qmap, a, stream);
+  return d == 128 ? launch_fused<128, kWhole>(kmap, qmap, a, stream) : launch_fused<64, kWhole>(kmap, qmap, a, stream);
 }
 
 cudaError_t launch_snapkv_lse(const ScoreArgs& a, const float* lse_win, cudaStream_t stream) {

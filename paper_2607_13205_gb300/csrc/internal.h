@@ -65,6 +65,8 @@ struct FusedArgs {
   ScoreArgs s;                      // s.n_chunks = chunks per unit, s.chunk_tiles = tiles per chunk
   int32_t* work;                    // [1 + u]: chunks of unit u done with pass 1 ([0] unused)
   int32_t n_items;
+  int32_t unit_tiles;               // > 0 (single, dense SnapKV): key tiles of a unit; the CTAs
+                                    // share all units' tiles evenly instead of taking items
   int32_t single;                   // 1: pass 2 only; SnapKV normalisers given in s.lse2,
                                     // H2O ones in h2o_lse
   const float* h2o_lse;             // H2O, single: natural-log LSE of every query row
