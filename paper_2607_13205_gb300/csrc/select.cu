@@ -61,6 +61,7 @@ constexpr uint32_t kCodeKeep = 0x40;   // the token's bucket keeps everything
 constexpr uint32_t kCodeDrop = 0x80;   // no bucket keeps the token
 // codes 0 .. kR-1: the token's bucket keeps only keys above a threshold
 constexpr int kMaxRanks = 8;           // CTAs per unit (the portable cluster size)
+constexpr int kDenseWords = 400;       // kept of 32 words above which a lane takes a slot, not an output
 constexpr int kRankCost = 3000;        // most compares (sum of squared runs) taken by rank
 constexpr int kTieCap = 256;           // ranked ties held in shared memory
 
@@ -1657,8 +1658,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
   // Warp w writes its words' positions, 32 words at a time, a lane per output:
   // the lane finds its word by a search over the words' prefix counts and its
   // bit by halves (a lane per word waits for the fullest word, 6.5k cycles at
-  // 1024 words a CTA and a tenth kept; a lane per slot idles in nine of ten).
+  // 1024 words a CTA and a tenth kept).  Its cost grows with what is kept;
+  // where that is much, a lane per slot of each word is cheaper.  512 x 8192
+  // tokens, search and slots: B 0.2 41.2 and 43.8 us, 0.3 43.2 and 44.4, 0.5
+  // 46.6 and 44.5; 1024 x 32768 at 0.3 223 and 231; 168 x 110545 at 0.5 229
+  // and 223: the line is drawn at kDenseWords, 0.39 of the slots.
   uint64_t kr_lo = 0, kr_hi = 0;                   // kept per role 0 .. 3, 4 .. 7, 16 bits each
+  auto put = [&](int pos, int t) {
+    if (in_bounds(pos, 1, width, a.status)) dst[pos] = t;   // (the unit's own row)
+    if (count_roles) {
+      const uint32_t role = __ldg(v.rp + t);
+      const uint64_t one = 1ull << (16u * (role & 3u));
+      kr_lo += role < 4u ? one : 0ull;
+      kr_hi += role - 4u < 4u ? one : 0ull;
+    }
+  };
   {
     const int wseg = (nwords + NW - 1) / NW;
     const int q_end = min(nwords, (warp + 1) * wseg);
@@ -1672,6 +1686,17 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
         if (lane >= o) incl += x;
       }
       const int tot = __shfl_sync(0xffffffffu, incl, 31);
+      if (tot > kDenseWords) {
+        const uint32_t below = (1u << lane) - 1u;
+#pragma unroll 4
+        for (int w = 0; w < 32; ++w) {
+          const uint32_t m = __shfl_sync(0xffffffffu, mine, w);
+          const int first = pos0 + __shfl_sync(0xffffffffu, incl, w) - __popc(m);
+          if ((m >> lane) & 1u) put(first + __popc(m & below), slot0 + (q0 + w) * 32 + lane - off);
+        }
+        pos0 += tot;
+        continue;
+      }
       for (int j0 = 0; j0 < tot; j0 += 32) {
         const int j = min(j0 + lane, tot - 1);
         int w = 0;                                 // first word with more than j bits up to it
@@ -1690,16 +1715,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
             bit += o;
           }
         }
-        const int pos = pos0 + j, t = slot0 + (q0 + w) * 32 + bit - off;
-        if (j0 + lane < tot) {
-          if (in_bounds(pos, 1, width, a.status)) dst[pos] = t;   // (the unit's own row)
-          if (count_roles) {
-            const uint32_t role = __ldg(v.rp + t);
-            const uint64_t one = 1ull << (16u * (role & 3u));
-            kr_lo += role < 4u ? one : 0ull;
-            kr_hi += role - 4u < 4u ? one : 0ull;
-          }
-        }
+        if (j0 + lane < tot) put(pos0 + j, slot0 + (q0 + w) * 32 + bit - off);
       }
       pos0 += tot;
     }

@@ -52,6 +52,12 @@ CASES = [
     (50001, 7, R.POLICY_ROLE_QUOTA, 7, 0.1, 32, "tied", (50001, 3, 0, 17111, 1)),
     (4096, 40, R.POLICY_ROLE_QUOTA, 7, 0.1, 0, "spread"),
     (8192, 160, R.POLICY_SLACK, 7, 0.3, 0, "tied"),
+    # positions written by slot where more than 0.39 of a run of words is kept
+    (5003, 40, R.POLICY_GLOBAL, 3, 0.6, 5, "spread"),
+    (2049, 40, R.POLICY_ROLE_QUOTA, 1, 0.4, 0, "spread"),
+    (8191, 2, R.POLICY_SLACK, 7, 0.4, 0, "constant"),
+    (45003, 20, R.POLICY_ROLE_QUOTA, 7, 0.5, 0, "spread"),
+    (70000, 20, R.POLICY_GLOBAL, 7, 1.0, 0, "tied"),
 ]
 
 
