@@ -1102,7 +1102,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         const FItem it = next_item<V>(fa, cur, end);
         const Unit& un = it.un;
         const int kt0 = it.kt0, kt1 = it.kt1;
-        if (kt1 == kt0) continue;
+        if (kt1 == kt0) {
+          // (it has no partials: it is only counted at its unit's meeting)
+          if (!single && !h2o) atomicAdd(fa.work + 1 + it.u, 1);
+          continue;
+        }
         // the item's query rows: the unit's window (SnapKV) or query block (H2O)
         if (!mbar_wait(sh.q_empty, (qload & 1) ^ 1, sh.abort_flag, a.status)) break;
         mbar_arrive_expect_tx(sh.q_full, static_cast<uint32_t>(a.nrows) * D * 2);
@@ -1148,7 +1152,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ------------------------------------------------------------------ MMA
     if (lane == 0) {
       int kuse = 0, quse = 0, pair = 0;
-      int lpop = 0;                                // items whose normalisers the epilogue forms
+      int lpop = 0;                                // items with key tiles: lse_ready phases
       bool ok = true;
       const uint64_t ones_desc = sdesc_kmajor_noswizzle(smem_u32(sh.ones), 128, 256);
       const uint64_t nl_desc0 = sdesc_kmajor_noswizzle(smem_u32(sh.nlb), 128, 256);
@@ -1158,15 +1162,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int cur = first_item<V>(fa), end = end_item<V>(fa); cur < end && ok;) {
         const FItem it = next_item<V>(fa, cur, end);
         const int kt0 = it.kt0, kt1 = it.kt1;
-        if (kt1 == kt0) {
-          if (a.mode != kModeH2O) {
-            // the epilogue still forms them; with supplied normalisers nothing
-            // else keeps this warp from running a phase ahead of the barrier
-            if (single && !mbar_wait(sh.lse_ready, lpop & 1, sh.abort_flag, a.status)) break;
-            ++lpop;
-          }
-          continue;
-        }
+        // An item without key tiles has no phase of any barrier.  Only an item's
+        // tiles keep this warp and the epilogue within a phase of each other,
+        // and a parity tells no more than that apart: with an lse_ready phase
+        // for it, this warp could take an older item's normalisers for the
+        // next one's, or miss the phase it waits for.
+        if (kt1 == kt0) continue;
         if (!mbar_wait(sh.q_full, quse & 1, sh.abort_flag, a.status)) break;
         ++quse;
         const uint64_t dq = sdesc_kmajor_sw128(smem_u32(sh.q));
@@ -1239,7 +1240,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const float2 cc = make_float2(c1, c1);
     int pair = 0, xchg = 0;
     bool ok = true;
-    int ipop = 0;                                  // items done: barrier phases
+    int ipop = 0;                                  // items with key tiles done: barrier phases
     uint32_t jphase = 0;
     const bool h2o = a.mode == kModeH2O;
     for (int cur = first_item<V>(fa), end = end_item<V>(fa); cur < end && ok;) {
@@ -1248,7 +1249,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const Unit& un = it.un;
       const int n = un.n;
       const int kt0 = it.kt0, kt1 = it.kt1;
-      if (h2o && kt1 == kt0) continue;           // a block past its sequence's end
+      if (kt1 == kt0) continue;
 
       if (!single) {
       // ---- pass 1: (max2, sum) of this thread's row over its keys, cell by
@@ -1256,7 +1257,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // joined in order, here or, where the chunk is split over CTAs, from
       // the cells' partials: the same bits either way.
       const int pos = row_position(a, n, rb, row);
-      const int step = h2o ? max(1, kt1 - kt0) : kCellTiles;
+      const int step = h2o ? kt1 - kt0 : kCellTiles;
       float m2 = -INFINITY, l = 0.f;
       for (int ck = kt0; ck < kt1 && ok; ck += step) {
         float cm = -INFINITY, cl = 0.f;
@@ -1394,14 +1395,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         } else if (PARTS) {
           if (p >= 0 && js > 0.f) nl = -(jm + log2f(js));
         } else if (p >= 0) {
-          // one online merge over the chunks, eight independent loads in flight
+          // one online merge over the chunks with keys, eight independent loads
+          // in flight
+          const int nt = (n + kTileKeys - 1) / kTileKeys;
+          const int ct = (nt + a.n_chunks - 1) / a.n_chunks;
+          const int nc = (nt + ct - 1) / ct;
           const float2* part_j = a.partials + static_cast<int64_t>(u) * a.n_chunks * kRowsMax + j;
           float m = -INFINITY, s = 0.f;
-          for (int c0 = 0; c0 < a.n_chunks; c0 += 8) {
+          for (int c0 = 0; c0 < nc; c0 += 8) {
             float2 v[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-              v[i] = (c0 + i < a.n_chunks &&
+              v[i] = (c0 + i < nc &&
                       in_bounds(static_cast<int64_t>(u) * a.n_chunks * kRowsMax + j + (c0 + i) * kRowsMax, 1,
                                 a.ext_partials, a.status))
                          ? __ldcg(&part_j[(c0 + i) * kRowsMax])
