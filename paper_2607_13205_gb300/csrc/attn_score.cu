@@ -1384,7 +1384,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int64_t Hq = static_cast<int64_t>(a.Hkv) * a.G;
             const int64_t o = a.varlen ? (un.l * Hq + hq) * a.T + un.tok0 + p
                                        : ((static_cast<int64_t>(un.l) * a.b + un.s) * Hq + hq) * a.n_max + p;
-            if (in_bounds(o, 1, fa.ext_h2o_lse, a.status)) nl = -__ldg(fa.h2o_lse + o) * kLog2e;
+            if (in_bounds(o, 1, fa.ext_h2o_lse, a.status)) nl = -fa.h2o_lse[o] * kLog2e;
           }
         } else if (h2o) {
           const float2 ml = sh.merge[j];
@@ -1522,7 +1522,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // Log2-domain normaliser of every SnapKV window row: combined from the pass-1
 // partials, or taken from a caller-supplied natural-log LSE.
-__global__ void snapkv_lse_kernel(const ScoreArgs a, const float* __restrict__ lse_win) {
+__global__ void snapkv_lse_kernel(const ScoreArgs a, const float* lse_win) {
   const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   wait_for_previous_kernels();
   if (idx >= static_cast<int64_t>(a.n_units) * kRowsMax) return;
@@ -1572,12 +1572,12 @@ __device__ __forceinline__ float4 pool_group(const float* row, int off, int n, i
     const int t = 4 * (g + o) - off;
     float4 f;
     if (t >= 0 && t + 4 <= n) {
-      f = __ldg(reinterpret_cast<const float4*>(row + t));
+      f = *reinterpret_cast<const float4*>(row + t);
     } else {
-      f.x = t >= 0 && t < n ? __ldg(row + t) : nan;
-      f.y = t + 1 >= 0 && t + 1 < n ? __ldg(row + t + 1) : nan;
-      f.z = t + 2 >= 0 && t + 2 < n ? __ldg(row + t + 2) : nan;
-      f.w = t + 3 >= 0 && t + 3 < n ? __ldg(row + t + 3) : nan;
+      f.x = t >= 0 && t < n ? row[t] : nan;
+      f.y = t + 1 >= 0 && t + 1 < n ? row[t + 1] : nan;
+      f.z = t + 2 >= 0 && t + 2 < n ? row[t + 2] : nan;
+      f.w = t + 3 >= 0 && t + 3 < n ? row[t + 3] : nan;
     }
     x[4 * (o + NB)] = f.x;
     x[4 * (o + NB) + 1] = f.y;
@@ -1599,9 +1599,8 @@ __device__ __forceinline__ float4 pool_group(const float* row, int off, int n, i
 // aligned 16-byte group of inputs, so the kernel moves 8 bytes a token with
 // 16-byte accesses (one output a thread from 4-byte loads took 161 us on
 // 15.7 M tokens, 126 MB of traffic; this form 48 us).
-__global__ void __launch_bounds__(kPoolThreads) maxpool_kernel(const ScoreArgs a, const float* __restrict__ in,
-                                                               float* __restrict__ out, int pool_k,
-                                                               int blocks_per_unit) {
+__global__ void __launch_bounds__(kPoolThreads) maxpool_kernel(const ScoreArgs a, const float* in, float* out,
+                                                               int pool_k, int blocks_per_unit) {
   const int u = blockIdx.x / blocks_per_unit;
   const int g = (blockIdx.x % blocks_per_unit) * kPoolThreads + threadIdx.x;
   wait_for_previous_kernels();

@@ -1,7 +1,7 @@
 // Gather-compaction of the retained K/V rows into a dense cache (Section 6:
 // the compacting implementation that realises the 1-B memory reduction).
 // Each kept slot j of a unit copies row keep_idx[j] of K and of V; a row is
-// d*2 bytes and is moved by d/8 lanes with 16-byte read-only loads and
+// d*2 bytes and is moved by d/8 lanes with 16-byte loads that skip L1 and
 // streaming stores, so a warp moves 32*16 = 512 contiguous-per-row bytes per
 // instruction and every HBM sector it touches is used whole.
 #include <cuda_runtime.h>
@@ -17,9 +17,9 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kRowsPerBlock = 64;
 
-__device__ __forceinline__ uint4 load_nc(const uint4* p) {
+__device__ __forceinline__ uint4 load_stream(const uint4* p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(p));
   return v;
@@ -76,9 +76,9 @@ __global__ void __launch_bounds__(kThreads) compact_kernel(const CompactArgs a, 
     uint4 kv = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
     if (idx >= 0 && idx < n) {
       if (in_bounds(kb + idx * a.k_tok + piece * 8, 8, a.ext_k, a.status))
-        kv = load_nc(reinterpret_cast<const uint4*>(a.k + kb + idx * a.k_tok) + piece);
+        kv = load_stream(reinterpret_cast<const uint4*>(a.k + kb + idx * a.k_tok) + piece);
       if (in_bounds(vb + idx * a.v_tok + piece * 8, 8, a.ext_v, a.status))
-        vv = load_nc(reinterpret_cast<const uint4*>(a.v + vb + idx * a.v_tok) + piece);
+        vv = load_stream(reinterpret_cast<const uint4*>(a.v + vb + idx * a.v_tok) + piece);
     } else if (idx >= n && a.status != nullptr && piece == 0) {
       atomicOr(a.status, ROLEKV_STATUS_BAD_INDEX);
     }

@@ -239,16 +239,16 @@ __global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(const Decod
     // B fragments of the query heads (head g of the group, zero past G)
     uint32_t qb[KS][2];
     {
-      const uint16_t* qp = a.q + l * a.q_layer + s * a.q_seq + static_cast<int64_t>(h * G + (g < G ? g : 0)) * a.q_head;
+      const uint16_t* qp = after_wait(a.q) + l * a.q_layer + s * a.q_seq + static_cast<int64_t>(h * G + (g < G ? g : 0)) * a.q_head;
 #pragma unroll
       for (int k = 0; k < KS; ++k) {
-        qb[k][0] = g < G ? __ldg(reinterpret_cast<const uint32_t*>(qp + k * 16 + 2 * t)) : 0u;
-        qb[k][1] = g < G ? __ldg(reinterpret_cast<const uint32_t*>(qp + k * 16 + 2 * t + 8)) : 0u;
+        qb[k][0] = g < G ? ld_u32(qp + k * 16 + 2 * t) : 0u;
+        qb[k][1] = g < G ? ld_u32(qp + k * 16 + 2 * t + 8) : 0u;
       }
     }
     const int32_t* idx = nullptr;
     if (a.keep_idx != nullptr)
-      idx = a.keep_idx + (a.varlen ? (static_cast<int64_t>(l) * a.Hkv + h) * a.Ktot + row0
+      idx = after_wait(a.keep_idx) + (a.varlen ? (static_cast<int64_t>(l) * a.Hkv + h) * a.Ktot + row0
                                    : static_cast<int64_t>(u) * a.K_dense);
     const float c1 = a.c1;
     const int d0 = lane * DPL;
@@ -257,8 +257,8 @@ __global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(const Decod
     // their latency hides behind the stage before
     auto load_idx = [&](int stt, int32_t& ia, int32_t& ib) {
       const int trr = r0 + stt * kStageRows + warp * kTileRows;
-      ia = (idx != nullptr && trr + g < r1) ? __ldg(idx + trr + g) : 0;
-      ib = (idx != nullptr && trr + g + 8 < r1) ? __ldg(idx + trr + g + 8) : 0;
+      ia = (idx != nullptr && trr + g < r1) ? static_cast<int32_t>(ld_u32(idx + trr + g)) : 0;
+      ib = (idx != nullptr && trr + g + 8 < r1) ? static_cast<int32_t>(ld_u32(idx + trr + g + 8)) : 0;
     };
     int32_t ia_cur, ib_cur;
     load_idx(0, ia_cur, ib_cur);

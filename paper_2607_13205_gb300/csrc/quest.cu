@@ -5,7 +5,7 @@
 // its page's bound, so the role-conditional selector (or its GLOBAL top-k)
 // runs on it unchanged.  One CTA per (layer, sequence, KV head): the mean of
 // the G x W_eff window rows goes to shared memory, then each warp takes whole
-// pages, streaming their key rows with 16-byte read-only loads (the kernel is
+// pages, streaming their key rows with 16-byte loads that skip L1 (the kernel is
 // bound by reading K once from HBM).  A unit's pages are split evenly over
 // CTAs, each of which forms the window mean itself (the window rows are
 // read from L2 after the first); the page minima and maxima stay packed
@@ -26,9 +26,9 @@ constexpr int kInFlight = 8;        // key-row loads a lane issues before using 
 constexpr int kCtasPerSm = 3;
 constexpr int kStartTokens = 500;   // keys a CTA could stream while one forms its window mean
 
-__device__ __forceinline__ uint4 load_nc(const uint4* p) {
+__device__ __forceinline__ uint4 load_stream(const uint4* p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(p));
   return v;
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) quest_kernel(const Quest
       for (int x = 0; x < kInFlight; ++x) {
         const int rr = r + x * RG;
         if (rr < rows)
-          v[x] = __ldg(reinterpret_cast<const uint4*>(q0 + rr / w_eff * a.q_head + rr % w_eff * a.q_tok) + c);
+          v[x] = reinterpret_cast<const uint4*>(q0 + rr / w_eff * a.q_head + rr % w_eff * a.q_tok)[c];
       }
 #pragma unroll
       for (int x = 0; x < kInFlight; ++x) {
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) quest_kernel(const Quest
 #pragma unroll
       for (int x = 0; x < kInFlight; ++x) {
         const int tt = t + x * TPI;
-        if (tt < t1) v[x] = load_nc(reinterpret_cast<const uint4*>(kb + tt * a.k_tok) + c);
+        if (tt < t1) v[x] = load_stream(reinterpret_cast<const uint4*>(kb + tt * a.k_tok) + c);
       }
 #pragma unroll
       for (int x = 0; x < kInFlight; ++x) {

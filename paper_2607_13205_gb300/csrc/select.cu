@@ -194,24 +194,24 @@ struct SelShared {
 // sp + (4g - off) is 16-byte aligned by the choice of off.
 __device__ __forceinline__ float4 load_slots(const float* sp, int off, int n, int g) {
   const int s0 = 4 * g - off;
-  if (s0 >= 0 && s0 + 4 <= n) return __ldg(reinterpret_cast<const float4*>(sp + s0));
+  if (s0 >= 0 && s0 + 4 <= n) return *reinterpret_cast<const float4*>(sp + s0);
   float4 r;
-  r.x = (s0 >= 0 && s0 < n) ? __ldg(sp + s0) : -INFINITY;
-  r.y = (s0 + 1 >= 0 && s0 + 1 < n) ? __ldg(sp + s0 + 1) : -INFINITY;
-  r.z = (s0 + 2 >= 0 && s0 + 2 < n) ? __ldg(sp + s0 + 2) : -INFINITY;
-  r.w = (s0 + 3 >= 0 && s0 + 3 < n) ? __ldg(sp + s0 + 3) : -INFINITY;
+  r.x = (s0 >= 0 && s0 < n) ? sp[s0] : -INFINITY;
+  r.y = (s0 + 1 >= 0 && s0 + 1 < n) ? sp[s0 + 1] : -INFINITY;
+  r.z = (s0 + 2 >= 0 && s0 + 2 < n) ? sp[s0 + 2] : -INFINITY;
+  r.w = (s0 + 3 >= 0 && s0 + 3 < n) ? sp[s0 + 3] : -INFINITY;
   return r;
 }
 
 // Role bytes of slots 4g .. 4g+3 (0xFF outside the sequence).
 __device__ __forceinline__ uint32_t load_roles(const uint8_t* rp, int off, int n, int g, bool vec) {
   const int s0 = 4 * g - off;
-  if (vec && s0 >= 0 && s0 + 4 <= n) return __ldg(reinterpret_cast<const uint32_t*>(rp + s0));
+  if (vec && s0 >= 0 && s0 + 4 <= n) return *reinterpret_cast<const uint32_t*>(rp + s0);
   uint32_t w = 0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int t = s0 + j;
-    const uint32_t r = (t >= 0 && t < n) ? static_cast<uint32_t>(__ldg(rp + t)) : 0xFFu;
+    const uint32_t r = (t >= 0 && t < n) ? static_cast<uint32_t>(rp[t]) : 0xFFu;
     w |= r << (8 * j);
   }
   return w;
@@ -1045,10 +1045,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
     bool seen = false;
     for (int t = max(0, slot0 - off) + tid; t < min(n, slot0 + 4 * ng - off); t += NT) {
       const int lo = max(0, t - (STREAM ? 0 : hw)), hi = min(n - 1, t + (STREAM ? 0 : hw));
-      float m = __ldg(v.sp + lo);
+      float m = v.sp[lo];
       bool nan_w = isnan(m);
       for (int x = lo + 1; x <= hi; ++x) {
-        const float f = __ldg(v.sp + x);
+        const float f = v.sp[x];
         nan_w |= isnan(f);
         m = fmaxf(m, f);
       }
@@ -1664,10 +1664,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
   // 46.6 and 44.5; 1024 x 32768 at 0.3 223 and 231; 168 x 110545 at 0.5 229
   // and 223: the line is drawn at kDenseWords, 0.39 of the slots.
   uint64_t kr_lo = 0, kr_hi = 0;                   // kept per role 0 .. 3, 4 .. 7, 16 bits each
+  const uint8_t* rp = after_wait(v.rp);
   auto put = [&](int pos, int t) {
+    const uint32_t role = count_roles ? ld_u8(rp + t) : 0u;
     if (in_bounds(pos, 1, width, a.status)) dst[pos] = t;   // (the unit's own row)
     if (count_roles) {
-      const uint32_t role = __ldg(v.rp + t);
       const uint64_t one = 1ull << (16u * (role & 3u));
       kr_lo += role < 4u ? one : 0ull;
       kr_hi += role - 4u < 4u ? one : 0ull;
