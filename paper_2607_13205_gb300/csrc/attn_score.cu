@@ -1665,9 +1665,8 @@ static cudaError_t launch_fused(const CUtensorMap& kmap, const CUtensorMap& qmap
   cudaError_t e = cudaFuncSetAttribute(snapkv_fused_kernel<D, V>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemAlloc);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const int sms = device_sms();
+  int per_sm = 0;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, snapkv_fused_kernel<D, V>, kThreads,
                                                          C::kSmemAlloc)) != cudaSuccess)
     return e;

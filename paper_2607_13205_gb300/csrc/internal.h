@@ -6,6 +6,7 @@
 
 #include <cstdint>
 
+#include "plans.h"
 #include "rolekv.h"
 
 namespace rolekv {
@@ -16,10 +17,9 @@ enum { kModeSnapKV = 0, kModeH2O = 1 };
 // when it runs out the kernel records ROLEKV_STATUS_TIMEOUT and unwinds.
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
-// Key tiles of a cell, the unit in which a SnapKV chunk's row statistics are
-// joined and, in small batches, split over CTAs.  The statistics of a row are
-// joined cell by cell in both cases, so the scores do not depend on the split.
-constexpr int kCellTiles = 4;
+// SMs of the calling thread's current device; GB300's where there is none (a
+// workspace sized on a host without a GPU).
+int device_sms();
 
 // Everything the two attention passes need, passed by value to the kernels.
 struct ScoreArgs {

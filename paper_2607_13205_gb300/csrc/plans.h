@@ -1,0 +1,201 @@
+// Launch plans: how the work of a call is cut over a device of `sms` SMs.  Host
+// arithmetic without CUDA, from sizes alone, so that it can be checked on its
+// own; times in the comments were measured on a GB300 (152 SMs).
+#pragma once
+
+#include <algorithm>
+#include <cstdint>
+
+namespace rolekv {
+
+// Score ----------------------------------------------------------------------
+
+// Key tiles of a cell, the unit in which a SnapKV chunk's row statistics are
+// joined and, in small batches, split over CTAs.  The statistics of a row are
+// joined cell by cell in both cases, so the scores do not depend on the split.
+constexpr int kCellTiles = 4;
+
+constexpr int kMeetingTiles = 7;   // cost of an item's start and meeting, in key tiles
+constexpr int kJoinTiles = 3;      // and of joining a cut chunk's cells
+
+// CTAs a chunk is cut into: the number of parts whose rounds of items cost
+// least, in key tiles: a part's own, seven for its start and meeting, three
+// more for the join of a cut chunk's cells.  8 units of 64 tiles: one CTA each
+// 84 us, sixteen 19 us; 160 units: two rounds of whole chunks 172 us, five of
+// quarters 143 us; 256 units: two rounds 176 us, seven of quarters 203 us; 76
+// units of 9 tiles: whole 29 us, halves 31 us.  (Packed batches, whose chunks
+// differ in length, are cut only while one round holds them.)
+inline int score_parts(bool varlen, int64_t units, int n_chunks, int chunk_tiles, int sms) {
+  const int cells = (chunk_tiles + kCellTiles - 1) / kCellTiles;
+  const int64_t chunks = units * n_chunks;
+  int parts = 1;
+  if (chunks > 4 * static_cast<int64_t>(sms)) return parts;
+  int64_t best = INT64_MAX;
+  for (int x = 1; x <= cells && x * n_chunks <= sms; ++x) {
+    const int64_t grid = sms / (n_chunks * x) * (n_chunks * x);
+    const int64_t rounds = (chunks * x + grid - 1) / grid;
+    if (x > 1 && rounds > 1 && (varlen || x > 8)) break;
+    const int64_t tiles = std::min((cells + x - 1) / x * kCellTiles, chunk_tiles);
+    const int64_t cost = rounds * (tiles + kMeetingTiles + (x > 1 ? kJoinTiles : 0));
+    if (cost < best) {
+      best = x == 1 ? cost - cost / 32 : cost;     // (whole chunks unless 3% dearer)
+      parts = x;
+    }
+  }
+  return parts;
+}
+
+// Decode ---------------------------------------------------------------------
+
+constexpr int kDecodeRowsPerSplit = 1024;
+constexpr int kDecodeSplitCost = 320;       // rows a CTA could stream while one starts and ends
+
+// Rows of a split: a unit's splits are equal in length, a multiple of the
+// kernel's 64-row stage, so that they finish together.  fine: as long as makes
+// the fewest rows pass one after another through an SM's CTAs (whole waves of
+// CTAs, and their starts); otherwise about kDecodeRowsPerSplit rows, which
+// they never pass (a warp's sums would get longer, their error larger).  8
+// units x 819 rows: 16.2 us in one split each, 6.7 us in seven; 32 x 3277 rows
+// 17.5 and 12.5 us; 8 x 131072 163 and 100 us.  Of start costs 40 to 320 rows
+// the last is best where the splits differ (256 x 820 rows 25.4 us, 26.4 at 80).
+// heads: layers x KV heads, of sequences with m_max rows (varlen: at most
+// m_max, `total` together).
+inline int64_t decode_split_rows(bool varlen, int64_t heads, int64_t b, int64_t m_max, int64_t total, int d,
+                                 bool fine, int sms) {
+  const int64_t ns = m_max > 0 ? (m_max + kDecodeRowsPerSplit - 1) / kDecodeRowsPerSplit : 1;
+  int64_t r = (m_max + ns - 1) / ns;
+  r = r > 0 ? (r + 63) / 64 * 64 : 64;
+  if (!fine) return r;
+  // CTAs resident at once: limited by their two stages of shared memory
+  const int64_t slots = static_cast<int64_t>(sms) * (d == 128 ? 3 : 6);
+  int64_t best = INT64_MAX;
+  for (int64_t x = 128; x <= kDecodeRowsPerSplit; x += 64) {
+    int64_t cost;
+    if (varlen) {
+      // splits of many lengths (half a split more per sequence on average):
+      // the rows and starts of a slot, and half a split until the last ends
+      const int64_t ctas = heads * (x >= m_max ? b : total / x + (b + 1) / 2);
+      cost = (heads * total + ctas * kDecodeSplitCost) / slots + (x + kDecodeSplitCost) / 2;
+    } else {
+      const int64_t ctas = heads * b * ((m_max + x - 1) / x);
+      cost = (ctas + slots - 1) / slots * (x + kDecodeSplitCost);
+    }
+    if (cost <= best) {
+      best = cost;
+      r = x;
+    }
+    if (x >= m_max) break;
+  }
+  return r;
+}
+
+// Quest ----------------------------------------------------------------------
+
+constexpr int kQuestCtasPerSm = 3;
+constexpr int kQuestStartTokens = 500;   // keys a CTA could stream while one forms its window mean
+
+struct QuestSplit {
+  int64_t ctas, pages;                   // CTAs of the longest unit, pages of each
+};
+
+// CTAs per unit: the number for which the fewest keys pass one after another
+// through a CTA slot of the SMs, counting whole waves of CTAs and each one's
+// start.  64 units of 2048 pages: 8 CTAs a unit are 1.12 waves (116 us), 7
+// just under one (84 us, 81 at the copy rate); 8 units of 512 pages 35.6 us
+// with two CTAs a unit, 8.3 us with 52.  A start costs about what streaming
+// 500 keys does: at 250, 240 units of 1255 keys went to three CTAs each (19.4
+// to 22.7 us); the long cases differ by 2% between 100 and 600.
+// heads: layers x KV heads, of b sequences of n_max tokens (varlen: at most
+// n_max, T together).
+inline QuestSplit quest_split(bool varlen, int64_t heads, int64_t b, int64_t n_max, int64_t T, int64_t page,
+                              int sms) {
+  const int64_t slots = static_cast<int64_t>(sms) * kQuestCtasPerSm;
+  const int64_t units = heads * b;
+  const int64_t pages = (n_max + page - 1) / page;
+  int64_t best = INT64_MAX, ctas = 1;
+  if (varlen) {
+    // rows of many lengths: the keys and
+    // starts of a slot, and half a CTA's keys until the last one ends
+    for (int64_t c = 1; c <= 64 && c <= pages; ++c) {
+      const int64_t keys = (pages + c - 1) / c * page;
+      const int64_t n = heads * (T / keys + (b + 1) / 2);
+      const int64_t cost = (heads * T + n * kQuestStartTokens) / slots + (keys + kQuestStartTokens) / 2;
+      if (cost < best) {
+        best = cost;
+        ctas = c;
+      }
+    }
+  }
+  for (int64_t waves = (units + slots - 1) / slots, i = 0; i < 12 && !varlen; ++waves, ++i) {
+    int64_t c = waves * slots / units;
+    c = c < 1 ? 1 : (c < pages ? c : pages);
+    const int64_t per = (pages + c - 1) / c;
+    const int64_t cost = waves * (per * page + kQuestStartTokens);
+    if (cost < best) {
+      best = cost;
+      ctas = (pages + per - 1) / per;
+    }
+    if (c == pages) break;
+  }
+  return {ctas, (pages + ctas - 1) / ctas};
+}
+
+// Selection ------------------------------------------------------------------
+
+// Longest row whose keys one CTA holds in shared memory.
+constexpr int kSmemMaxN = 40960;
+
+// How a unit's row is held.
+enum { kOne = 0, kCluster = 1, kStream = 2 };
+
+struct SelectRoute {
+  int mode, ranks, threads;   // ranks: CTAs per unit (the cluster size)
+  int groups;                 // groups (of four slots) a rank's memory holds
+  bool wide;                  // the long rows' digits and list
+};
+
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int plan_groups(int groups, int ranks) {
+  return ((groups + ranks - 1) / ranks + 31) & ~31;
+}
+
+// Route, ranks and threads of a unit, by the row length and the number of
+// units.  A unit on one CTA is bound by its serial phases (set-up, quotas,
+// digit searches: 8 us for the shortest row) and by its passes over shared
+// memory (about 6 us per 8192 tokens at 1024 threads); a cluster divides the
+// passes but pays some 1 us per exchange, eight of them.  Times, role quotas,
+// pool 7, B = 0.1:
+//   8 units x 32768   one CTA 28.7 us, cluster of 4 22.5 us
+//   8 units x 131072  streaming 102.4 us, cluster of 4 36.4 us, of 8 36.8 us
+//   64 x 131072       streaming 103.4 us, cluster of 4 70.9 us (two waves)
+//   128 x 131072      streaming 103.5 us, cluster of 4 141 us (four waves)
+//   1024 x 32768      one CTA 200 us, cluster of 4 327 us (same threads)
+// so clusters are for batches that leave SMs idle: one wave of them up to
+// kSmemMaxN tokens, two beyond.  (At 8192 tokens a cluster of 4 takes 18.4 us
+// against 15.9 us for one CTA of 512 threads.)  clusters: whether the device
+// can hold a cluster of the route at all (a partition of few SMs may not).
+inline SelectRoute select_route(int n_max, int64_t units, int sms, bool clusters) {
+  const int all = (n_max + 3 + 3) / 4;             // up to three leading slots
+  SelectRoute r{kOne, 1, 0, 0, false};
+  if (n_max > kSmemMaxN) {
+    r.ranks = n_max > 4 * 32768 + 64 ? 8 : 4;
+    r.mode = clusters && units * r.ranks <= 2 * static_cast<int64_t>(sms) ? kCluster : kStream;
+  } else if (clusters && n_max > 16384 && units <= sms / 4) {
+    r.ranks = 4;
+    r.mode = kCluster;
+  }
+  if (r.mode != kCluster) r.ranks = 1;
+  r.groups = plan_groups(all, r.ranks);
+  const int slots = r.groups * 4;                  // of one rank
+  r.wide = r.mode == kStream || slots > 16384 + 128;
+  // Threads: enough for a short latency while the SMs hold all units, no more
+  // than leave room for several units on an SM otherwise (1024 x 8192 tokens:
+  // 60.7 us at 256 threads, 66.7 at 512; 8 x 8192: 18.9 and 15.9; 304 CTAs of
+  // 512 threads fit: 320 x 2628 17.4 and 21.9, 560 x 6844 42 and 55).
+  r.threads = r.wide ? 1024 : slots > 8192 + 128 || (slots > 2048 + 128 && units <= 2 * static_cast<int64_t>(sms)) ? 512 : 256;
+  return r;
+}
+
+}  // namespace rolekv

@@ -23,8 +23,6 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kInFlight = 8;        // key-row loads a lane issues before using them
-constexpr int kCtasPerSm = 3;
-constexpr int kStartTokens = 500;   // keys a CTA could stream while one forms its window mean
 
 __device__ __forceinline__ uint4 load_stream(const uint4* p) {
   uint4 v;
@@ -50,7 +48,7 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 
-__global__ void __launch_bounds__(kThreads, kCtasPerSm) quest_kernel(const QuestArgs a, int ctas_per_unit,
+__global__ void __launch_bounds__(kThreads, kQuestCtasPerSm) quest_kernel(const QuestArgs a, int ctas_per_unit,
                                                                      int pages_per_cta) {
   __shared__ float qpart[kThreads / 8][8 * 8 + 1];   // [row group][dims of a 16-byte chunk ...]
   __shared__ float qbar[128];
@@ -198,50 +196,11 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) quest_kernel(const Quest
 
 }  // namespace
 
-// CTAs per unit: the number for which the fewest keys pass one after another
-// through a CTA slot of the SMs, counting whole waves of CTAs and each one's
-// start.  64 units of 2048 pages: 8 CTAs a unit are 1.12 waves (116 us), 7
-// just under one (84 us, 81 at the copy rate); 8 units of 512 pages 35.6 us
-// with two CTAs a unit, 8.3 us with 52.  A start costs about what streaming
-// 500 keys does: at 250, 240 units of 1255 keys went to three CTAs each (19.4
-// to 22.7 us); the long cases differ by 2% between 100 and 600.
 cudaError_t launch_quest(const QuestArgs& a, cudaStream_t stream) {
   if (a.n_units == 0 || a.n_max == 0) return cudaSuccess;
-  int dev = 0, sms = 0;
-  cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  const int64_t slots = static_cast<int64_t>(sms) * kCtasPerSm;
-  const int64_t pages = (a.n_max + a.page - 1) / a.page;
-  int64_t best = INT64_MAX, ctas = 1;
-  if (a.varlen) {
-    // rows of many lengths: the keys and
-    // starts of a slot, and half a CTA's keys until the last one ends
-    const int64_t heads = static_cast<int64_t>(a.L) * a.Hkv;
-    for (int64_t c = 1; c <= 64 && c <= pages; ++c) {
-      const int64_t keys = (pages + c - 1) / c * a.page;
-      const int64_t n = heads * (a.T / keys + (a.b + 1) / 2);
-      const int64_t cost = (heads * a.T + n * kStartTokens) / slots + (keys + kStartTokens) / 2;
-      if (cost < best) {
-        best = cost;
-        ctas = c;
-      }
-    }
-  }
-  for (int64_t waves = (a.n_units + slots - 1) / slots, i = 0; i < 12 && !a.varlen; ++waves, ++i) {
-    int64_t c = waves * slots / a.n_units;
-    c = c < 1 ? 1 : (c < pages ? c : pages);
-    const int64_t per = (pages + c - 1) / c;
-    const int64_t cost = waves * (per * a.page + kStartTokens);
-    if (cost < best) {
-      best = cost;
-      ctas = (pages + per - 1) / per;
-    }
-    if (c == pages) break;
-  }
-  const int64_t per = (pages + ctas - 1) / ctas;
-  return launch_early(quest_kernel, static_cast<unsigned>(a.n_units * ctas), kThreads, 0, stream, 1, a,
-                      static_cast<int>(ctas), static_cast<int>(per));
+  const QuestSplit q = quest_split(a.varlen, static_cast<int64_t>(a.L) * a.Hkv, a.b, a.n_max, a.T, a.page, device_sms());
+  return launch_early(quest_kernel, static_cast<unsigned>(a.n_units * q.ctas), kThreads, 0, stream, 1, a,
+                      static_cast<int>(q.ctas), static_cast<int>(q.pages));
 }
 
 }  // namespace rolekv

@@ -20,6 +20,14 @@
 
 namespace rolekv {
 
+int device_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return 152;
+  return sms;
+}
+
 namespace {
 
 thread_local char g_err[512] = "no error";
@@ -197,17 +205,6 @@ bool make_decode_v_map(CUtensorMap* map, const rolekv_tensor& v, int64_t span, i
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int num_sms() {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      sms = 148;
-  }
-  return sms;
-}
-
 // ------------------------------------------------------------ score plans --
 
 struct ScorePlan {
@@ -225,8 +222,6 @@ struct ScorePlan {
 // grid (152 SMs = 19 x 8) deals a unit's chunks to CTAs of the same round.
 constexpr int kFusedChunkTiles = 64;
 constexpr int kFusedMaxChunks = 8;
-constexpr int kMeetingTiles = 7;   // cost of an item's start and meeting, in key tiles
-constexpr int kJoinTiles = 3;      // and of joining a cut chunk's cells
 
 int64_t score_elems(const BatchInfo& bi) {
   return bi.varlen ? static_cast<int64_t>(bi.L) * bi.Hkv * bi.T : bi.n_units * bi.n_max;
@@ -278,28 +273,7 @@ int plan_score(int mode, const BatchInfo& bi, int W, bool need_partials, bool ne
     p->grid2 = p->grid1;
     a.nrb_max = 1;
     a.cells_max = (a.chunk_tiles + kCellTiles - 1) / kCellTiles;
-    // Chunks are cut into the number of parts whose rounds of items cost least,
-    // in key tiles: a part's own, seven for its start and meeting, three more
-    // for the join of a cut chunk's cells.  8 units of 64 tiles: one CTA each
-    // 84 us, sixteen 19 us; 160 units: two rounds of whole chunks 172 us, five
-    // of quarters 143 us; 256 units: two rounds 176 us, seven of quarters 203
-    // us; 76 units of 9 tiles: whole 29 us, halves 31 us.  (Packed batches,
-    // whose chunks differ in length, are cut only while one round holds them.)
-    const int64_t chunks = static_cast<int64_t>(a.n_units) * a.n_chunks;
-    if (p->fused && split && chunks <= 4 * num_sms()) {
-      int64_t best = INT64_MAX;
-      for (int x = 1; x <= a.cells_max && x * a.n_chunks <= num_sms(); ++x) {
-        const int64_t grid = num_sms() / (a.n_chunks * x) * (a.n_chunks * x);
-        const int64_t rounds = (chunks * x + grid - 1) / grid;
-        if (x > 1 && rounds > 1 && (bi.varlen || x > 8)) break;
-        const int64_t tiles = std::min((a.cells_max + x - 1) / x * kCellTiles, a.chunk_tiles);
-        const int64_t cost = rounds * (tiles + kMeetingTiles + (x > 1 ? kJoinTiles : 0));
-        if (cost < best) {
-          best = x == 1 ? cost - cost / 32 : cost;   // (whole chunks unless 3% dearer)
-          a.n_parts = x;
-        }
-      }
-    }
+    if (p->fused && split) a.n_parts = score_parts(a.varlen, a.n_units, a.n_chunks, a.chunk_tiles, device_sms());
     p->n_items = a.n_units * a.n_chunks * a.n_parts;
   } else {
     a.nrb_max = (bi.n_max + a.P - 1) / a.P;
@@ -394,7 +368,7 @@ int run_snapkv(const BatchInfo& bi, const int32_t* cu_seqlens, const rolekv_tens
     // with a few tiles a CTA, where a share would touch two units (8 units of
     // 64 tiles: 10.4 us, parts 9.8 us).
     const int64_t tiles = static_cast<int64_t>(a.n_units) * ((bi.n_max + kTileKeys - 1) / kTileKeys);
-    if (fa.single && !bi.varlen && tiles >= 8 * num_sms() && tiles < (1 << 30)) {
+    if (fa.single && !bi.varlen && tiles >= 8 * device_sms() && tiles < (1 << 30)) {
       fa.unit_tiles = (bi.n_max + kTileKeys - 1) / kTileKeys;
       fa.s.n_parts = 1;
     }
@@ -790,45 +764,10 @@ int role_alloc_select(const rolekv_batch* batch, const float* scores, const uint
 }
 
 namespace {
-constexpr int kDecodeRowsPerSplit = 1024;
-constexpr int kDecodeSplitCost = 320;       // rows a CTA could stream while one starts and ends
-
-// Splits of a unit's rows: equal in length, a multiple of the kernel's 64-row
-// stage, so that a unit's splits finish together.  fine: as long as makes the
-// fewest rows pass one after another through an SM's CTAs (whole waves of
-// CTAs, and their starts); otherwise about kDecodeRowsPerSplit rows, which
-// they never pass (a warp's sums would get longer, their error larger).  8
-// units x 819 rows: 16.2 us in one split each, 6.7 us in seven; 32 x 3277 rows
-// 17.5 and 12.5 us; 8 x 131072 163 and 100 us.  Of start costs 40 to 320 rows
-// the last is best where the splits differ (256 x 820 rows 25.4 us, 26.4 at 80).
 void decode_split(const BatchInfo& bi, int64_t m_max, int64_t total, bool fine, int32_t* rows_per_split,
                   int32_t* n_splits) {
-  const int64_t ns = m_max > 0 ? (m_max + kDecodeRowsPerSplit - 1) / kDecodeRowsPerSplit : 1;
-  int64_t r = (m_max + ns - 1) / ns;
-  r = r > 0 ? (r + 63) / 64 * 64 : 64;
-  if (fine) {
-    // CTAs resident at once: limited by their two stages of shared memory
-    const int64_t slots = static_cast<int64_t>(num_sms()) * (bi.d == 128 ? 3 : 6);
-    const int64_t heads = static_cast<int64_t>(bi.L) * bi.Hkv;
-    int64_t best = INT64_MAX;
-    for (int64_t x = 128; x <= kDecodeRowsPerSplit; x += 64) {
-      int64_t cost;
-      if (bi.varlen) {
-        // splits of many lengths (half a split more per sequence on average):
-        // the rows and starts of a slot, and half a split until the last ends
-        const int64_t ctas = heads * (x >= m_max ? bi.b : total / x + (bi.b + 1) / 2);
-        cost = (heads * total + ctas * kDecodeSplitCost) / slots + (x + kDecodeSplitCost) / 2;
-      } else {
-        const int64_t ctas = heads * bi.b * ((m_max + x - 1) / x);
-        cost = (ctas + slots - 1) / slots * (x + kDecodeSplitCost);
-      }
-      if (cost <= best) {
-        best = cost;
-        r = x;
-      }
-      if (x >= m_max) break;
-    }
-  }
+  const int64_t r = decode_split_rows(bi.varlen, static_cast<int64_t>(bi.L) * bi.Hkv, bi.b, m_max, total, bi.d, fine,
+                                      device_sms());
   *rows_per_split = static_cast<int32_t>(r);
   *n_splits = static_cast<int32_t>((m_max + r - 1) / r);
 }

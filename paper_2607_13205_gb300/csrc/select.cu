@@ -65,12 +65,6 @@ constexpr int kDenseWords = 400;       // kept of 32 words above which a lane ta
 constexpr int kRankCost = 3000;        // most compares (sum of squared runs) taken by rank
 constexpr int kTieCap = 256;           // ranked ties held in shared memory
 
-// Longest row whose keys one CTA holds in shared memory.
-constexpr int kSmemMaxN = 40960;
-
-// How a unit's row is held.
-enum { kOne = 0, kCluster = 1, kStream = 2 };
-
 // Launch plan of one call: ranks and threads per unit, and the layout of a
 // rank's shared memory.
 struct SelectPlan {
@@ -83,10 +77,6 @@ struct SelectPlan {
   int32_t hist_ints;   // the two digit-count buffers (and the first-digit sums)
   int32_t region_words;   // pass-1 histograms, then the candidate list
 };
-
-__host__ __device__ inline int plan_groups(int groups, int ranks) {
-  return ((groups + ranks - 1) / ranks + 31) & ~31;
-}
 
 // Monotone map of a float to uint32 (larger float -> larger key); -0 is folded
 // onto +0 so equal floats give equal keys.
@@ -1770,47 +1760,37 @@ cudaError_t launch_select_nt(const SelectArgs& a, const SelectPlan& p, size_t sm
                       static_cast<unsigned>(p.ranks), a, p);
 }
 
-// Route, ranks and threads of a unit, by the row length and the number of
-// units.  A unit on one CTA is bound by its serial phases (set-up, quotas,
-// digit searches: 8 us for the shortest row) and by its passes over shared
-// memory (about 6 us per 8192 tokens at 1024 threads); a cluster divides the
-// passes but pays some 1 us per exchange, eight of them.  Times on a GB300,
-// role quotas, pool 7, B = 0.1:
-//   8 units x 32768   one CTA 28.7 us, cluster of 4 22.5 us
-//   8 units x 131072  streaming 102.4 us, cluster of 4 36.4 us, of 8 36.8 us
-//   64 x 131072       streaming 103.4 us, cluster of 4 70.9 us (two waves)
-//   128 x 131072      streaming 103.5 us, cluster of 4 141 us (four waves)
-//   1024 x 32768      one CTA 200 us, cluster of 4 327 us (same threads)
-// so clusters are for batches that leave SMs idle: one wave of them up to
-// kSmemMaxN tokens, two beyond.  (At 8192 tokens a cluster of 4 takes 18.4 us
-// against 15.9 us for one CTA of 512 threads.)
-void plan_select(const SelectArgs& a, SelectPlan* p, int* mode, int* nt, size_t* smem) {
-  constexpr int kSms = 152;
-  const int groups = (a.n_max + 3 + 3) / 4;        // up to three leading slots
-  int ranks = 1;
-  *mode = kOne;
-  if (a.n_max > kSmemMaxN) {
-    ranks = a.n_max > 4 * 32768 + 64 ? 8 : 4;
-    *mode = static_cast<int64_t>(a.n_units) * ranks <= 2 * kSms ? kCluster : kStream;
-  } else if (a.n_max > 16384 && a.n_units <= kSms / 4) {
-    ranks = 4;
-    *mode = kCluster;
-  }
-  if (*mode == kStream) ranks = 1;
-  p->ranks = ranks;
-  p->groups = plan_groups(groups, ranks);
-  const int slots = p->groups * 4;                 // of one rank
-  const bool stream = *mode == kStream, wide = stream || slots > 16384 + 128;
-  // Threads: enough for a short latency while the SMs hold all units, no more
-  // than leave room for several units on an SM otherwise (1024 x 8192 tokens:
-  // 60.7 us at 256 threads, 66.7 at 512; 8 x 8192: 18.9 and 15.9; 304 CTAs of
-  // 512 threads fit: 320 x 2628 17.4 and 21.9, 560 x 6844 42 and 55).
-  *nt = wide ? 1024 : slots > 8192 + 128 || (slots > 2048 + 128 && a.n_units <= 2 * kSms) ? 512 : 256;
+// Clusters of the plan that the device (or the partition of it that this
+// context has) holds at once; 0: not even one.
+template <int NT>
+cudaError_t resident_clusters(const SelectPlan& p, size_t smem, int* n) {
+  cudaError_t e = cudaFuncSetAttribute(select_kernel<NT, kCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(p.ranks));
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = static_cast<unsigned>(p.ranks);
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaOccupancyMaxActiveClusters(n, select_kernel<NT, kCluster>, &cfg);
+}
+
+void plan_select(const SelectArgs& a, const SelectRoute& r, SelectPlan* p, size_t* smem) {
+  const bool stream = r.mode == kStream, wide = r.wide;
+  const int slots = r.groups * 4;                  // of one rank
+  p->ranks = r.ranks;
+  p->groups = r.groups;
   p->nb = wide ? 11 : 10;
   p->n_hist = a.policy == ROLEKV_POLICY_GLOBAL ? 1 : a.n_roles;
   p->list_cap = wide ? 8192 : slots < 4096 ? slots : 4096;
   p->hist_ints = 2 * p->n_hist * 256;
-  if ((ranks > 1 || a.policy == ROLEKV_POLICY_SLACK) && p->hist_ints < (1 << p->nb)) p->hist_ints = 1 << p->nb;
+  if ((r.ranks > 1 || a.policy == ROLEKV_POLICY_SLACK) && p->hist_ints < (1 << p->nb)) p->hist_ints = 1 << p->nb;
   p->region_words = p->n_hist << (stream ? p->nb : p->nb - 1);
   const int list_words = stream ? 2 * p->list_cap : p->list_cap;
   if (p->region_words < list_words) p->region_words = list_words;
@@ -1824,16 +1804,27 @@ void plan_select(const SelectArgs& a, SelectPlan* p, int* mode, int* nt, size_t*
 
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t stream) {
   if (a.n_units == 0) return cudaSuccess;
+  const int sms = device_sms();
   SelectPlan p;
-  int mode, nt;
   size_t smem;
-  plan_select(a, &p, &mode, &nt, &smem);
-  if (mode == kStream) return launch_select_nt<1024, kStream>(a, p, smem, stream);
-  if (mode == kCluster)
-    return nt == 1024 ? launch_select_nt<1024, kCluster>(a, p, smem, stream)
-                      : launch_select_nt<512, kCluster>(a, p, smem, stream);
-  if (nt == 1024) return launch_select_nt<1024, kOne>(a, p, smem, stream);
-  if (nt == 512) return launch_select_nt<512, kOne>(a, p, smem, stream);
+  SelectRoute r = select_route(a.n_max, a.n_units, sms, true);
+  plan_select(a, r, &p, &smem);
+  if (r.mode == kCluster) {
+    int held = 0;
+    const cudaError_t e = r.threads == 1024 ? resident_clusters<1024>(p, smem, &held)
+                                            : resident_clusters<512>(p, smem, &held);
+    if (e != cudaSuccess) return e;
+    if (held < 1) {
+      r = select_route(a.n_max, a.n_units, sms, false);
+      plan_select(a, r, &p, &smem);
+    }
+  }
+  if (r.mode == kStream) return launch_select_nt<1024, kStream>(a, p, smem, stream);
+  if (r.mode == kCluster)
+    return r.threads == 1024 ? launch_select_nt<1024, kCluster>(a, p, smem, stream)
+                             : launch_select_nt<512, kCluster>(a, p, smem, stream);
+  if (r.threads == 1024) return launch_select_nt<1024, kOne>(a, p, smem, stream);
+  if (r.threads == 512) return launch_select_nt<512, kOne>(a, p, smem, stream);
   return launch_select_nt<256, kOne>(a, p, smem, stream);
 }
 

@@ -1,0 +1,127 @@
+"""The launch plans (csrc/plans.h, host arithmetic) over devices of many sizes,
+compiled on their own."""
+
+import ctypes
+import glob
+import os
+import re
+import subprocess
+
+import pytest
+
+from paper_2607_13205_gb300.build import CSRC
+
+SHIM = r"""
+#include "plans.h"
+using namespace rolekv;
+extern "C" {
+int score(int varlen, long units, int chunks, int tiles, int sms) { return score_parts(varlen, units, chunks, tiles, sms); }
+long decode(int varlen, long heads, long b, long m_max, long total, int d, int fine, int sms) {
+  return decode_split_rows(varlen, heads, b, m_max, total, d, fine, sms);
+}
+void quest(int varlen, long heads, long b, long n_max, long T, long page, int sms, long* out) {
+  const QuestSplit q = quest_split(varlen, heads, b, n_max, T, page, sms);
+  out[0] = q.ctas;
+  out[1] = q.pages;
+}
+void select_(int n_max, long units, int sms, int clusters, int* out) {
+  const SelectRoute r = select_route(n_max, units, sms, clusters);
+  out[0] = r.mode; out[1] = r.ranks; out[2] = r.threads; out[3] = r.groups; out[4] = r.wide;
+}
+}
+"""
+
+SMS = (1, 7, 14, 30, 76, 132, 148, 152, 160)
+ONE, CLUSTER, STREAM = 0, 1, 2
+
+
+@pytest.fixture(scope="module")
+def plans(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plans")
+    src, so = os.path.join(d, "shim.cpp"), os.path.join(d, "shim.so")
+    with open(src, "w") as f:
+        f.write(SHIM)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-shared", "-fPIC", "-I", CSRC, "-o", so, src], check=True)
+    lib = ctypes.CDLL(so)
+    L, I = ctypes.c_long, ctypes.c_int
+    lib.score.argtypes = [I, L, I, I, I]
+    lib.decode.argtypes = [I, L, L, L, L, I, I, I]
+    lib.decode.restype = L
+    lib.quest.argtypes = [I, L, L, L, L, L, I, ctypes.POINTER(L)]
+    lib.quest.restype = None
+    lib.select_.argtypes = [I, L, I, I, ctypes.POINTER(I)]
+    lib.select_.restype = None
+    return lib
+
+
+def _quest(plans, *args):
+    out = (ctypes.c_long * 2)()
+    plans.quest(*args, out)
+    return out[0], out[1]
+
+
+def _select(plans, *args):
+    out = (ctypes.c_int * 5)()
+    plans.select_(*args, out)
+    return list(out)
+
+
+def test_one_source_of_the_sm_count():
+    """The device's size is asked for on each call (the current device may
+    change), in one place."""
+    code = "".join(open(f).read() for f in glob.glob(os.path.join(CSRC, "*")))
+    assert len(re.findall(r"cudaDevAttrMultiProcessorCount", code)) == 1
+    assert not re.search(r"static int \w*sm\w*|kSms\b", code)
+
+
+@pytest.mark.parametrize("sms", SMS)
+def test_score_gangs_are_resident(plans, sms):
+    for chunks in range(1, min(8, sms) + 1):
+        for tiles in (1, 4, 5, 33, 64, 200):
+            for units in (1, 2, 8, 76, 160, 256, 4096):
+                for varlen in (0, 1):
+                    x = plans.score(varlen, units, chunks, tiles, sms)
+                    assert 1 <= x <= max(1, sms // chunks) and x <= (tiles + 3) // 4
+
+
+@pytest.mark.parametrize("sms", SMS)
+def test_decode_splits(plans, sms):
+    for heads, b in ((1, 1), (8, 4), (64, 64)):
+        for m in (0, 1, 63, 64, 65, 820, 3277, 131072):
+            for varlen in (0, 1):
+                for d in (64, 128):
+                    coarse = plans.decode(varlen, heads, b, m, m * b, d, 0, sms)
+                    fine = plans.decode(varlen, heads, b, m, m * b, d, 1, sms)
+                    for r in (coarse, fine):
+                        assert 64 <= r <= 1024 and r % 64 == 0
+                    # a workspace of the fine splits holds the coarse ones' partials
+                    assert -(-m // fine) >= -(-m // coarse)
+
+
+@pytest.mark.parametrize("sms", SMS)
+def test_quest_splits_cover_the_pages(plans, sms):
+    for heads, b in ((1, 1), (8, 4), (512, 1), (7, 64)):
+        for n in (1, 15, 512, 2000, 65536):
+            for page in (1, 16, 4096):
+                for varlen in (0, 1):
+                    ctas, per = _quest(plans, varlen, heads, b, n, n * b, page, sms)
+                    pages = -(-n // page)
+                    assert 1 <= ctas <= pages and ctas * per >= pages and (ctas - 1) * per < pages
+
+
+@pytest.mark.parametrize("sms", SMS)
+def test_select_routes(plans, sms):
+    for n in (0, 1, 2048, 8192, 16384, 16385, 32768, 40960, 40961, 65536, 131072, 131137, 163840, 262144):
+        for units in (1, 8, 38, 39, 76, 77, 152, 1024):
+            mode, ranks, threads, groups, wide = _select(plans, n, units, sms, 1)
+            assert groups * 4 * ranks >= n + 3
+            assert mode == STREAM or groups * 4 <= 40960 + 128       # a rank's keys fit its shared memory
+            assert (mode == CLUSTER) == (ranks > 1) and ranks in (1, 2, 4, 8)
+            assert threads in ((512, 1024) if mode == CLUSTER else (1024,) if wide else (256, 512))
+            assert wide or groups * 4 <= 16384 + 128
+            # a device that holds no such cluster: another route, not a refusal
+            mode, ranks, threads, groups, wide = _select(plans, n, units, sms, 0)
+            assert mode == (STREAM if n > 40960 else ONE) and ranks == 1
+    # the plan follows the device
+    assert _select(plans, 65536, 57, 152, 1)[0] == CLUSTER
+    assert _select(plans, 65536, 57, 76, 1)[0] == STREAM
