@@ -92,52 +92,77 @@ inline int64_t decode_split_rows(bool varlen, int64_t heads, int64_t b, int64_t 
 // Quest ----------------------------------------------------------------------
 
 constexpr int kQuestCtasPerSm = 3;
-constexpr int kQuestStartTokens = 500;   // keys a CTA could stream while one forms its window mean
+constexpr int kQuestWarps = 8;           // warps of a CTA, each taking whole pages
+constexpr int kQuestLoads = 8 * 32;      // 16-byte loads a warp has in flight
 
 struct QuestSplit {
   int64_t ctas, pages;                   // CTAs of the longest unit, pages of each
 };
 
-// CTAs per unit: the number for which the fewest keys pass one after another
-// through a CTA slot of the SMs, counting whole waves of CTAs and each one's
-// start.  64 units of 2048 pages: 8 CTAs a unit are 1.12 waves (116 us), 7
-// just under one (84 us, 81 at the copy rate); 8 units of 512 pages 35.6 us
-// with two CTAs a unit, 8.3 us with 52.  A start costs about what streaming
-// 500 keys does: at 250, 240 units of 1255 keys went to three CTAs each (19.4
-// to 22.7 us); the long cases differ by 2% between 100 and 600.
+// CTAs per unit: the cut that takes least time by this account, in ns.  A CTA
+// starts with the window mean (4 us and 1 us for 64 rows); then each of its
+// warps takes every eighth page, 0.8 us and another 0.8 for each batch of
+// loads of a page; the CTAs resident at once share 7 TB/s.  Dense units go in
+// whole waves; packed ones, of many lengths, follow each other without gaps,
+// and half a CTA passes until the last one ends.  64 units of 2048 16-token
+// pages: 8 CTAs a unit are 1.12 waves (116 us), 7 just under one (84 us, 81 at
+// the copy rate).  With keys alone counted (500 of them for a start), 300
+// units of 1500 one-token pages took one CTA each, 245 us against 187 with
+// three; 256 units of 32 64-token pages three, 31 us against 26 with one;
+// 256 units of eight 512-token pages three, 72 us against 48; one packed unit
+// of 65536 one-token pages at most 64, 127 us against 36 with 384.
 // heads: layers x KV heads, of b sequences of n_max tokens (varlen: at most
-// n_max, T together).
+// n_max, T together); rows: of the window, over the group's heads.
 inline QuestSplit quest_split(bool varlen, int64_t heads, int64_t b, int64_t n_max, int64_t T, int64_t page,
-                              int sms) {
+                              int64_t rows, int d, int sms) {
   const int64_t slots = static_cast<int64_t>(sms) * kQuestCtasPerSm;
   const int64_t units = heads * b;
   const int64_t pages = (n_max + page - 1) / page;
-  int64_t best = INT64_MAX, ctas = 1;
-  if (varlen) {
-    // rows of many lengths: the keys and
-    // starts of a slot, and half a CTA's keys until the last one ends
-    for (int64_t c = 1; c <= 64 && c <= pages; ++c) {
-      const int64_t keys = (pages + c - 1) / c * page;
-      const int64_t n = heads * (T / keys + (b + 1) / 2);
-      const int64_t cost = (heads * T + n * kQuestStartTokens) / slots + (keys + kQuestStartTokens) / 2;
-      if (cost < best) {
-        best = cost;
-        ctas = c;
-      }
+  const int64_t start = 4000 + rows * 16;
+  const int64_t page_ns = 800 * (1 + (page * (d / 8) + kQuestLoads - 1) / kQuestLoads);
+  const auto stream_ns = [&](int64_t keys) { return keys * 2 * d / 7000; };   // at 7 TB/s
+  // (the streams and the warps' turns hold each other up a little)
+  const auto longer = [](int64_t x, int64_t y) { return std::max(x, y) + std::min(x, y) / 8; };
+  const auto cost = [&](int64_t per) {
+    const int64_t warp = (per + kQuestWarps - 1) / kQuestWarps * page_ns;
+    if (varlen && b > 1) {
+      const int64_t all = stream_ns(heads * T);
+      const int64_t n = std::max(units, heads * (T / std::min(per * page, n_max) + (b + 1) / 2));
+      if (n <= slots) return start + longer(all, warp);
+      return std::max(all + start, n * (start + warp) / slots) + (start + warp) / 2;
     }
-  }
-  for (int64_t waves = (units + slots - 1) / slots, i = 0; i < 12 && !varlen; ++waves, ++i) {
-    int64_t c = waves * slots / units;
-    c = c < 1 ? 1 : (c < pages ? c : pages);
-    const int64_t per = (pages + c - 1) / c;
-    const int64_t cost = waves * (per * page + kQuestStartTokens);
-    if (cost < best) {
-      best = cost;
-      ctas = (pages + per - 1) / per;
+    const int64_t cut = (pages + per - 1) / per, n = units * cut, last = n % slots;
+    return n / slots * (start + longer(stream_ns(slots * n_max / cut), warp)) +
+           (last > 0 ? start + longer(stream_ns(last * n_max / cut), warp) : 0);
+  };
+  int64_t best = INT64_MAX, per = pages;
+  const auto consider = [&](int64_t p) {
+    p = p < 1 ? 1 : (p < pages ? p : pages);
+    const int64_t c = cost(p);
+    if (c < best) {
+      best = c;
+      per = p;
     }
-    if (c == pages) break;
+  };
+  // The CTAs of 1, 2, ... waves, and as many pages more as its warps take in
+  // the same number of turns.
+  const int64_t all_pages = varlen && b > 1 ? heads * ((T + page - 1) / page) : units * pages;
+  const int64_t first = (units + slots - 1) / slots;
+  for (int64_t w = first; w < first + 12; ++w) {
+    int64_t p;
+    if (varlen && b > 1) {
+      const int64_t ctas = w * slots - heads * ((b + 1) / 2);   // less the sequences' short last ones
+      p = ctas > 0 ? (all_pages + ctas - 1) / ctas : pages;
+    } else {
+      p = (pages + w * slots / units - 1) / (w * slots / units);
+    }
+    // (CTAs with an SM each to themselves are not joined for that)
+    if (all_pages > p * sms) consider((p + kQuestWarps - 1) / kQuestWarps * kQuestWarps);
+    consider(p);
+    if (p <= 1) break;
   }
-  return {ctas, (pages + ctas - 1) / ctas};
+  consider(pages);
+  return {(pages + per - 1) / per, per};
 }
 
 // Selection ------------------------------------------------------------------

@@ -12,6 +12,7 @@
 // bf16 pairs until the dot product.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "device_common.cuh"
@@ -22,7 +23,8 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kInFlight = 8;        // key-row loads a lane issues before using them
+constexpr int kInFlight = kQuestLoads / 32;   // key-row loads a lane issues before using them
+static_assert(kWarps == kQuestWarps, "the plan counts a CTA's warps");
 
 __device__ __forceinline__ uint4 load_stream(const uint4* p) {
   uint4 v;
@@ -92,30 +94,24 @@ __global__ void __launch_bounds__(kThreads, kQuestCtasPerSm) quest_kernel(const 
 
   // ---- mean of the window rows (the last W_eff positions of the G heads):
   // thread (row group rg, chunk c) sums chunk c of rows rg, rg + RG, ...
+  // (Eight rows' loads issued before the first sum are slower: 300 units of 300
+  // keys, 256 window rows, 10.5 to 11.3 us; 1024 units 29.2 to 32.0.)
   {
     const int w_eff = a.W < n ? a.W : n;
     const int rows = a.G * w_eff;
     const int RG = kThreads / CR;
     const int c = tid % CR, rg = tid / CR;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const uint16_t* q0 = a.q + l * a.q_layer + s * a.q_seq + static_cast<int64_t>(h) * a.G * a.q_head;
-    for (int r = rg; r < rows; r += RG * kInFlight) {
-      uint4 v[kInFlight];                          // (the rows' loads in flight, added in order)
+    for (int r = rg; r < rows; r += RG) {
+      const int g = r / w_eff, i = r % w_eff;
+      const int64_t o = l * a.q_layer + s * a.q_seq + static_cast<int64_t>(h * a.G + g) * a.q_head +
+                        i * a.q_tok;
+      const uint4 v = reinterpret_cast<const uint4*>(a.q + o)[c];
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-      for (int x = 0; x < kInFlight; ++x) {
-        const int rr = r + x * RG;
-        if (rr < rows)
-          v[x] = reinterpret_cast<const uint4*>(q0 + rr / w_eff * a.q_head + rr % w_eff * a.q_tok)[c];
-      }
-#pragma unroll
-      for (int x = 0; x < kInFlight; ++x) {
-        if (r + x * RG >= rows) continue;
-        const uint32_t w[4] = {v[x].x, v[x].y, v[x].z, v[x].w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          acc[2 * j] += bf16_lo(w[j]);
-          acc[2 * j + 1] += bf16_hi(w[j]);
-        }
+      for (int j = 0; j < 4; ++j) {
+        acc[2 * j] += bf16_lo(w[j]);
+        acc[2 * j + 1] += bf16_hi(w[j]);
       }
     }
     // qpart[rg][c*8 + j] holds row group rg's sum of dim c*8 + j (d <= 128:
@@ -198,7 +194,8 @@ __global__ void __launch_bounds__(kThreads, kQuestCtasPerSm) quest_kernel(const 
 
 cudaError_t launch_quest(const QuestArgs& a, cudaStream_t stream) {
   if (a.n_units == 0 || a.n_max == 0) return cudaSuccess;
-  const QuestSplit q = quest_split(a.varlen, static_cast<int64_t>(a.L) * a.Hkv, a.b, a.n_max, a.T, a.page, device_sms());
+  const QuestSplit q = quest_split(a.varlen, static_cast<int64_t>(a.L) * a.Hkv, a.b, a.n_max, a.T, a.page,
+                                   static_cast<int64_t>(a.G) * std::min(a.W, a.n_max), a.d, device_sms());
   return launch_early(quest_kernel, static_cast<unsigned>(a.n_units * q.ctas), kThreads, 0, stream, 1, a,
                       static_cast<int>(q.ctas), static_cast<int>(q.pages));
 }

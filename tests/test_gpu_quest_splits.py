@@ -22,7 +22,8 @@ def _bounds(k, qbar, page):
 
 CASES = [(1, 1, 1, 1, 128, 1, 16, 8), (1, 1, 2, 4, 64, 17, 16, 8), (1, 1, 8, 4, 128, 4095, 16, 64),
          (1, 1, 8, 4, 128, 4097, 8, 32), (1, 1, 1, 7, 128, 40000, 64, 32), (60, 1, 8, 1, 64, 33, 16, 8),
-         (2, 4, 4, 7, 128, 3000, 16, 32, (3000, 0, 1, 700)), (1, 2, 4, 8, 128, 257, 4096, 32)]
+         (2, 4, 4, 7, 128, 3000, 16, 32, (3000, 0, 1, 700)), (1, 2, 4, 8, 128, 257, 4096, 32),
+         (1, 1, 1, 4, 128, 20001, 2, 64, (20001,)), (2, 3, 2, 4, 64, 9001, 8, 32, (9001, 7, 4000))]
 
 
 @pytest.mark.parametrize("case", CASES, ids=["x".join(map(str, c[:8])) for c in CASES])

@@ -19,8 +19,8 @@ int score(int varlen, long units, int chunks, int tiles, int sms) { return score
 long decode(int varlen, long heads, long b, long m_max, long total, int d, int fine, int sms) {
   return decode_split_rows(varlen, heads, b, m_max, total, d, fine, sms);
 }
-void quest(int varlen, long heads, long b, long n_max, long T, long page, int sms, long* out) {
-  const QuestSplit q = quest_split(varlen, heads, b, n_max, T, page, sms);
+void quest(int varlen, long heads, long b, long n_max, long T, long page, long rows, int d, int sms, long* out) {
+  const QuestSplit q = quest_split(varlen, heads, b, n_max, T, page, rows, d, sms);
   out[0] = q.ctas;
   out[1] = q.pages;
 }
@@ -47,7 +47,7 @@ def plans(tmp_path_factory):
     lib.score.argtypes = [I, L, I, I, I]
     lib.decode.argtypes = [I, L, L, L, L, I, I, I]
     lib.decode.restype = L
-    lib.quest.argtypes = [I, L, L, L, L, L, I, ctypes.POINTER(L)]
+    lib.quest.argtypes = [I, L, L, L, L, L, L, I, I, ctypes.POINTER(L)]
     lib.quest.restype = None
     lib.select_.argtypes = [I, L, I, I, ctypes.POINTER(I)]
     lib.select_.restype = None
@@ -104,9 +104,25 @@ def test_quest_splits_cover_the_pages(plans, sms):
         for n in (1, 15, 512, 2000, 65536):
             for page in (1, 16, 4096):
                 for varlen in (0, 1):
-                    ctas, per = _quest(plans, varlen, heads, b, n, n * b, page, sms)
+                    ctas, per = _quest(plans, varlen, heads, b, n, n * b, page, 128, 128, sms)
                     pages = -(-n // page)
                     assert 1 <= ctas <= pages and ctas * per >= pages and (ctas - 1) * per < pages
+
+
+def test_quest_splits_fit_the_page_size(plans):
+    """152 SMs, three CTAs of eight warps each."""
+    # one long packed sequence of small pages takes as many CTAs as the SMs hold
+    for n in (65536, 131072, 300000):
+        for page in (1, 4, 16):
+            ctas, per = _quest(plans, 1, 1, 1, n, n, page, 128, 128, 152)
+            assert ctas >= min(256, -(-n // page) // 8) and per * page <= 1024
+    # a batch that fills the SMs is not cut into CTAs of fewer pages than warps,
+    # nor where the starts cost more than the balance gains
+    assert _quest(plans, 0, 256, 1, 4096, 256 * 4096, 512, 128, 128, 152)[0] == 1
+    assert _quest(plans, 1, 1, 256, 4096, 256 * 4096, 512, 128, 128, 152)[0] == 1
+    assert _quest(plans, 0, 256, 1, 2000, 256 * 2000, 64, 256, 128, 152)[0] == 1
+    # one-token pages are bound by their number, not by their bytes
+    assert _quest(plans, 0, 300, 1, 1500, 300 * 1500, 1, 128, 128, 152)[0] >= 3
 
 
 @pytest.mark.parametrize("sms", SMS)
