@@ -186,41 +186,63 @@ inline int plan_groups(int groups, int ranks) {
   return ((groups + ranks - 1) / ranks + 31) & ~31;
 }
 
-// Route, ranks and threads of a unit, by the row length and the number of
-// units.  A unit on one CTA is bound by its serial phases (set-up, quotas,
-// digit searches: 8 us for the shortest row) and by its passes over shared
-// memory (about 6 us per 8192 tokens at 1024 threads); a cluster divides the
-// passes but pays some 1 us per exchange, eight of them.  Times, role quotas,
-// pool 7, B = 0.1:
-//   8 units x 32768   one CTA 28.7 us, cluster of 4 22.5 us
-//   8 units x 131072  streaming 102.4 us, cluster of 4 36.4 us, of 8 36.8 us
-//   64 x 131072       streaming 103.4 us, cluster of 4 70.9 us (two waves)
-//   128 x 131072      streaming 103.5 us, cluster of 4 141 us (four waves)
-//   1024 x 32768      one CTA 200 us, cluster of 4 327 us (same threads)
-// so clusters are for batches that leave SMs idle: one wave of them up to
-// kSmemMaxN tokens, two beyond.  (At 8192 tokens a cluster of 4 takes 18.4 us
-// against 15.9 us for one CTA of 512 threads.)  clusters: whether the device
-// can hold a cluster of the route at all (a partition of few SMs may not).
-inline SelectRoute select_route(int n_max, int64_t units, int sms, bool clusters) {
-  const int all = (n_max + 3 + 3) / 4;             // up to three leading slots
-  SelectRoute r{kOne, 1, 0, 0, false};
-  if (n_max > kSmemMaxN) {
-    r.ranks = n_max > 4 * 32768 + 64 ? 8 : 4;
-    r.mode = clusters && units * r.ranks <= 2 * static_cast<int64_t>(sms) ? kCluster : kStream;
-  } else if (clusters && n_max > 16384 && units <= sms / 4) {
-    r.ranks = 4;
-    r.mode = kCluster;
-  }
-  if (r.mode != kCluster) r.ranks = 1;
-  r.groups = plan_groups(all, r.ranks);
+// Threads and memory of a unit on `ranks` CTAs.  Threads: enough for a short
+// latency while the SMs hold all units, no more than leave room for several
+// units on an SM otherwise (1024 x 8192 tokens: 60.7 us at 256 threads, 66.7
+// at 512; 8 x 8192: 18.9 and 15.9; 304 CTAs of 512 threads fit: 320 x 2628
+// 17.4 and 21.9, 560 x 6844 42 and 55).  One CTA of a row beyond 16384 tokens
+// has 1024 from the first token on while each has an SM (16385 tokens, 38
+// units 21.4 us, 23.9 at 512; 300 units 41.9 and 33.3).
+inline SelectRoute select_shape(int n_max, int64_t units, int sms, int mode, int ranks) {
+  SelectRoute r{mode, ranks, 0, plan_groups((n_max + 3 + 3) / 4, ranks), false};   // up to three leading slots
   const int slots = r.groups * 4;                  // of one rank
-  r.wide = r.mode == kStream || slots > 16384 + 128;
-  // Threads: enough for a short latency while the SMs hold all units, no more
-  // than leave room for several units on an SM otherwise (1024 x 8192 tokens:
-  // 60.7 us at 256 threads, 66.7 at 512; 8 x 8192: 18.9 and 15.9; 304 CTAs of
-  // 512 threads fit: 320 x 2628 17.4 and 21.9, 560 x 6844 42 and 55).
-  r.threads = r.wide ? 1024 : slots > 8192 + 128 || (slots > 2048 + 128 && units <= 2 * static_cast<int64_t>(sms)) ? 512 : 256;
+  r.wide = mode == kStream || slots > 16384 + 128 || (mode == kOne && n_max > 16384 && units <= sms);
+  r.threads = r.wide ? 1024
+              : slots > 8192 + 128 || (slots > 2048 + 128 && units <= 2 * static_cast<int64_t>(sms)) ? 512
+                                                                                                     : 256;
   return r;
+}
+
+// Route of a call, by the row length and the number of units.  A unit on one
+// CTA is bound by its serial phases (set-up, quotas, digit searches: 8 us for
+// the shortest row) and by its passes over shared memory (about 6 us per 8192
+// tokens at 1024 threads); a cluster divides the passes but pays some 1 us per
+// exchange, eight of them: 18.4 us at 8192 tokens against 15.9 us for one CTA
+// of 512 threads.  Clusters run in waves of as many as the device holds:
+// held(route, alone) of them, alone with an SM for each CTA (a GPC's last SMs
+// hold none: 36 of four CTAs, 15 of eight; 74 of four at 512 threads, two CTAs
+// on an SM; 0 on a device too small for one).  Times, role quotas, pool 7,
+// B = 0.1, of one CTA or streaming and of the cluster:
+//   36 and 38 units x 20000   22.0 and 22.0; cluster of 4 22.1 and 24.0 us
+//   38 units x 28000, 32768   26.1 and 28.3; 27.2 and 28.6 (GLOBAL 29.4 and
+//                             33.2; 26.1 and 27.2)
+//   74 and 76 x 40961, 65536  44.3 and 57.7; 34.8 and 54.8, 40.1 and 62.2
+//   36, 72, 76 x 100000       81.8; 34.6, 66.9, 97.4 (one to three waves)
+//   14, 16 x 150000           114.7; of 8 38.1 and 70.5, of 4 41.2 and 41.0
+//   14, 26, 38 x 262144       189; of 8 45.0, 86.7, 128
+// so: up to kSmemMaxN tokens clusters with an SM for each CTA, above 28672
+// also those that share; beyond, of four CTAs one wave of 512 threads or two
+// of 1024; above 131136 tokens of eight while they fit one wave, or three
+// where four ranks hold no more.  (Three waves of four at 131072 tokens suit
+// GLOBAL, 115 us against 125, and cost the other policies as much.)
+template <class Held>
+inline SelectRoute select_route(int n_max, int64_t units, int sms, Held held) {
+  const auto waves = [&](const SelectRoute& r, bool alone, int64_t most) {
+    return held(r, alone) * most >= units;
+  };
+  if (n_max <= kSmemMaxN) {
+    if (n_max > 16384 && units <= sms / 4) {
+      const SelectRoute r = select_shape(n_max, units, sms, kCluster, 4);
+      if (waves(r, n_max <= 28672, 1)) return r;
+    }
+    return select_shape(n_max, units, sms, kOne, 1);
+  }
+  const SelectRoute four = select_shape(n_max, units, sms, kCluster, 4);
+  const SelectRoute eight = select_shape(n_max, units, sms, kCluster, 8);
+  const bool fits4 = n_max <= 4 * kSmemMaxN;
+  if (n_max > 4 * 32768 + 64 && waves(eight, true, fits4 ? 1 : 3)) return eight;
+  if (fits4 && waves(four, false, four.wide ? 2 : 1)) return four;
+  return select_shape(n_max, units, sms, kStream, 1);
 }
 
 }  // namespace rolekv

@@ -1761,12 +1761,11 @@ cudaError_t launch_select_nt(const SelectArgs& a, const SelectPlan& p, size_t sm
 }
 
 // Clusters of the plan that the device (or the partition of it that this
-// context has) holds at once; 0: not even one.
+// context has) holds at once; alone: with at most one CTA on an SM.
 template <int NT>
-cudaError_t resident_clusters(const SelectPlan& p, size_t smem, int* n) {
-  cudaError_t e = cudaFuncSetAttribute(select_kernel<NT, kCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
+int64_t resident_clusters(const SelectPlan& p, size_t smem, bool alone) {
+  constexpr size_t kOverHalf = 120 * 1024;         // of an SM's shared memory
+  if (alone && smem < kOverHalf) smem = kOverHalf;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(p.ranks));
   cfg.blockDim = dim3(NT);
@@ -1778,7 +1777,14 @@ cudaError_t resident_clusters(const SelectPlan& p, size_t smem, int* n) {
   attr.val.clusterDim.z = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(n, select_kernel<NT, kCluster>, &cfg);
+  int held = 0;
+  if (cudaFuncSetAttribute(select_kernel<NT, kCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(smem)) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&held, select_kernel<NT, kCluster>, &cfg) != cudaSuccess) {
+    cudaGetLastError();                            // (the other routes decide whether the call fails)
+    return 0;
+  }
+  return held;
 }
 
 void plan_select(const SelectArgs& a, const SelectRoute& r, SelectPlan* p, size_t* smem) {
@@ -1804,21 +1810,13 @@ void plan_select(const SelectArgs& a, const SelectRoute& r, SelectPlan* p, size_
 
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t stream) {
   if (a.n_units == 0) return cudaSuccess;
-  const int sms = device_sms();
   SelectPlan p;
   size_t smem;
-  SelectRoute r = select_route(a.n_max, a.n_units, sms, true);
+  const SelectRoute r = select_route(a.n_max, a.n_units, device_sms(), [&](const SelectRoute& x, bool alone) {
+    plan_select(a, x, &p, &smem);
+    return x.threads == 1024 ? resident_clusters<1024>(p, smem, alone) : resident_clusters<512>(p, smem, alone);
+  });
   plan_select(a, r, &p, &smem);
-  if (r.mode == kCluster) {
-    int held = 0;
-    const cudaError_t e = r.threads == 1024 ? resident_clusters<1024>(p, smem, &held)
-                                            : resident_clusters<512>(p, smem, &held);
-    if (e != cudaSuccess) return e;
-    if (held < 1) {
-      r = select_route(a.n_max, a.n_units, sms, false);
-      plan_select(a, r, &p, &smem);
-    }
-  }
   if (r.mode == kStream) return launch_select_nt<1024, kStream>(a, p, smem, stream);
   if (r.mode == kCluster)
     return r.threads == 1024 ? launch_select_nt<1024, kCluster>(a, p, smem, stream)

@@ -49,6 +49,8 @@ CASES = [
     (65537, 20, R.POLICY_FAIR, 7, 0.05, 0, "nan"),
     (131137, 10, R.POLICY_GLOBAL, 7, 0.1, 64, "spread"),
     (262144, 10, R.POLICY_ROLE_QUOTA, 7, 0.02, 0, "tied"),
+    (132100, 4, R.POLICY_SLACK, 7, 0.2, 0, "tied"),
+    (163840, 5, R.POLICY_GLOBAL, 7, 0.1, 32, "spread"),
     (50001, 7, R.POLICY_ROLE_QUOTA, 7, 0.1, 32, "tied", (50001, 3, 0, 17111, 1)),
     (4096, 40, R.POLICY_ROLE_QUOTA, 7, 0.1, 0, "spread"),
     (8192, 160, R.POLICY_SLACK, 7, 0.3, 0, "tied"),

@@ -24,8 +24,12 @@ void quest(int varlen, long heads, long b, long n_max, long T, long page, long r
   out[0] = q.ctas;
   out[1] = q.pages;
 }
+// clusters held, as a GB300 answers (152 SMs), other devices in proportion; or none
 void select_(int n_max, long units, int sms, int clusters, int* out) {
-  const SelectRoute r = select_route(n_max, units, sms, clusters);
+  const SelectRoute r = select_route(n_max, units, sms, [&](const SelectRoute& x, bool alone) {
+    const int two = x.threads == 512 && !alone;
+    return clusters ? static_cast<int64_t>(sms) * (x.ranks == 4 ? (two ? 74 : 36) : (two ? 36 : 15)) / 152 : int64_t{0};
+  });
   out[0] = r.mode; out[1] = r.ranks; out[2] = r.threads; out[3] = r.groups; out[4] = r.wide;
 }
 }
@@ -138,6 +142,21 @@ def test_select_routes(plans, sms):
             # a device that holds no such cluster: another route, not a refusal
             mode, ranks, threads, groups, wide = _select(plans, n, units, sms, 0)
             assert mode == (STREAM if n > 40960 else ONE) and ranks == 1
+
+
+def test_select_routes_by_waves(plans):
+    """A cluster that has no SM of its own left, or a wave too many, is slower
+    than one CTA or streaming."""
+    def mode(n, units, sms=152):
+        return _select(plans, n, units, sms, 1)[:2]
+    assert mode(16385, 36) == [CLUSTER, 4] and mode(16385, 38) == [ONE, 1] and mode(24000, 38) == [ONE, 1]
+    assert mode(32768, 38) == [CLUSTER, 4] and mode(32768, 39) == [ONE, 1]
+    assert mode(40961, 72) == [CLUSTER, 4] and mode(40961, 76) == [STREAM, 1] and mode(65536, 76) == [STREAM, 1]
+    assert mode(100000, 64) == [CLUSTER, 4] and mode(100000, 76) == [STREAM, 1]
+    assert mode(150000, 14) == [CLUSTER, 8] and mode(150000, 20) == [CLUSTER, 4]
+    assert mode(262144, 38) == [CLUSTER, 8]
     # the plan follows the device
-    assert _select(plans, 65536, 57, 152, 1)[0] == CLUSTER
-    assert _select(plans, 65536, 57, 76, 1)[0] == STREAM
+    assert mode(65536, 57) == [CLUSTER, 4] and mode(65536, 57, 76) == [STREAM, 1]
+    # threads: one CTA of a row just beyond 16384 tokens, alone on its SM
+    assert _select(plans, 16385, 39, 152, 1)[2] == 1024 and _select(plans, 16385, 300, 152, 1)[2] == 512
+    assert _select(plans, 16384, 39, 152, 1)[2] == 512
