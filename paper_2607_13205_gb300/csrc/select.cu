@@ -130,6 +130,13 @@ __device__ __forceinline__ void unit_sync() {
   }
 }
 
+// x << n, 0 for n > 63.
+__device__ __forceinline__ uint64_t shl64(uint64_t x, uint32_t n) {
+  uint64_t r;
+  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+  return r;
+}
+
 __device__ __forceinline__ int warp_sum(int v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -1653,15 +1660,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
   // tokens, search and slots: B 0.2 41.2 and 43.8 us, 0.3 43.2 and 44.4, 0.5
   // 46.6 and 44.5; 1024 x 32768 at 0.3 223 and 231; 168 x 110545 at 0.5 229
   // and 223: the line is drawn at kDenseWords, 0.39 of the slots.
-  uint64_t kr_lo = 0, kr_hi = 0;                   // kept per role 0 .. 3, 4 .. 7, 16 bits each
+  // kept per role, a lane's share: eight bits each (a lane writes at most one
+  // position of each of its warp's words, 41 of them where keys are held), in
+  // streaming mode (257) 16 bits each, roles 0 .. 3 and 4 .. 7
+  uint64_t kr_lo = 0, kr_hi = 0;
   const uint8_t* rp = after_wait(v.rp);
   auto put = [&](int pos, int t) {
     const uint32_t role = count_roles ? ld_u8(rp + t) : 0u;
     if (in_bounds(pos, 1, width, a.status)) dst[pos] = t;   // (the unit's own row)
     if (count_roles) {
-      const uint64_t one = 1ull << (16u * (role & 3u));
-      kr_lo += role < 4u ? one : 0ull;
-      kr_hi += role - 4u < 4u ? one : 0ull;
+      if constexpr (STREAM) {
+        kr_lo += shl64(1ull, 16u * role);
+        kr_hi += shl64(1ull, 16u * (role ^ 4u));
+      } else {
+        kr_lo += shl64(1ull, 8u * role);
+      }
     }
   };
   {
@@ -1679,7 +1692,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
       const int tot = __shfl_sync(0xffffffffu, incl, 31);
       if (tot > kDenseWords) {
         const uint32_t below = (1u << lane) - 1u;
-#pragma unroll 4
+#pragma unroll 8
         for (int w = 0; w < 32; ++w) {
           const uint32_t m = __shfl_sync(0xffffffffu, mine, w);
           const int first = pos0 + __shfl_sync(0xffffffffu, incl, w) - __popc(m);
@@ -1733,7 +1746,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
   if (count_roles) {
 #pragma unroll
     for (int r = 0; r < kR; ++r) {
-      const uint32_t mine = static_cast<uint32_t>((r < 4 ? kr_lo : kr_hi) >> (16 * (r & 3))) & 0xFFFFu;
+      const uint32_t mine = STREAM ? static_cast<uint32_t>((r < 4 ? kr_lo : kr_hi) >> (16 * (r & 3))) & 0xFFFFu
+                                   : static_cast<uint32_t>(kr_lo >> (8 * r)) & 0xFFu;
       const int c = static_cast<int>(__reduce_add_sync(0xffffffffu, mine));
       if (lane == 0 && c) {
         if constexpr (CL)

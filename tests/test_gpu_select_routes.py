@@ -106,3 +106,16 @@ def test_routes_agree(case):
         row = got[0, h, cu[s]:cu[s + 1]] if ob.varlen else got.reshape(ob.n_units, -1)[u]
         assert np.array_equal(row, idx), f"unit {u}"
         assert list(per[u]) == counts, f"unit {u} per-role counts"
+
+
+@pytest.mark.parametrize("n,units,role", [(8192, 400, 0), (8192, 8, 3), (40960, 40, 2), (163840, 20, 1), (262144, 48, 3)])
+def test_counts_of_one_role_and_everything_kept(n, units, role):
+    """The largest share of a role's count that a lane can hold, on each route."""
+    batch = R.Batch(units, 1, 1, 1, 64, n)
+    roles = torch.full((1, n), role, dtype=torch.uint8, device=DEV)
+    params = R.select_params(1.0, I.PAPER_ALPHA, policy=R.POLICY_GLOBAL)
+    idx = torch.full(batch.kept_shape(1.0), -7, dtype=torch.int32, device=DEV)
+    per = torch.full((units, I.N_ROLES), -1, dtype=torch.int32, device=DEV)
+    R.role_alloc_select(batch, torch.rand(units, 1, 1, n, device=DEV), roles, params, idx, kept_per_role=per)
+    assert torch.equal(idx, torch.arange(n, dtype=torch.int32, device=DEV).expand_as(idx))
+    assert per.tolist() == [[n if r == role else 0 for r in range(I.N_ROLES)]] * units
