@@ -61,13 +61,17 @@ constexpr int kDecodeSplitCost = 320;       // rows a CTA could stream while one
 // heads: layers x KV heads, of sequences with m_max rows (varlen: at most
 // m_max, `total` together).
 inline int64_t decode_split_rows(bool varlen, int64_t heads, int64_t b, int64_t m_max, int64_t total, int d,
-                                 bool fine, int sms) {
+                                 int G, bool fine, int sms) {
   const int64_t ns = m_max > 0 ? (m_max + kDecodeRowsPerSplit - 1) / kDecodeRowsPerSplit : 1;
   int64_t r = (m_max + ns - 1) / ns;
   r = r > 0 ? (r + 63) / 64 * 64 : 64;
   if (!fine) return r;
-  // CTAs resident at once: limited by their two stages of shared memory
-  const int64_t slots = static_cast<int64_t>(sms) * (d == 128 ? 3 : 6);
+  // CTAs resident at once: limited by their two stages of shared memory, or
+  // with eight heads' sums at d = 64 by their registers (counted as six, 152
+  // units of 3277 rows took 38.4 us against 33.2).  Packed splits leave their
+  // slots one by one, and six suits them (23.7 us for 32 of 5 to 13 thousand
+  // rows, 25.6 counted as five).
+  const int64_t slots = static_cast<int64_t>(sms) * (d == 128 ? 3 : G > 4 && !varlen ? 5 : 6);
   int64_t best = INT64_MAX;
   for (int64_t x = 128; x <= kDecodeRowsPerSplit; x += 64) {
     int64_t cost;
@@ -76,6 +80,8 @@ inline int64_t decode_split_rows(bool varlen, int64_t heads, int64_t b, int64_t 
       // the rows and starts of a slot, and half a split until the last ends
       const int64_t ctas = heads * (x >= m_max ? b : total / x + (b + 1) / 2);
       cost = (heads * total + ctas * kDecodeSplitCost) / slots + (x + kDecodeSplitCost) / 2;
+      // (one split each needs no merge: 512 rows of 1 to 300, 13.2 us against 14.2)
+      if (x >= m_max) cost -= cost / 16;
     } else {
       const int64_t ctas = heads * b * ((m_max + x - 1) / x);
       cost = (ctas + slots - 1) / slots * (x + kDecodeSplitCost);

@@ -766,7 +766,7 @@ int role_alloc_select(const rolekv_batch* batch, const float* scores, const uint
 namespace {
 void decode_split(const BatchInfo& bi, int64_t m_max, int64_t total, bool fine, int32_t* rows_per_split,
                   int32_t* n_splits) {
-  const int64_t r = decode_split_rows(bi.varlen, static_cast<int64_t>(bi.L) * bi.Hkv, bi.b, m_max, total, bi.d, fine,
+  const int64_t r = decode_split_rows(bi.varlen, static_cast<int64_t>(bi.L) * bi.Hkv, bi.b, m_max, total, bi.d, bi.G, fine,
                                       device_sms());
   *rows_per_split = static_cast<int32_t>(r);
   *n_splits = static_cast<int32_t>((m_max + r - 1) / r);

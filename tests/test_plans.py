@@ -16,8 +16,8 @@ SHIM = r"""
 using namespace rolekv;
 extern "C" {
 int score(int varlen, long units, int chunks, int tiles, int sms) { return score_parts(varlen, units, chunks, tiles, sms); }
-long decode(int varlen, long heads, long b, long m_max, long total, int d, int fine, int sms) {
-  return decode_split_rows(varlen, heads, b, m_max, total, d, fine, sms);
+long decode(int varlen, long heads, long b, long m_max, long total, int d, int G, int fine, int sms) {
+  return decode_split_rows(varlen, heads, b, m_max, total, d, G, fine, sms);
 }
 void quest(int varlen, long heads, long b, long n_max, long T, long page, long rows, int d, int sms, long* out) {
   const QuestSplit q = quest_split(varlen, heads, b, n_max, T, page, rows, d, sms);
@@ -49,7 +49,7 @@ def plans(tmp_path_factory):
     lib = ctypes.CDLL(so)
     L, I = ctypes.c_long, ctypes.c_int
     lib.score.argtypes = [I, L, I, I, I]
-    lib.decode.argtypes = [I, L, L, L, L, I, I, I]
+    lib.decode.argtypes = [I, L, L, L, L, I, I, I, I]
     lib.decode.restype = L
     lib.quest.argtypes = [I, L, L, L, L, L, L, I, I, ctypes.POINTER(L)]
     lib.quest.restype = None
@@ -94,12 +94,23 @@ def test_decode_splits(plans, sms):
         for m in (0, 1, 63, 64, 65, 820, 3277, 131072):
             for varlen in (0, 1):
                 for d in (64, 128):
-                    coarse = plans.decode(varlen, heads, b, m, m * b, d, 0, sms)
-                    fine = plans.decode(varlen, heads, b, m, m * b, d, 1, sms)
+                    coarse = plans.decode(varlen, heads, b, m, m * b, d, 8, 0, sms)
+                    fine = plans.decode(varlen, heads, b, m, m * b, d, 8, 1, sms)
                     for r in (coarse, fine):
                         assert 64 <= r <= 1024 and r % 64 == 0
                     # a workspace of the fine splits holds the coarse ones' partials
                     assert -(-m // fine) >= -(-m // coarse)
+
+
+def test_decode_splits_fill_whole_waves(plans):
+    """152 SMs hold 760 CTAs of eight heads' sums at d = 64 (912 of four): the
+    splits of 152 units make whole waves of those."""
+    for m in (1638, 3277):
+        for G, slots in ((4, 912), (8, 760)):
+            ctas = 152 * -(-m // plans.decode(0, 152, 1, m, 152 * m, 64, G, 1, 152))
+            assert ctas <= slots or ctas % slots > slots // 2 or ctas % slots == 0
+    # short packed rows, whose merge costs more than the balance gains
+    assert plans.decode(1, 8, 64, 300, 9600, 64, 4, 1, 152) >= 300
 
 
 @pytest.mark.parametrize("sms", SMS)
