@@ -238,13 +238,22 @@ def workspace(op: int, batch: Batch, W: int = 0, device="cuda") -> torch.Tensor:
     return torch.empty(max(workspace_size(op, batch, W), 256), dtype=torch.uint8, device=device)
 
 
+def _scratch(make, stream, *args, **kw) -> torch.Tensor:
+    """A call's own workspace, allocated on the stream the call runs on: the
+    caching allocator hands a freed block to its own stream alone."""
+    if stream is None:
+        return make(*args, **kw)
+    with torch.cuda.stream(stream):
+        return make(*args, **kw)
+
+
 def snapkv_score(batch: Batch, q_win: torch.Tensor, k: torch.Tensor, W: int, pool_k: int,
                  scores: torch.Tensor, scores_prepool: Optional[torch.Tensor] = None,
                  lse_win: Optional[torch.Tensor] = None, scale: float = 0.0,
                  ws: Optional[torch.Tensor] = None, status: Optional[torch.Tensor] = None,
                  stream=None) -> torch.Tensor:
     if ws is None:
-        ws = workspace(OP_SNAPKV, batch, W, device=k.device)
+        ws = _scratch(workspace, stream, OP_SNAPKV, batch, W, device=k.device)
     _check(lib().snapkv_score(ctypes.byref(batch.desc), tensor_desc(q_win), tensor_desc(k, batch.varlen),
                               W, pool_k, scale, _ptr(lse_win), _ptr(scores), _ptr(scores_prepool),
                               _ptr(ws), ws.numel(), _ptr(status), _stream(stream)))
@@ -296,7 +305,7 @@ def decode_attention(batch: Batch, q: torch.Tensor, k_cache: torch.Tensor, v_cac
                      status: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """q bf16 [L][b][Hq][d] -> out fp32 [L][b][Hq][d]."""
     if ws is None:
-        ws = decode_workspace(batch, budget, device=q.device)
+        ws = _scratch(decode_workspace, stream, batch, budget, device=q.device)
     if q.dtype != torch.bfloat16 or q.dim() != 4 or q.stride(-1) != 1:
         raise ValueError("q is a bf16 [L][b][Hq][d] tensor with a contiguous last axis")
     sl, ss, sh, _ = q.stride()
@@ -313,7 +322,7 @@ def h2o_score(batch: Batch, q: torch.Tensor, k: torch.Tensor, scores: torch.Tens
     """lse: optional fp32 natural-log normalisers of every query row (dense
     [L][b][Hq][n], varlen [L][Hq][T]); given, the score is one pass over K."""
     if ws is None:
-        ws = workspace(OP_H2O, batch, 0, device=k.device)
+        ws = _scratch(workspace, stream, OP_H2O, batch, 0, device=k.device)
     _check(lib().h2o_score(ctypes.byref(batch.desc), tensor_desc(q, batch.varlen),
                            tensor_desc(k, batch.varlen), scale, _ptr(lse), _ptr(scores), _ptr(ws),
                            ws.numel(), _ptr(status), _stream(stream)))

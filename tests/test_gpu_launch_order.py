@@ -182,3 +182,32 @@ def test_captured_calls_in_a_row():
         torch.cuda.synchronize()
         for a, b in zip(got, ref):
             assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
+
+
+@pytest.mark.parametrize("call", ["score", "h2o", "decode"])
+def test_own_workspace_on_another_stream(call, monkeypatch):
+    """A call on a stream of its own without a workspace: what the call
+    allocates is not handed out to the current stream while the call may still
+    run."""
+    c = Case(6)
+    qf = I.make_q_full(c.w, 6, device=DEV)
+    kept = []
+    for name in ("workspace", "decode_workspace"):
+        make = getattr(R, name)
+        monkeypatch.setattr(R, name, lambda *a, make=make, **k: kept.append(make(*a, **k)) or kept[-1])
+    s = torch.cuda.Stream()
+    out = torch.empty(c.batch.score_shape(), device=DEV)
+    o = torch.empty((c.w.L, c.w.b, c.w.Hq, c.w.d), device=DEV)
+    torch.cuda.synchronize()
+    if call == "score":
+        R.snapkv_score(c.batch, c.qw, c.k, c.w.W, 7, out, stream=s)
+    elif call == "h2o":
+        R.h2o_score(c.batch, qf, c.k, out, stream=s)
+    else:
+        R.decode_attention(c.batch, c.qd, c.k, c.v, None, 1.0, o, compacted=False, stream=s)
+    assert len(kept) == 1
+    ptr, size = kept[0].data_ptr(), kept[0].numel()
+    kept.clear()                                     # freed, as when the call returns
+    later = [torch.empty(size, dtype=torch.uint8, device=DEV) for _ in range(4)]
+    assert all(t.data_ptr() != ptr for t in later)
+    torch.cuda.synchronize()
