@@ -174,7 +174,13 @@ int64_t rolekv_kept_rows(int64_t n, float budget, int32_t kept_extra);
 /* Bytes of device workspace snapkv_score / h2o_score / rolekv_compress need for
  * this batch (op: 0 snapkv_score, 1 h2o_score, 2 rolekv_compress; W the SnapKV
  * window).  The workspace is caller-owned scratch, 256-byte aligned, reusable
- * across calls on the same stream; its contents need no initialisation. */
+ * across calls on the same stream; its contents need no initialisation.
+ * The size does not grow with the batch throughout: a batch that leaves SMs
+ * idle has its key chunks split over CTAs and then wants up to 64 KB a chunk
+ * (at most 40 MB) where a larger one wants 2 KB.  A program that keeps one
+ * workspace for several batch shapes takes the largest of their sizes.  One
+ * that only holds whole chunks is used without the split: the same scores,
+ * more time; a smaller one is refused (ROLEKV_ERR_WORKSPACE). */
 int rolekv_workspace_size(int op, const rolekv_batch* batch, int32_t W, size_t* bytes);
 
 /* SnapKV windowed score (Section 2; Section 4 'SnapKV mechanism'; Algorithm 1,
@@ -263,7 +269,13 @@ int quest_score(const rolekv_batch* batch, rolekv_tensor q_win, rolekv_tensor k,
  *   scale    <= 0: 1/sqrt(d).
  *   out      fp32 [L][b][Hq][d], contiguous.
  *   workspace  rolekv_decode_workspace_size() bytes (partials of the split
- *            rows), caller-owned, no initialisation needed.
+ *            rows), caller-owned, no initialisation needed.  Where the rows are
+ *            split follows the whole batch (layers, sequences, heads, rows) and
+ *            the device; a workspace that only holds splits of about 1024 rows
+ *            is used with those, a smaller one is refused.  The outputs of one
+ *            sequence or layer are the same bits for the same batch shape and
+ *            workspace size, and agree to fp32 rounding (about 5e-7 relative)
+ *            across them.
  *   status_dev optional int32 status word (ROLEKV_STATUS_TIMEOUT).
  * d must be 64 or 128 and G <= 8; a unit with no valid row gives zeros. */
 int rolekv_decode_workspace_size(const rolekv_batch* batch, float budget, size_t* bytes);

@@ -1,6 +1,10 @@
 """Small batches split a unit's key chunks over CTAs; the scores are the same
-bits as where a chunk is one CTA's: a batch too large for the split against
-its layers one at a time, and against the oracle."""
+bits as where a chunk is one CTA's: a layer with the workspace it asks for
+against the same layer with one that only holds whole chunks, a batch of many
+layers (cut less or not at all) against its layers one at a time, and against
+the oracle."""
+
+import math
 
 import pytest
 import torch
@@ -20,12 +24,15 @@ def _w(L, Hkv, G, d, n, W, lens=None):
                       (1, 3), seqlens=lens)
 
 
-# the whole batch has more than 76 chunks (no split), a layer at most 20
+# One layer of each is cut on 152 SMs, except where it says so (a chunk of less
+# than eight tiles gains nothing).
 CASES = {
     "one_cell": _w(40, 2, 4, 128, 512, 32),
     "cell_and_a_tile": _w(40, 2, 4, 128, 513, 32),
-    "odd_tiles_two_row_tiles": _w(20, 4, 4, 128, 1500, 64),
     "d64_shorter_than_window": _w(40, 2, 8, 64, 20, 32),
+    "two_cells": _w(40, 2, 4, 128, 1024, 32),
+    "two_cells_and_a_key": _w(40, 2, 8, 64, 1025, 32),
+    "odd_tiles_two_row_tiles": _w(20, 4, 4, 128, 1500, 64),
     "g7_padded_rows": _w(20, 4, 7, 128, 2177, 32),
     "two_chunks": _w(10, 4, 4, 128, 8500, 32),
     "eight_chunks": _w(4, 4, 2, 64, 66000, 64),
@@ -38,6 +45,18 @@ CASES = {
     "rounds_varlen": _w(40, 2, 4, 128, 4000, 32, (4000, 1, 0, 1030, 2300)),
     "varlen_chunks_g7": _w(7, 4, 7, 128, 9000, 32, (9000, 129, 5000)),
 }
+UNCUT = {"one_cell", "cell_and_a_tile", "d64_shorter_than_window"}
+
+
+def _whole_chunks_bytes(batch):
+    """The two-pass workspace of the plan that cuts no chunk."""
+    tiles = (batch.n_max + 127) // 128
+    nc = max(1, min(8, (tiles + 63) // 64))
+    per = max(1, (tiles + nc - 1) // nc)
+    chunks = max(1, (tiles + per - 1) // per)
+    al = lambda x: (x + 255) // 256 * 256
+    units, elems = batch.n_units, math.prod(batch.score_shape())
+    return 256 + al(units * chunks * 256 * 8) + al(units * 256 * 4) + al(elems * 4) + al((units + 1) * 4)
 
 
 def _inputs(w):
@@ -64,6 +83,13 @@ def test_split_scores_match_whole_chunks(name):
     one = w.scaled(L=1)
     parts = [_score(one, K[l:l + 1], qw[l:l + 1]) for l in range(w.L)]
     assert torch.equal(whole, torch.cat(parts, dim=0))
+    # a layer, cut and not
+    layer = lib_batch(one, DEV)
+    uncut, asked = _whole_chunks_bytes(layer), R.workspace_size(R.OP_SNAPKV, layer, w.W)
+    assert (asked == uncut) if name in UNCUT else (asked > uncut)
+    small = torch.empty(uncut, dtype=torch.uint8, device=DEV)
+    for l in (0, w.L - 1):
+        assert torch.equal(parts[l], _score(one, K[l:l + 1], qw[l:l + 1], ws=small))
     # with supplied normalisers: pass 2 alone, split or not
     lse = 0.5 + torch.rand(w.L, w.b, w.Hq, w.W, device=DEV)
     whole = _score(w, K, qw, lse_win=lse)
@@ -76,19 +102,29 @@ def test_split_scores_match_whole_chunks(name):
         assert_scores_close(ob.score_view(got, u), pre, f"{name} unit {u}")
 
 
-def test_workspace_of_the_unsplit_plan_is_accepted():
-    """A workspace too small for the split's partials is used without it."""
+def test_a_workspace_too_small_for_whole_chunks_is_refused():
     w = CASES["two_chunks"].scaled(L=1)
     K, qw = _inputs(w)
     batch = lib_batch(w, DEV)
-    full = R.workspace_size(R.OP_SNAPKV, batch, w.W)
-    al = lambda x: (x + 255) // 256 * 256
-    units, chunks = batch.n_units, 2
-    need = 256 + al(units * chunks * 256 * 8) + al(units * 256 * 4) + al(units * w.n * 4) + al((units + 1) * 4)
-    assert need < full
-    a = _score(w, K, qw)
-    b = _score(w, K, qw, ws=torch.empty(need, dtype=torch.uint8, device=DEV))
-    assert torch.equal(a, b)
     sc = torch.empty(batch.score_shape(), device=DEV)
+    ws = torch.empty(_whole_chunks_bytes(batch) - 256, dtype=torch.uint8, device=DEV)
     with pytest.raises(R.RolekvError):
-        R.snapkv_score(batch, qw, K, w.W, 7, sc, ws=torch.empty(need - 256, dtype=torch.uint8, device=DEV))
+        R.snapkv_score(batch, qw, K, w.W, 7, sc, ws=ws)
+
+
+def test_compression_with_a_workspace_for_whole_chunks():
+    """A workspace that only holds whole chunks gives the same kept rows."""
+    w = CASES["odd_tiles_two_row_tiles"].scaled(L=1)
+    roles = I.workload_roles(w, 4)
+    K, V = I.make_kv(w, roles, 4, device=DEV)
+    qw = I.make_q_window(w, 4, device=DEV)
+    batch = lib_batch(w, DEV)
+    params = R.select_params(0.2, I.PAPER_ALPHA, alpha_key=0.02, key_role=I.ROLE_KEY)
+    out = []
+    for size in (R.workspace_size(R.OP_COMPRESS, batch, w.W), _whole_chunks_bytes(batch)):
+        idx = torch.empty(batch.kept_shape(0.2), dtype=torch.int32, device=DEV)
+        kv = torch.empty((2,) + R.compact_shape(batch, 0.2), dtype=torch.bfloat16, device=DEV)
+        R.rolekv_compress(batch, qw, K, V, w.W, 7, torch.as_tensor(roles, device=DEV), params, idx, kv[0], kv[1],
+                          torch.empty(size, dtype=torch.uint8, device=DEV))
+        out.append((idx, kv))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1].view(torch.int16), out[1][1].view(torch.int16))
