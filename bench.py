@@ -144,10 +144,10 @@ class ClockSampler:
 # capture whose sources have changed since is stale and gives null.
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic.md")
 KERNEL_SOURCES = {
-    ("snapkv", "score"): ["attn_score.cu", "device_common.cuh", "internal.h"],
-    ("h2o", "score"): ["attn_score.cu", "device_common.cuh", "internal.h"],
-    ("quest", "score"): ["quest.cu", "device_common.cuh", "internal.h"],
-    ("snapkv", "select"): ["select.cu", "device_common.cuh", "internal.h"],
+    ("snapkv", "score"): ["attn_score.cu", "device_common.cuh", "internal.h", "plans.h"],
+    ("h2o", "score"): ["attn_score.cu", "device_common.cuh", "internal.h", "plans.h"],
+    ("quest", "score"): ["quest.cu", "device_common.cuh", "internal.h", "plans.h"],
+    ("snapkv", "select"): ["select.cu", "device_common.cuh", "internal.h", "plans.h"],
     ("snapkv", "compact"): ["compact.cu", "device_common.cuh", "internal.h"],
 }
 

@@ -26,12 +26,14 @@
 // (items = chunks of a unit's keys; the chunks of a unit exchange their row
 // statistics through global memory between the passes) and for H2O (items =
 // query blocks; a block's normalisers are its own, so they stay on chip).
-// What bounds it (32 layers x 4 x 32768 tokens, 3.2 ms, timing-only copies):
-// the MMAs alone 2.77 ms, the epilogue alone 2.97, both with the keys from L2
-// 3.16; with one row tile the keys' two readings through L2 (27 bytes a clock
-// and SM, 1.24k cycles a tile with no arithmetic at all).  Small batches cut
-// a chunk into parts of whole cells, each a CTA (kSplit); with supplied
-// normalisers the CTAs share the key tiles evenly (kShares).
+// What bounds it, by copies that leave something out (timing only).  1024
+// units x 32768 keys, two row tiles, 3.33 ms: 2.75 without the epilogue's
+// arithmetic, 2.88 with one MMA k-step of eight, 3.09 with every key tile in
+// L2, 2.59 with that and no arithmetic: three limits close together.  152
+// units x 8192, one row tile, 102 us: 98, 97, 84 and 76, so there the keys'
+// two readings.  Small batches cut a chunk into parts of whole cells, each a
+// CTA (kSplit); with supplied normalisers the CTAs share the key tiles evenly
+// (kShares).
 // attn_pass_kernel runs one pass per launch (the no-workspace SnapKV call).
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -884,10 +886,11 @@ __device__ __forceinline__ int chunk_cells(int kt0, int kt1) {
   return (kt1 - kt0 + kCellTiles - 1) / kCellTiles;
 }
 
-// Item `item` of the fused launch.  SnapKV: (unit, chunk of its key tiles),
-// or one of the n_parts parts of a chunk, each a run of whole cells.  H2O: (unit, query block), the longest blocks first, over the key tiles up
-// to the block's last position; its rows' normalisers are its own (no other
-// CTA contributes), so the block needs no cross-CTA exchange.
+// Item `item` of the fused launch.  SnapKV: (unit, chunk of its key tiles), or
+// one of the n_parts parts of a chunk, each a run of whole cells.  H2O: (unit,
+// query block), the longest blocks first, over the key tiles up to the block's
+// last position; its rows' normalisers are its own (no other CTA contributes),
+// so the block needs no cross-CTA exchange.
 struct FItem {
   int u, chunk, cell0, rb, kt0, kt1;
   Unit un;

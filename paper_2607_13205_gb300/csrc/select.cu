@@ -36,8 +36,8 @@
 // Kept positions are then written in ascending order from a scan of the bit
 // words, each rank at the offset of the ranks before it.
 //
-// Rows longer than kSmemMaxN tokens in batches of more units than clusters
-// can be resident (streaming mode, one CTA per unit) do not keep their keys:
+// Rows longer than kSmemMaxN tokens in batches of more units than a few waves
+// of clusters (streaming mode, one CTA per unit) do not keep their keys:
 // every pass recomputes a group's pooled keys from the score row (read again
 // from L2), the first-digit histograms count in 32 bits and a candidate-list
 // entry carries its key beside (bucket << 24) | slot.

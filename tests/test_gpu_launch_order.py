@@ -148,8 +148,9 @@ def test_after_a_kernel_that_releases_early(late_copy, shape):
             assert torch.equal(got.view(torch.uint8), want.view(torch.uint8)), (call, name)
 
 
-def test_two_streams():
-    cases = [Case(2), Case(3)]
+@pytest.mark.parametrize("shape", [(3001, 2), (45003, 2)], ids=["one", "cluster"])
+def test_two_streams(shape):
+    cases = [Case(2, *shape), Case(3, *shape)]
     want = [c.all() for c in cases]
     torch.cuda.synchronize()
     streams = [torch.cuda.Stream() for _ in cases]
@@ -165,8 +166,9 @@ def test_two_streams():
                 assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
 
 
-def test_captured_calls_in_a_row():
-    c, other = Case(4), Case(5)
+@pytest.mark.parametrize("shape", [(3001, 2), (45003, 2)], ids=["one", "cluster"])
+def test_captured_calls_in_a_row(shape):
+    c, other = Case(4, *shape), Case(5, *shape)
     want = [c.all(), other.all()]
     g = torch.cuda.CUDAGraph()
     with torch.cuda.graph(g):
