@@ -1765,10 +1765,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) select_kernel(const SelectArgs 
   if (tid == 0 && S.nan_seen && a.status != nullptr) atomicOr(a.status, ROLEKV_STATUS_NONFINITE);
 }
 
+// Dynamic shared memory a launch may ask for: the same for every call, since
+// the limit belongs to the kernel and another thread's call may set it between
+// this one's setting and its launch.
+constexpr int kMaxDynamicSmem = 227 * 1024 - 5 * 1024;
+static_assert(sizeof(SelShared) <= 5 * 1024, "beside the dynamic part");
+
 template <int NT, int MODE>
 cudaError_t launch_select_nt(const SelectArgs& a, const SelectPlan& p, size_t smem, cudaStream_t stream) {
   cudaError_t e = cudaFuncSetAttribute(select_kernel<NT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+                                       kMaxDynamicSmem);
   if (e != cudaSuccess) return e;
   return launch_early(select_kernel<NT, MODE>, static_cast<unsigned>(a.n_units) * p.ranks, NT, smem, stream,
                       static_cast<unsigned>(p.ranks), a, p);
@@ -1793,7 +1799,7 @@ int64_t resident_clusters(const SelectPlan& p, size_t smem, bool alone) {
   cfg.numAttrs = 1;
   int held = 0;
   if (cudaFuncSetAttribute(select_kernel<NT, kCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(smem)) != cudaSuccess ||
+                           kMaxDynamicSmem) != cudaSuccess ||
       cudaOccupancyMaxActiveClusters(&held, select_kernel<NT, kCluster>, &cfg) != cudaSuccess) {
     cudaGetLastError();                            // (the other routes decide whether the call fails)
     return 0;

@@ -3,6 +3,8 @@ streaming) give the same kept sets: a batch large enough for one route against
 its layers one at a time, which take another, and sampled units against the
 oracle."""
 
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -119,3 +121,35 @@ def test_counts_of_one_role_and_everything_kept(n, units, role):
     R.role_alloc_select(batch, torch.rand(units, 1, 1, n, device=DEV), roles, params, idx, kept_per_role=per)
     assert torch.equal(idx, torch.arange(n, dtype=torch.int32, device=DEV).expand_as(idx))
     assert per.tolist() == [[n if r == role else 0 for r in range(I.N_ROLES)]] * units
+
+
+@pytest.mark.parametrize("sizes", [((40960, 76), (20000, 76)), ((131072, 8), (70000, 8)), ((40960, 8), (17000, 8))],
+                         ids=["one", "cluster", "cluster_512"])
+def test_two_threads_with_rows_of_different_lengths(sizes):
+    """Calls of the same kernel with more and less shared memory from two
+    threads at once: neither is refused for the other's limit."""
+    errors = []
+
+    def work(n, units):
+        try:
+            batch = R.Batch(units, 1, 1, 1, 64, n)
+            g = torch.Generator(device=DEV).manual_seed(n)
+            scores = torch.rand(batch.score_shape(), generator=g, device=DEV)
+            roles = torch.zeros((1, n), dtype=torch.uint8, device=DEV)
+            params = R.select_params(0.1, I.PAPER_ALPHA, policy=R.POLICY_GLOBAL)
+            s = torch.cuda.Stream()
+            s.wait_stream(torch.cuda.current_stream())
+            idx = [torch.empty(batch.kept_shape(0.1), dtype=torch.int32, device=DEV) for _ in range(2)]
+            for i in range(1500):
+                R.role_alloc_select(batch, scores, roles, params, idx[i > 0], stream=s)
+            s.synchronize()
+            assert torch.equal(idx[0], idx[1])
+        except Exception as e:                       # noqa: BLE001  (reported by the main thread)
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=x) for x in sizes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
